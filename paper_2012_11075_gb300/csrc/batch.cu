@@ -30,6 +30,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -137,9 +138,13 @@ __global__ void __launch_bounds__(TX, Staging<T>::min_blocks_batch(TX))
     // and no reloads after the population stores (which could alias
     // device memory)
     __shared__ KParams s_kp;
-    if (threadIdx.x == 0) {
-      s_kp = cs.kp;
-      s_kp.step += j;                      // the case's time step of this item
+    static_assert(sizeof(KParams) % 8 == 0 && sizeof(KParams) / 8 <= 2 * 32 &&
+                      offsetof(KParams, step) % 8 == 0,
+                  "copied in 8-byte words");
+    for (unsigned q = threadIdx.x; q < sizeof(KParams) / 8; q += TX) {
+      long long v = reinterpret_cast<const long long*>(&cs.kp)[q];
+      if (q == offsetof(KParams, step) / 8) v += j;   // the case's time step of this item
+      reinterpret_cast<long long*>(&s_kp)[q] = v;
     }
     __syncthreads();
     const KParams& kp = s_kp;
@@ -407,14 +412,7 @@ KParams case_kparams(const wblbe_batch::Case& c, int rows) {
   k.pitch = c.pitch;
   k.rows = rows;
   k.plane = c.plane;
-  k.omega = 1.0 / p.tau;
-  k.kforce = 1.0 - 1.0 / (2.0 * p.tau);
-  k.kappa = p.kappa;
-  k.two_beta = 2.0 * p.beta;
-  const double rr = batch_rho_ref(p);
-  k.rho_ref = rr;
-  k.dl = rr - p.rho_l;
-  k.dg = rr - p.rho_g;
+  set_physics(k, p.tau, p.kappa, p.beta, p.rho_l, p.rho_g, batch_rho_ref(p));
   k.step = c.steps;                        // advanced on the device by each launch
   k.row_lo = 0;
   k.row_hi = p.ny;

@@ -64,9 +64,10 @@ __host__ __device__ constexpr double w3(int i) {
 struct P3 {
   int nx, ny, nz, pitch;
   long long plane;                 // elements per population plane / field
-  double omega, kforce, kappa, two_beta, rho_l, rho_g;
+  double omega, kforce, kappa, two_beta;
   // storage shift density (0 in FP64) and rho_ref - rho_l, rho_ref - rho_g
   double rho_ref, dl, dg;
+  NodeConsts<float> f;             // the FP32 constants, converted on the host
   long long step;                  // the step being taken (FP32 rounding draws)
 };
 
@@ -99,6 +100,23 @@ __device__ __forceinline__ float node_uniform(uint32_t k, uint32_t ht) {
 __device__ __forceinline__ float round_stochastic1(float h, float e, float u) {
   const float n = next_toward(h, e);
   return fabsf(__fmul_rn(u, __fsub_rn(n, h))) < fabsf(e) ? n : h;
+}
+
+template <typename T>
+__device__ __forceinline__ NodeConsts<T> consts3(const P3& p) {
+  if constexpr (sizeof(T) == 4) {
+    return p.f;
+  } else {
+    NodeConsts<double> q{};
+    q.omega = p.omega;
+    q.keep = 1.0 - p.omega;
+    q.kf = p.kforce;
+    q.kappa = p.kappa;
+    q.two_beta = p.two_beta;
+    q.dl = p.dl;
+    q.dg = p.dg;
+    return q;
+  }
 }
 
 struct Out3 {
@@ -142,6 +160,23 @@ __global__ void __launch_bounds__(kBlock3) d3_density(const T* __restrict__ src,
   }
 }
 
+// mu from the sums of the axis and edge neighbours' densities and the own
+// one.  The FP32 functions of this file name each rounding (mu3,
+// grad3_from, force3, update3_f32): a result then does not depend on which
+// multiply-adds the compiler contracts in one kernel or another.
+__device__ __forceinline__ double mu3(double ax, double ed, double c, const NodeConsts<double>& q) {
+  const double lap = (1.0 / 3.0) * (ax - 6.0 * c) + (1.0 / 6.0) * (ed - 12.0 * c);
+  const double a = c + q.dl, b = c + q.dg;
+  return q.two_beta * a * b * (a + b) - q.kappa * lap;
+}
+__device__ __forceinline__ float mu3(float ax, float ed, float c, const NodeConsts<float>& q) {
+  const float lap = __fmaf_rn(1.0f / 3.0f, __fmaf_rn(-6.0f, c, ax),
+                              __fmul_rn(1.0f / 6.0f, __fmaf_rn(-12.0f, c, ed)));
+  const float a = __fadd_rn(c, q.dl), b = __fadd_rn(c, q.dg);
+  return __fmaf_rn(__fmul_rn(__fmul_rn(q.two_beta, a), b), __fadd_rn(a, b),
+                   -__fmul_rn(q.kappa, lap));
+}
+
 // mu = mu_0(rho) - kappa lap(rho), mu_0 = 2 beta a b (a + b), a = rho - rho_l,
 // b = rho - rho_g (Eq. doubleWell), lap = 6 sum_i w_i (rho(x + c_i) - rho(x)).
 // The field holds rho - rho_ref (rho_ref = 0 in FP64), which the Laplacian
@@ -164,9 +199,7 @@ __global__ void __launch_bounds__(kBlock3) d3_chem_pot(const T* __restrict__ rho
     if (i == 7) continue;
     if (i < 7) ax += nbr(i); else ed += nbr(i);
   }
-  const T lap = T(1.0 / 3.0) * (ax - T(6) * c) + T(1.0 / 6.0) * (ed - T(12) * c);
-  const T a = c + T(p.dl), b = c + T(p.dg);
-  mu[at3(p, x, y, z)] = T(p.two_beta) * a * b * (a + b) - T(p.kappa) * lap;
+  mu[at3(p, x, y, z)] = mu3(ax, ed, c, consts3<T>(p));
 }
 
 // 12 grad(phi) = 36 sum_i w_i c_i phi(x + c_i): 2 (axis differences) +
@@ -183,9 +216,102 @@ __device__ __forceinline__ void grad3x12(const T* __restrict__ phi, const P3& p,
   const T exy1 = v(1, 1, 0) - v(-1, -1, 0), exy2 = v(1, -1, 0) - v(-1, 1, 0);
   const T exz1 = v(1, 0, 1) - v(-1, 0, -1), exz2 = v(1, 0, -1) - v(-1, 0, 1);
   const T eyz1 = v(0, 1, 1) - v(0, -1, -1), eyz2 = v(0, 1, -1) - v(0, -1, 1);
-  gx = T(2) * axx + ((exy1 + exy2) + (exz1 + exz2));
-  gy = T(2) * axy + ((exy1 - exy2) + (eyz1 + eyz2));
-  gz = T(2) * axz + ((exz1 - exz2) + (eyz1 - eyz2));
+  gx = fma(T(2), axx, (exy1 + exy2) + (exz1 + exz2));
+  gy = fma(T(2), axy, (exy1 - exy2) + (eyz1 + eyz2));
+  gz = fma(T(2), axz, (exz1 - exz2) + (eyz1 - eyz2));
+}
+
+// One component of F from 12 grad mu and 12 grad rho, nr = -rho / 12:
+// -rho grad mu (Eq. mF), or the potential form of the standard scheme.
+template <bool WB>
+__device__ __forceinline__ double force3(double nr, double gm, double gr) {
+  return WB ? nr * gm : (1.0 / 36.0) * gr + nr * gm;
+}
+template <bool WB>
+__device__ __forceinline__ float force3(float nr, float gm, float gr) {
+  return WB ? __fmul_rn(nr, gm) : __fmaf_rn(nr, gm, __fmul_rn(1.0f / 36.0f, gr));
+}
+// (j + F/2) / rho
+__device__ __forceinline__ double vel3(double j, double F, double inv) {
+  return (j + 0.5 * F) * inv;
+}
+__device__ __forceinline__ float vel3(float j, float F, float inv) {
+  return __fmul_rn(__fmaf_rn(0.5f, F, j), inv);
+}
+
+// a x + b y + c z, the first product of the innermost sum fused
+__device__ __forceinline__ float dot3(float ax, float bx, float ay, float by, float az, float bz) {
+  return __fmaf_rn(az, bz, __fmaf_rn(ax, bx, __fmul_rn(ay, by)));
+}
+
+// The FP32 update of one node's populations (the terms of d3_collide below):
+// F the force, gr 12 grad rho, key the node's number and ht the step's key
+// (the draw of the rest population's rounding).
+template <bool WB>
+__device__ __forceinline__ void update3_f32(float (&g)[19], float rs, float r, float Fx, float Fy,
+                                            float Fz, float grx, float gry, float grz, float ux,
+                                            float uy, float uz, const NodeConsts<float>& q,
+                                            uint32_t key, uint32_t ht) {
+  const float om = q.omega, kf = q.kf, keep = q.keep, c36 = 1.0f / 36.0f;
+  const float m_in = moving_sum3(g);
+  const float Gx = WB ? __fmaf_rn(c36, grx, Fx) : Fx;     // F + cs^2 grad rho
+  const float Gy = WB ? __fmaf_rn(c36, gry, Fy) : Fy;
+  const float Gz = WB ? __fmaf_rn(c36, grz, Fz) : Fz;
+  const float orho = __fmul_rn(om, r);
+  const float t = __fmaf_rn(__fmul_rn(-1.5f, orho), dot3(ux, ux, uy, uy, uz, uz),
+                            -__fmul_rn(__fmul_rn(3.0f, kf), dot3(ux, Gx, uy, Gy, uz, Gz)));
+  float Ca, Ce;
+  if (WB) {
+    const float ku = __fmul_rn(__fmul_rn(kf, 1.0f / 12.0f), dot3(ux, grx, uy, gry, uz, grz));
+    Ca = __fmul_rn(1.0f / 18.0f, t);
+    Ce = __fmul_rn(c36, __fmaf_rn(1.5f, ku, t));
+  } else {
+    const float b = __fmaf_rn(om, rs, t);
+    Ca = __fmul_rn(1.0f / 18.0f, b);
+    Ce = __fmul_rn(c36, b);
+  }
+  const float Aa = __fmul_rn(0.25f, orho), Ae = __fmul_rn(0.125f, orho);
+  const float kh = __fmul_rn(0.5f, kf), kq = __fmul_rn(0.25f, kf), k6 = __fmul_rn(kf, 1.0f / 6.0f);
+  const float o6 = __fmul_rn(orho, 1.0f / 6.0f);
+  const float Mx = __fmaf_rn(k6, Fx, __fmul_rn(o6, ux));
+  const float My = __fmaf_rn(k6, Fy, __fmul_rn(o6, uy));
+  const float Mz = __fmaf_rn(k6, Fz, __fmul_rn(o6, uz));
+  const float Key = __fmul_rn(kq, Gy), Kez = __fmul_rn(kq, Gz);
+  auto axis = [&](int i, int j, float cu, float G, float M) {
+    const float E = __fmaf_rn(cu, __fmaf_rn(kh, G, __fmul_rn(Aa, cu)), Ca);
+    g[i] = __fmaf_rn(keep, g[i], __fadd_rn(E, M));
+    g[j] = __fmaf_rn(keep, g[j], __fsub_rn(E, M));
+    return E;
+  };
+  auto edge = [&](int i, int j, float cu, float K, float S) {
+    const float E = __fmaf_rn(cu, __fmaf_rn(Ae, cu, K), Ce);
+    g[i] = __fmaf_rn(keep, g[i], __fmaf_rn(0.5f, S, E));
+    g[j] = __fmaf_rn(keep, g[j], __fmaf_rn(-0.5f, S, E));
+    return E;
+  };
+  const float Ea1 = axis(1, 2, ux, Gx, Mx);
+  const float Ea2 = axis(3, 4, uy, Gy, My);
+  const float Ea3 = axis(5, 6, uz, Gz, Mz);
+  const float Ee1 = edge(7, 8, __fadd_rn(ux, uy), __fmaf_rn(kq, Gx, Key), __fadd_rn(Mx, My));
+  const float Ee2 = edge(9, 10, __fsub_rn(ux, uy), __fmaf_rn(kq, Gx, -Key), __fsub_rn(Mx, My));
+  const float Ee3 = edge(11, 12, __fadd_rn(ux, uz), __fmaf_rn(kq, Gx, Kez), __fadd_rn(Mx, Mz));
+  const float Ee4 = edge(13, 14, __fsub_rn(ux, uz), __fmaf_rn(kq, Gx, -Kez), __fsub_rn(Mx, Mz));
+  const float Ee5 = edge(15, 16, __fadd_rn(uy, uz), __fadd_rn(Key, Kez), __fadd_rn(My, Mz));
+  const float Ee6 = edge(17, 18, __fsub_rn(uy, uz), __fsub_rn(Key, Kez), __fsub_rn(My, Mz));
+  if (WB) {
+    // The collision conserves the node's mass, so the rest population
+    // follows from the balance: g_0' = g_0 + omega m_in - 2 sum E (the
+    // moving ones leave as keep g + E +- O).  Its small one-signed O(u^2)
+    // part would be lost in rounding g_0 ~ rho - rho_ref to float; TwoSum
+    // keeps the remainder and a zero-mean rounding, seeded by the node and
+    // the step, takes it into account.
+    const float sE = ((Ea1 + Ea2) + Ea3) + (((Ee1 + Ee2) + (Ee3 + Ee4)) + (Ee5 + Ee6));
+    float hsum, err;
+    two_sum1(g[0], __fmaf_rn(-2.0f, sE, __fmul_rn(om, m_in)), hsum, err);
+    g[0] = round_stochastic1(hsum, err, node_uniform(key, ht));
+  } else {
+    g[0] = __fsub_rn(rs, moving_sum3(g));      // the standard scheme: the mass balance
+  }
 }
 
 // The collision of one node, and its stores (MOMENTS: fields and stats
@@ -216,23 +342,15 @@ __global__ void __launch_bounds__(kBlock3) d3_collide(const T* __restrict__ src,
                                    wrap3(z - cz3(i), p.nz))];
     const long long k = at3(p, x, y, z);
     const T rs = rho[k];                         // rho - rho_ref (rho in FP64)
-    const T r = kShifted ? rs + T(p.rho_ref) : rs;
+    const T r = kShifted ? rs + consts3<T>(p).rho_ref : rs;
     // 12 grad mu, 12 grad rho; F = -rho grad mu (Eq. mF), or the potential
     // form cs^2 grad rho - rho grad mu of the standard scheme
     T gmx, gmy, gmz, grx, gry, grz;
     grad3x12<T>(mu, p, x, y, z, gmx, gmy, gmz);
     grad3x12<T>(rho, p, x, y, z, grx, gry, grz);
     const T nr = r * T(-1.0 / 12.0);
-    T Fx, Fy, Fz;
-    if (WB) {
-      Fx = nr * gmx;
-      Fy = nr * gmy;
-      Fz = nr * gmz;
-    } else {
-      Fx = T(1.0 / 36.0) * grx + nr * gmx;
-      Fy = T(1.0 / 36.0) * gry + nr * gmy;
-      Fz = T(1.0 / 36.0) * grz + nr * gmz;
-    }
+    const T Fx = force3<WB>(nr, gmx, grx), Fy = force3<WB>(nr, gmy, gry),
+            Fz = force3<WB>(nr, gmz, grz);
     // momentum from the differences of opposite pairs (each edge difference
     // serves two components)
     const T d12 = g[1] - g[2], d34 = g[3] - g[4], d56 = g[5] - g[6];
@@ -242,8 +360,7 @@ __global__ void __launch_bounds__(kBlock3) d3_collide(const T* __restrict__ src,
     const T jy = ((d34 + d78) - (d910 - d1516)) + d1718;
     const T jz = ((d56 + d1112) - (d1314 - d1516)) - d1718;
     const T inv = recip(r);
-    const T ux = (jx + T(0.5) * Fx) * inv, uy = (jy + T(0.5) * Fy) * inv,
-            uz = (jz + T(0.5) * Fz) * inv;                       // Eq. rhoU
+    const T ux = vel3(jx, Fx, inv), uy = vel3(jy, Fy, inv), uz = vel3(jz, Fz, inv);  // Eq. rhoU
     const T muc = mu[k];
     if (MOMENTS) {
       const double rd = kShifted ? (double)rs + p.rho_ref : (double)r;
@@ -261,80 +378,56 @@ __global__ void __launch_bounds__(kBlock3) d3_collide(const T* __restrict__ src,
       st[4] = mud;
       st[5] = (!isfinite(rd) || !isfinite(mud) || !isfinite(u2)) ? 1.0 : 0.0;
     } else {
-      T om = T(p.omega);
-      const T kf = T(p.kforce);
-      T keep = T(1) - om;
-      if (kShifted && om < T(0.5)) {
-        // keep + omega == 1 exactly in float (the update then conserves
-        // mass); 1 - omega is exact by Sterbenz only for omega >= 1/2
-        keep = T(1.0 - p.omega);
-        om = T(1) - keep;
-      }
-      // FP32: the moving populations' sum before the collision (the same
-      // grouping as the density), for the exact node mass balance below
-      const T m_in = kShifted ? moving_sum3(g) : T(0);
-      T Gx = Fx, Gy = Fy, Gz = Fz;
-      if (WB) {
-        Gx = Fx + T(1.0 / 36.0) * grx;                          // G = F + cs^2 grad rho
-        Gy = Fy + T(1.0 / 36.0) * gry;
-        Gz = Fz + T(1.0 / 36.0) * grz;
-      }
-      const T orho = om * r;
-      const T obase = om * rs;                   // omega (rho - rho_ref): the stored base
-      const T t = T(-1.5) * orho * (ux * ux + uy * uy + uz * uz) -
-                  T(3.0) * kf * (ux * Gx + uy * Gy + uz * Gz);
-      const T ku = WB ? (kf * T(1.0 / 12.0)) * (ux * grx + uy * gry + uz * grz) : T(0);
-      // per-node constants of the pairs, with the weights folded in
-      // (w_ax = 1/18, w_edge = 1/36): E = C + cu (A cu + K.c), O = 3 w c.M
-      const T Ca = WB ? T(1.0 / 18.0) * t : T(1.0 / 18.0) * (t + obase);
-      const T Ce = WB ? T(1.0 / 36.0) * (t + T(1.5) * ku) : T(1.0 / 36.0) * (t + obase);
-      const T Aa = T(0.25) * orho, Ae = T(0.125) * orho;         // w 9/2 omega rho
-      const T kh = T(0.5) * kf, kq = T(0.25) * kf, k6 = kf * T(1.0 / 6.0);
-      const T Kax = kh * Gx, Kay = kh * Gy, Kaz = kh * Gz;       // 9 w_ax kforce G
-      const T Kex = kq * Gx, Key = kq * Gy, Kez = kq * Gz;       // 9 w_edge kforce G
-      const T o6 = orho * T(1.0 / 6.0);                          // 3 w_ax (omega rho u + kforce F)
-      const T Mx = o6 * ux + k6 * Fx, My = o6 * uy + k6 * Fy, Mz = o6 * uz + k6 * Fz;
-      auto axis = [&](int i, int j, T cu, T K, T M) {
-        const T E = Ca + cu * (Aa * cu + K);
-        g[i] = keep * g[i] + (E + M);
-        g[j] = keep * g[j] + (E - M);
-        return E;
-      };
-      // edge pair: 3 w_edge c.M = (Ma + Mb) / 2 for c = a + b
-      auto edge = [&](int i, int j, T cu, T K, T S) {
-        const T E = Ce + cu * (Ae * cu + K);
-        g[i] = keep * g[i] + (E + T(0.5) * S);
-        g[j] = keep * g[j] + (E - T(0.5) * S);
-        return E;
-      };
-      const T Ea1 = axis(1, 2, ux, Kax, Mx);
-      const T Ea2 = axis(3, 4, uy, Kay, My);
-      const T Ea3 = axis(5, 6, uz, Kaz, Mz);
-      const T Ee1 = edge(7, 8, ux + uy, Kex + Key, Mx + My);
-      const T Ee2 = edge(9, 10, ux - uy, Kex - Key, Mx - My);
-      const T Ee3 = edge(11, 12, ux + uz, Kex + Kez, Mx + Mz);
-      const T Ee4 = edge(13, 14, ux - uz, Kex - Kez, Mx - Mz);
-      const T Ee5 = edge(15, 16, uy + uz, Key + Kez, My + Mz);
-      const T Ee6 = edge(17, 18, uy - uz, Key - Kez, My - Mz);
+      const NodeConsts<T> q = consts3<T>(p);
       if constexpr (kShifted) {
-        if (WB) {
-          // The collision conserves the node's mass, so the rest population
-          // follows from the balance: g_0' = g_0 + omega m_in - 2 sum E (the
-          // moving ones leave as keep g + E +- O).  Its small one-signed
-          // O(u^2) part would be lost in rounding g_0 ~ rho - rho_ref to
-          // float; TwoSum keeps the remainder and a zero-mean rounding,
-          // seeded by the node and the step, takes it into account.
-          const T sE = ((Ea1 + Ea2) + Ea3) + (((Ee1 + Ee2) + (Ee3 + Ee4)) + (Ee5 + Ee6));
-          T hsum, err;
-          two_sum1(g[0], __fmaf_rn(-2.0f, sE, om * m_in), hsum, err);
-          const uint32_t key = (uint32_t)(((long long)z * p.ny + y) * p.nx + x);
-          g[0] = round_stochastic1(hsum, err, node_uniform(key, step_key(p.step)));
-        } else {
-          g[0] = rs - moving_sum3(g);          // the standard scheme: the mass balance
-        }
+        const uint32_t key = (uint32_t)(((long long)z * p.ny + y) * p.nx + x);
+        update3_f32<WB>(g, rs, r, Fx, Fy, Fz, grx, gry, grz, ux, uy, uz, q, key,
+                        step_key(p.step));
       } else {
-        (void)Ea1; (void)Ea2; (void)Ea3; (void)Ee1; (void)Ee2; (void)Ee3;
-        (void)Ee4; (void)Ee5; (void)Ee6; (void)m_in;
+        const T om = q.omega, kf = q.kf, keep = q.keep;
+        T Gx = Fx, Gy = Fy, Gz = Fz;
+        if (WB) {
+          Gx = Fx + T(1.0 / 36.0) * grx;                          // G = F + cs^2 grad rho
+          Gy = Fy + T(1.0 / 36.0) * gry;
+          Gz = Fz + T(1.0 / 36.0) * grz;
+        }
+        const T orho = om * r;
+        const T obase = om * rs;                   // omega (rho - rho_ref): the stored base
+        const T t = T(-1.5) * orho * (ux * ux + uy * uy + uz * uz) -
+                    T(3.0) * kf * (ux * Gx + uy * Gy + uz * Gz);
+        const T ku = WB ? (kf * T(1.0 / 12.0)) * (ux * grx + uy * gry + uz * grz) : T(0);
+        // per-node constants of the pairs, with the weights folded in
+        // (w_ax = 1/18, w_edge = 1/36): E = C + cu (A cu + K.c), O = 3 w c.M
+        const T Ca = WB ? T(1.0 / 18.0) * t : T(1.0 / 18.0) * (t + obase);
+        const T Ce = WB ? T(1.0 / 36.0) * (t + T(1.5) * ku) : T(1.0 / 36.0) * (t + obase);
+        const T Aa = T(0.25) * orho, Ae = T(0.125) * orho;         // w 9/2 omega rho
+        const T kh = T(0.5) * kf, kq = T(0.25) * kf, k6 = kf * T(1.0 / 6.0);
+        const T Kax = kh * Gx, Kay = kh * Gy, Kaz = kh * Gz;       // 9 w_ax kforce G
+        const T Kex = kq * Gx, Key = kq * Gy, Kez = kq * Gz;       // 9 w_edge kforce G
+        const T o6 = orho * T(1.0 / 6.0);                          // 3 w_ax (omega rho u + kforce F)
+        const T Mx = o6 * ux + k6 * Fx, My = o6 * uy + k6 * Fy, Mz = o6 * uz + k6 * Fz;
+        auto axis = [&](int i, int j, T cu, T K, T M) {
+          const T E = Ca + cu * (Aa * cu + K);
+          g[i] = keep * g[i] + (E + M);
+          g[j] = keep * g[j] + (E - M);
+          return E;
+        };
+        // edge pair: 3 w_edge c.M = (Ma + Mb) / 2 for c = a + b
+        auto edge = [&](int i, int j, T cu, T K, T S) {
+          const T E = Ce + cu * (Ae * cu + K);
+          g[i] = keep * g[i] + (E + T(0.5) * S);
+          g[j] = keep * g[j] + (E - T(0.5) * S);
+          return E;
+        };
+        const T Ea1 = axis(1, 2, ux, Kax, Mx);
+        const T Ea2 = axis(3, 4, uy, Kay, My);
+        const T Ea3 = axis(5, 6, uz, Kaz, Mz);
+        const T Ee1 = edge(7, 8, ux + uy, Kex + Key, Mx + My);
+        const T Ee2 = edge(9, 10, ux - uy, Kex - Key, Mx - My);
+        const T Ee3 = edge(11, 12, ux + uz, Kex + Kez, Mx + Mz);
+        const T Ee4 = edge(13, 14, ux - uz, Kex - Kez, Mx - Mz);
+        const T Ee5 = edge(15, 16, uy + uz, Key + Kez, My + Mz);
+        const T Ee6 = edge(17, 18, uy - uz, Key - Kez, My - Mz);
         // rest: WB f_0^eq - s_0 = rho - w_0 3/2 rho u.u, F_0 = w_0 (-3 u.G - 3/2 u.grad rho);
         // standard f_0^eq = w_0 rho (1 - 3/2 u.u), F_0 = w_0 (-3 u.G)
         const T w0 = T(1.0 / 3.0);
@@ -508,16 +601,15 @@ P3 p3_of(const wblbe3_ctx* h) {
   q.nz = h->p.nz;
   q.pitch = h->L.pitch;
   q.plane = h->L.plane;
+  // FP32 stores deviations from the rest equilibrium at rho_ref = rho_g
+  q.rho_ref = h->p.precision == WBLBE_FP64 ? 0.0 : h->p.rho_g;
   q.omega = 1.0 / h->p.tau;
   q.kforce = 1.0 - 1.0 / (2.0 * h->p.tau);
   q.kappa = h->p.kappa;
   q.two_beta = 2.0 * h->p.beta;
-  q.rho_l = h->p.rho_l;
-  q.rho_g = h->p.rho_g;
-  // FP32 stores deviations from the rest equilibrium at rho_ref = rho_g
-  q.rho_ref = h->p.precision == WBLBE_FP64 ? 0.0 : h->p.rho_g;
   q.dl = q.rho_ref - h->p.rho_l;
   q.dg = q.rho_ref - h->p.rho_g;
+  q.f.set(q.omega, q.kforce, q.kappa, q.two_beta, q.dl, q.dg, q.rho_ref);
   q.step = h->steps;
   return q;
 }

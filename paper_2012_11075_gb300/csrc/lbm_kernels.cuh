@@ -32,17 +32,57 @@ namespace wblbe {
 constexpr int kHalo = 2;          // density halo radius (mu needs 1, grad mu 2)
 constexpr int kMaxTile = 256;
 
+// Constants of the node update in the arithmetic type.  The host converts
+// them once (set_physics): a float <- double conversion in a kernel runs on
+// the FP64 pipe, which GB300 has at two lanes per SM and clock, and nvcc
+// repeats it inside the row loop rather than hold its result in a register.
+// FP32 step of the 4096^2 well-balanced lattice: FP64 pipe busy 48 % of the
+// time with conversions in the kernel, 235.8 us per step; without, 218.5 us.
+// keep = 1 - omega must hold exactly in the arithmetic type: the update
+// keep * g + omega * (...) conserves mass only if keep + omega == 1, and a
+// rounded pair would scale the mass every step.  For omega >= 1/2 (tau <= 2)
+// 1 - omega is exact (Sterbenz); for smaller omega, omega is taken as 1 - keep.
+template <typename T>
+struct NodeConsts {
+  T omega, keep, kf, kf_m3, kf12;   // 1/tau, 1 - omega, 1 - 1/(2 tau), -3 kf, kf/12
+  T kfm12, kf36, kf432;             // -kf/12, kf/36, kf/432 (collide_wb12)
+  T rho_ref, kappa, kappa6;         // kappa6 = kappa / 6
+  T two_beta, half_beta, dl, dg;    // 2 beta, beta, rho_ref - rho_l, rho_ref - rho_g
+
+  __host__ __device__ void set(double om, double kforce, double kappa_, double two_beta_, double dl_, double dg_,
+           double rho_ref_) {
+    const T w = T(om);
+    if (w >= T(0.5)) {
+      omega = w;
+      keep = T(1) - w;
+    } else {
+      keep = T(1.0 - om);
+      omega = T(1) - keep;
+    }
+    kf = T(kforce);
+    kf_m3 = T(-3.0 * kforce);
+    kf12 = T(kforce / 12.0);
+    kfm12 = T(-kforce / 12.0);
+    kf36 = T(kforce / 36.0);
+    kf432 = T(kforce / 432.0);
+    rho_ref = T(rho_ref_);
+    kappa = T(kappa_);
+    kappa6 = T(kappa_ / 6.0);
+    two_beta = T(two_beta_);
+    half_beta = T(0.5 * two_beta_);
+    dl = T(dl_);
+    dg = T(dg_);
+  }
+};
+
 // Parameters of one launch, passed by value.
 struct KParams {
   int nx, ny, pitch, rows;        // rows: lattice rows marched by one CTA
   long long plane;                // elements per population plane
-  // physics (stored as double; cast to the arithmetic type in the kernel)
-  double omega;                   // 1/tau
-  double kforce;                  // 1 - 1/(2 tau)
-  double kappa;
-  double two_beta;                // 2 beta
-  double dl, dg;                  // rho_ref - rho_l, rho_ref - rho_g
-  double rho_ref;                 // 0 in FP64
+  // physics, and the FP32 update's constants converted from it
+  double omega, kforce, kappa, two_beta;   // 1/tau, 1 - 1/(2 tau), kappa, 2 beta
+  double dl, dg, rho_ref;         // rho_ref - rho_l, rho_ref - rho_g, shift (0 in FP64)
+  NodeConsts<float> f;
   // Time step t of the state being updated, which seeds the stochastic
   // rounding of the FP32 well-balanced update: t = step + *step_base
   // (step_base may be null; a graph replay reads its base from device memory).
@@ -55,6 +95,29 @@ struct KParams {
   // rows around them).
   int row_lo, row_hi, y_offset;
 };
+
+// Fill the physics of a launch from the paper's parameters (Sec. IV) and the
+// storage shift density rho_ref (0 in FP64).
+inline void set_physics(KParams& k, double tau, double kappa, double beta, double rho_l,
+                        double rho_g, double rho_ref) {
+  k.omega = 1.0 / tau;
+  k.kforce = 1.0 - 1.0 / (2.0 * tau);
+  k.kappa = kappa;
+  k.two_beta = 2.0 * beta;
+  k.dl = rho_ref - rho_l;
+  k.dg = rho_ref - rho_g;
+  k.rho_ref = rho_ref;
+  k.f.set(k.omega, k.kforce, k.kappa, k.two_beta, k.dl, k.dg, k.rho_ref);
+}
+
+// The launch's constants in the arithmetic type (FP64: formed in the kernel,
+// no conversion is needed).
+__device__ __forceinline__ NodeConsts<float> consts_of(const KParams& p, float) { return p.f; }
+__device__ __forceinline__ NodeConsts<double> consts_of(const KParams& p, double) {
+  NodeConsts<double> q;
+  q.set(p.omega, p.kforce, p.kappa, p.two_beta, p.dl, p.dg, p.rho_ref);
+  return q;
+}
 
 // Outputs of the moments mode (any pointer may be null).
 struct MomentsOut {
@@ -164,34 +227,10 @@ __device__ __forceinline__ double recip(double x) {
   return fma(r, fma(e, e, e), r);
 }
 
-// Collision constants in the arithmetic type, converted once per kernel (a
-// float <- double conversion inside the row loop would run on the FP64 pipe).
 // The rho0 terms of the well-balanced equilibrium never reach the kernel: in
 // both precisions the planes store deviations from a shift that contains the
 // node-independent rho0 vector (-(1-w0) rho0, w_i rho0), which the BGK update
 // and streaming carry unchanged.
-// keep = 1 - omega must hold exactly in the arithmetic type: the update
-// keep * g + omega * (...) conserves mass only if keep + omega == 1, and a
-// rounded pair would scale the mass every step.  For omega >= 1/2 (tau <= 2)
-// 1 - omega is exact (Sterbenz); for smaller omega, omega is taken as 1 - keep.
-template <typename T>
-struct CollideConsts {
-  T omega, kf, keep, kf_m3, rho_ref, kappa, kf12;
-  T kfm12, kf36, kf432;             // -kforce/12, kforce/36, kforce/432 (collide_wb12)
-  __device__ explicit CollideConsts(const KParams& p)
-      : kf(T(p.kforce)), kf_m3(T(-3.0 * p.kforce)), rho_ref(T(p.rho_ref)), kappa(T(p.kappa)),
-        kf12(T(p.kforce / 12.0)), kfm12(T(-p.kforce / 12.0)), kf36(T(p.kforce / 36.0)),
-        kf432(T(p.kforce / 432.0)) {
-    const T w = T(p.omega);
-    if (w >= T(0.5)) {
-      omega = w;
-      keep = T(1) - w;
-    } else {
-      keep = T(1.0 - p.omega);
-      omega = T(1) - keep;
-    }
-  }
-};
 
 // Collision of one node in stored variables.  Inputs: the nine pulled
 // populations g, the stored density rs (rho = rs + rho_ref), gradients of mu
@@ -214,7 +253,7 @@ struct CollideConsts {
 // textbook forcing term the collision takes textbook_pairs below.
 template <typename T>
 __device__ __forceinline__ void textbook_pairs(T (&g)[9], T rs, T rho, T ux, T uy, T Fx,
-                                               T Fy, const CollideConsts<T>& q);
+                                               T Fy, const NodeConsts<T>& q);
 
 // The well-balanced collision from 12 grad mu and 12 grad rho (iso_grad12),
 // the same terms as collide below arranged for fewer operations, which is
@@ -225,7 +264,7 @@ __device__ __forceinline__ void textbook_pairs(T (&g)[9], T rs, T rho, T ux, T u
 // E_dg = t' + 2 k_u', E_ax = 3 t' + E_dg and E_0 = 16 (t' - k_u') + omega b_0.
 template <typename T>
 __device__ __forceinline__ void collide_wb12(T (&g)[9], T rs, T gmx, T gmy, T grx, T gry,
-                                             const CollideConsts<T>& q, T& ux_out,
+                                             const NodeConsts<T>& q, T& ux_out,
                                              T& uy_out) {
   constexpr bool kShifted = sizeof(T) == 4;
   const T omega = q.omega;
@@ -285,7 +324,7 @@ __device__ __forceinline__ void collide_wb12(T (&g)[9], T rs, T gmx, T gmy, T gr
 // few places that use them; 1: plain gradients).
 template <typename T, int SCH, int GS = 1>
 __device__ __forceinline__ void collide(T (&g)[9], T rs, T gmx, T gmy, T grx,
-                                        T gry, const CollideConsts<T>& q, T& ux_out,
+                                        T gry, const NodeConsts<T>& q, T& ux_out,
                                         T& uy_out) {
   constexpr bool WB = SCH == kSchWB;
   constexpr bool kShifted = sizeof(T) == 4;   // FP32 storage is always shifted
@@ -410,7 +449,7 @@ __device__ __forceinline__ void collide(T (&g)[9], T rs, T gmx, T gmy, T grx,
 //   O = omega w rho 3 c.u + kforce 3w (e c.F - 3 (c.u) u.F).
 template <typename T>
 __device__ __forceinline__ void textbook_pairs(T (&g)[9], T rs, T rho, T ux, T uy, T Fx,
-                                               T Fy, const CollideConsts<T>& q) {
+                                               T Fy, const NodeConsts<T>& q) {
   constexpr bool kShifted = sizeof(T) == 4;
   const T omega = q.omega, kf = q.kf, keep = q.keep;
   const T uu = ux * ux + uy * uy, uF = ux * Fx + uy * Fy;
@@ -596,7 +635,7 @@ __device__ __forceinline__ void iso_grad_x2(float2 e, float2 w, float2 n, float2
 // textbook_pairs<float> on a pair of nodes
 __device__ __forceinline__ void textbook_pairs_x2(float2 (&g)[9], float2 rs, float2 rho,
                                                   float2 ux, float2 uy, float2 Fx, float2 Fy,
-                                                  const CollideConsts<float>& q) {
+                                                  const NodeConsts<float>& q) {
   const float2 omega = splat(q.omega), kf3 = mul2(splat(q.kf), splat(3.0f)), keep = splat(q.keep);
   const float2 uu = fma2(ux, ux, mul2(uy, uy)), uF = fma2(ux, Fx, mul2(uy, Fy));
   const float2 e0 = fma2(splat(-1.5f), uu, splat(1.0f));
@@ -633,7 +672,7 @@ __device__ __forceinline__ void textbook_pairs_x2(float2 (&g)[9], float2 rs, flo
 // population (well-balanced scheme only, see round_stochastic).
 template <int SCH>
 __device__ __forceinline__ void collide_x2(float2 (&g)[9], float2 rs, float2 gmx, float2 gmy,
-                                           float2 grx, float2 gry, const CollideConsts<float>& q,
+                                           float2 grx, float2 gry, const NodeConsts<float>& q,
                                            float2& ux_out, float2& uy_out, float2 rnd) {
   constexpr bool WB = SCH == kSchWB;
   const float2 omega = splat(q.omega), kf = splat(q.kf), third = splat(1.0f / 3.0f);
@@ -861,6 +900,50 @@ struct StatsAcc {
   int bad = 0;
 };
 
+// One CTA's statistics record from its threads' accumulators (every thread of
+// the CTA calls it): warp shuffles, then thread 0 over the warps; a fixed
+// order, so the record does not vary from run to run.
+template <int NT>
+__device__ __forceinline__ void write_stats_record(const StatsAcc& acc, double* rec) {
+  __shared__ double red[NT / 32][kStatRec];
+  double v[kStatRec] = {acc.mass, acc.kin, acc.u2, acc.mumin, acc.mumax, (double)acc.bad};
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    double o0 = __shfl_down_sync(0xffffffffu, v[0], off);
+    double o1 = __shfl_down_sync(0xffffffffu, v[1], off);
+    double o2 = __shfl_down_sync(0xffffffffu, v[2], off);
+    double o3 = __shfl_down_sync(0xffffffffu, v[3], off);
+    double o4 = __shfl_down_sync(0xffffffffu, v[4], off);
+    double o5 = __shfl_down_sync(0xffffffffu, v[5], off);
+    v[0] += o0;
+    v[1] += o1;
+    v[2] = fmax(v[2], o2);
+    v[3] = fmin(v[3], o3);
+    v[4] = fmax(v[4], o4);
+    v[5] = fmax(v[5], o5);
+  }
+  const int tx = threadIdx.x, warp = tx >> 5, lane = tx & 31;
+  if (lane == 0)
+#pragma unroll
+    for (int q = 0; q < kStatRec; ++q) red[warp][q] = v[q];
+  __syncthreads();
+  if (tx == 0) {
+    double r[kStatRec];
+#pragma unroll
+    for (int q = 0; q < kStatRec; ++q) r[q] = red[0][q];
+    for (int q = 1; q < NT / 32; ++q) {
+      r[0] += red[q][0];
+      r[1] += red[q][1];
+      r[2] = fmax(r[2], red[q][2]);
+      r[3] = fmin(r[3], red[q][3]);
+      r[4] = fmax(r[4], red[q][4]);
+      r[5] = fmax(r[5], red[q][5]);
+    }
+#pragma unroll
+    for (int q = 0; q < kStatRec; ++q) rec[q] = r[q];
+  }
+}
+
 // One collided node of row c: store its nine populations (and the ghost
 // copies of a boundary column), or write its moment fields, and fold its
 // statistics.  Forced inline so that the population array stays in registers.
@@ -964,15 +1047,15 @@ __device__ __forceinline__ void strip_pass(const T* __restrict__ src, T* __restr
   // each side, rounded up to whole chunks; never past the stage row)
   const int nch_rt = GHOST ? (w + 2 * kPad + E - 1) / E : NCH;
 
-  const T two_beta = T(p.two_beta), dl = T(p.dl), dg = T(p.dg), kappa6 = T(p.kappa / 6.0);
-  const CollideConsts<T> cc(p);
+  const NodeConsts<T> cc = consts_of(p, T(0));
+  const T two_beta = cc.two_beta, dl = cc.dl, dg = cc.dg, kappa6 = cc.kappa6;
   // The second ring holds mu, or lap(rho) with the pressure-form force
   // (chem_pot with beta = 0 and kappa/6 -> -1/6 gives exactly lap(rho)); the
   // gradient carried to the collision is grad(rho), or grad(cs^2 rho - p_0).
   constexpr bool kPress = SCH == kSchPressure;
   const T ring_tb = kPress ? T(0) : two_beta;
   const T ring_k6 = kPress ? T(-1.0 / 6.0) : kappa6;
-  const T half_beta = T(0.5 * p.two_beta), rho_ref_t = T(p.rho_ref);
+  const T half_beta = cc.half_beta, rho_ref_t = cc.rho_ref;
   // cs^2 rho - p_0 from a stored density v (rho = v + rho_ref, up to a
   // constant): p_0 = rho mu_0 - psi_0 = beta a b (2 rho (a + b) - a b),
   // a = rho - rho_l, b = rho - rho_g
@@ -1340,46 +1423,7 @@ __device__ __forceinline__ void strip_pass(const T* __restrict__ src, T* __restr
   }
   cp_async_wait<0>();
 
-  if (STATS && stats_rec) {
-    // deterministic block reduction: warp shuffle, then thread 0 over warps
-    __shared__ double red[kMaxTile / 32][kStatRec];
-    double v[kStatRec] = {acc.mass, acc.kin, acc.u2, acc.mumin, acc.mumax, (double)acc.bad};
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      double o0 = __shfl_down_sync(0xffffffffu, v[0], off);
-      double o1 = __shfl_down_sync(0xffffffffu, v[1], off);
-      double o2 = __shfl_down_sync(0xffffffffu, v[2], off);
-      double o3 = __shfl_down_sync(0xffffffffu, v[3], off);
-      double o4 = __shfl_down_sync(0xffffffffu, v[4], off);
-      double o5 = __shfl_down_sync(0xffffffffu, v[5], off);
-      v[0] += o0;
-      v[1] += o1;
-      v[2] = fmax(v[2], o2);
-      v[3] = fmin(v[3], o3);
-      v[4] = fmax(v[4], o4);
-      v[5] = fmax(v[5], o5);
-    }
-    const int warp = tx >> 5, lane = tx & 31, nw = TX >> 5;
-    if (lane == 0)
-#pragma unroll
-      for (int q = 0; q < kStatRec; ++q) red[warp][q] = v[q];
-    __syncthreads();
-    if (tx == 0) {
-      double r[kStatRec];
-#pragma unroll
-      for (int q = 0; q < kStatRec; ++q) r[q] = red[0][q];
-      for (int q = 1; q < nw; ++q) {
-        r[0] += red[q][0];
-        r[1] += red[q][1];
-        r[2] = fmax(r[2], red[q][2]);
-        r[3] = fmin(r[3], red[q][3]);
-        r[4] = fmax(r[4], red[q][4]);
-        r[5] = fmax(r[5], red[q][5]);
-      }
-#pragma unroll
-      for (int q = 0; q < kStatRec; ++q) stats_rec[q] = r[q];
-    }
-  }
+  if (STATS && stats_rec) write_stats_record<TX>(acc, stats_rec);
 }
 
 // One CTA per strip segment: blockIdx.x picks the strip, blockIdx.y the run

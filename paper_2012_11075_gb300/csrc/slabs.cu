@@ -253,14 +253,7 @@ KParams slab_kparams(const wblbe_slabs* h, int k, int rows) {
   kp.pitch = h->pitch;
   kp.rows = rows;
   kp.plane = s.plane;
-  kp.omega = 1.0 / p.tau;
-  kp.kforce = 1.0 - 1.0 / (2.0 * p.tau);
-  kp.kappa = p.kappa;
-  kp.two_beta = 2.0 * p.beta;
-  const double rr = slab_rho_ref(p);
-  kp.rho_ref = rr;
-  kp.dl = rr - p.rho_l;
-  kp.dg = rr - p.rho_g;
+  set_physics(kp, p.tau, p.kappa, p.beta, p.rho_l, p.rho_g, slab_rho_ref(p));
   kp.step = h->steps;
   kp.row_lo = kGhost;
   kp.row_hi = kGhost + s.n;

@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(kE6Threads)
                                kappa6);
   }
   __syncthreads();
-  const CollideConsts<double> cc(p);
+  const NodeConsts<double> cc = consts_of(p, 0.0);
   StatsAcc acc;
   const bool acc_on = MODE != kModeStep;
 #pragma unroll

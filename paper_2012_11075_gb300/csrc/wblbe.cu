@@ -161,14 +161,7 @@ KParams make_kparams(const wblbe_ctx* h, int rows) {
   k.pitch = h->L.pitch;
   k.rows = rows;
   k.plane = h->L.plane;
-  k.omega = 1.0 / p.tau;
-  k.kforce = 1.0 - 1.0 / (2.0 * p.tau);
-  k.kappa = p.kappa;
-  k.two_beta = 2.0 * p.beta;
-  const double rr = rho_ref_of(p);
-  k.rho_ref = rr;
-  k.dl = rr - p.rho_l;
-  k.dg = rr - p.rho_g;
+  set_physics(k, p.tau, p.kappa, p.beta, p.rho_l, p.rho_g, rho_ref_of(p));
   k.row_lo = 0;
   k.row_hi = p.ny;
   k.y_offset = 0;

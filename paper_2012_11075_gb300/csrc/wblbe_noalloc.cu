@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(kTileX* kTileY)
     for (int i = 0; i < 9; ++i) g[i] = f[i * plane + k];
     const double rs = rho_s[ry][rx];
     double ux, uy;
-    const CollideConsts<double> cc(p);
+    const NodeConsts<double> cc = consts_of(p, 0.0);
     collide<double, WB ? kSchWB : kSchStandard>(g, rs, gmx, gmy, grx, gry, cc, ux, uy);
     const double mu = mu_s[my][mx];
     if (rho_out) rho_out[k] = rs;
@@ -209,13 +209,7 @@ wblbe_status wblbe_moments_noalloc(const wblbe_params* params, const double* f,
   KParams kp{};
   kp.nx = params->nx;
   kp.ny = params->ny;
-  kp.omega = 1.0 / params->tau;
-  kp.kforce = 1.0 - 1.0 / (2.0 * params->tau);
-  kp.kappa = params->kappa;
-  kp.two_beta = 2.0 * params->beta;
-  kp.dl = -params->rho_l;
-  kp.dg = -params->rho_g;
-  kp.rho_ref = 0.0;
+  set_physics(kp, params->tau, params->kappa, params->beta, params->rho_l, params->rho_g, 0.0);
 
   dim3 grid((unsigned)gx, (unsigned)gy), block(kTileX, kTileY);
   if (params->scheme == WBLBE_WELL_BALANCED)
