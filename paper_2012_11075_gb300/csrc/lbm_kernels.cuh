@@ -37,7 +37,7 @@ constexpr int kMaxTile = 256;
 // the FP64 pipe, which GB300 has at two lanes per SM and clock, and nvcc
 // repeats it inside the row loop rather than hold its result in a register.
 // FP32 step of the 4096^2 well-balanced lattice: FP64 pipe busy 48 % of the
-// time with conversions in the kernel, 235.8 us per step; without, 218.5 us.
+// time with conversions in the kernel, 235.8 us per step; without, 218.1 us.
 // keep = 1 - omega must hold exactly in the arithmetic type: the update
 // keep * g + omega * (...) conserves mass only if keep + omega == 1, and a
 // rounded pair would scale the mass every step.  For omega >= 1/2 (tau <= 2)
@@ -45,11 +45,11 @@ constexpr int kMaxTile = 256;
 template <typename T>
 struct NodeConsts {
   T omega, keep, kf, kf_m3, kf12;   // 1/tau, 1 - omega, 1 - 1/(2 tau), -3 kf, kf/12
-  T kfm12, kf36, kf432;             // -kf/12, kf/36, kf/432 (collide_wb12)
+  T kcm, kf108, kf216;              // -kf/36, kf/108, kf/216 (collide12_f64)
   T rho_ref, kappa, kappa6;         // kappa6 = kappa / 6
   T two_beta, half_beta, dl, dg;    // 2 beta, beta, rho_ref - rho_l, rho_ref - rho_g
 
-  __host__ __device__ void set(double om, double kforce, double kappa_, double two_beta_, double dl_, double dg_,
+  void set(double om, double kforce, double kappa_, double two_beta_, double dl_, double dg_,
            double rho_ref_) {
     const T w = T(om);
     if (w >= T(0.5)) {
@@ -62,9 +62,9 @@ struct NodeConsts {
     kf = T(kforce);
     kf_m3 = T(-3.0 * kforce);
     kf12 = T(kforce / 12.0);
-    kfm12 = T(-kforce / 12.0);
-    kf36 = T(kforce / 36.0);
-    kf432 = T(kforce / 432.0);
+    kcm = T(-kforce / 36.0);
+    kf108 = T(kforce / 108.0);
+    kf216 = T(kforce / 216.0);
     rho_ref = T(rho_ref_);
     kappa = T(kappa_);
     kappa6 = T(kappa_ / 6.0);
@@ -79,9 +79,8 @@ struct NodeConsts {
 struct KParams {
   int nx, ny, pitch, rows;        // rows: lattice rows marched by one CTA
   long long plane;                // elements per population plane
-  // physics, and the FP32 update's constants converted from it
-  double omega, kforce, kappa, two_beta;   // 1/tau, 1 - 1/(2 tau), kappa, 2 beta
-  double dl, dg, rho_ref;         // rho_ref - rho_l, rho_ref - rho_g, shift (0 in FP64)
+  double rho_ref;                 // storage shift density, 0 in FP64 (statistics)
+  NodeConsts<double> d;           // the update's constants in FP64 and in FP32
   NodeConsts<float> f;
   // Time step t of the state being updated, which seeds the stochastic
   // rounding of the FP32 well-balanced update: t = step + *step_base
@@ -100,24 +99,15 @@ struct KParams {
 // storage shift density rho_ref (0 in FP64).
 inline void set_physics(KParams& k, double tau, double kappa, double beta, double rho_l,
                         double rho_g, double rho_ref) {
-  k.omega = 1.0 / tau;
-  k.kforce = 1.0 - 1.0 / (2.0 * tau);
-  k.kappa = kappa;
-  k.two_beta = 2.0 * beta;
-  k.dl = rho_ref - rho_l;
-  k.dg = rho_ref - rho_g;
+  const double om = 1.0 / tau, kf = 1.0 - 1.0 / (2.0 * tau);
+  const double dl = rho_ref - rho_l, dg = rho_ref - rho_g;
   k.rho_ref = rho_ref;
-  k.f.set(k.omega, k.kforce, k.kappa, k.two_beta, k.dl, k.dg, k.rho_ref);
+  k.d.set(om, kf, kappa, 2.0 * beta, dl, dg, rho_ref);
+  k.f.set(om, kf, kappa, 2.0 * beta, dl, dg, rho_ref);
 }
 
-// The launch's constants in the arithmetic type (FP64: formed in the kernel,
-// no conversion is needed).
-__device__ __forceinline__ NodeConsts<float> consts_of(const KParams& p, float) { return p.f; }
-__device__ __forceinline__ NodeConsts<double> consts_of(const KParams& p, double) {
-  NodeConsts<double> q;
-  q.set(p.omega, p.kforce, p.kappa, p.two_beta, p.dl, p.dg, p.rho_ref);
-  return q;
-}
+__device__ __forceinline__ const NodeConsts<float>& consts_of(const KParams& p, float) { return p.f; }
+__device__ __forceinline__ const NodeConsts<double>& consts_of(const KParams& p, double) { return p.d; }
 
 // Outputs of the moments mode (any pointer may be null).
 struct MomentsOut {
@@ -174,27 +164,26 @@ __device__ __forceinline__ int wrap_index(int a, int n) {
 // stored densities rs (rho = rs + rho_ref):
 //   mu_0 = 2 beta (rho - rho_l)(rho - rho_g)(2 rho - rho_l - rho_g)
 //   lap  = [4 (E + W + N + S) + (NE + NW + SE + SW) - 20 C] / 6
-// kappa6 = kappa / 6.
-template <typename T>
-__device__ __forceinline__ T chem_pot(T c, T e, T w, T n, T s, T ne, T nw, T se,
-                                      T sw, T two_beta, T dl, T dg, T kappa6) {
-  T a = c + dl, b = c + dg;
-  T mu0 = two_beta * a * b * (a + b);
-  T lap6 = T(4) * ((e + w) + (n + s)) + ((ne + nw) + (se + sw)) - T(20) * c;
-  return mu0 - kappa6 * lap6;
+// kappa6 = kappa / 6.  chem_pot_rows takes the row sums ew = e + w,
+// nenw = ne + nw and sesw = se + sw (the strip kernel forms each row's sum
+// once and carries it to the two rows above): the same operations in the
+// same order.  In FP64 every rounding is named, so that all kernels give the
+// same bits whatever the compiler would contract in each of them (the FP32
+// form on pairs, chem_pot_x2, does so too).
+__device__ __forceinline__ double chem_pot_rows(double c, double ew, double n, double s,
+                                                double nenw, double sesw, double two_beta,
+                                                double dl, double dg, double kappa6) {
+  const double a = __dadd_rn(c, dl), b = __dadd_rn(c, dg);
+  const double mu0 = __dmul_rn(__dmul_rn(__dmul_rn(two_beta, a), b), __dadd_rn(a, b));
+  const double lap6 = __fma_rn(-20.0, c, __fma_rn(4.0, __dadd_rn(ew, __dadd_rn(n, s)),
+                                                  __dadd_rn(nenw, sesw)));
+  return __fma_rn(-kappa6, lap6, mu0);
 }
-
-// chem_pot with the row sums ew = e + w, nenw = ne + nw and sesw = se + sw
-// passed in (the FP64 strip kernel forms each row's sum once and carries it
-// to the two rows above): the same operations in the same order, so the
-// same result.
-template <typename T>
-__device__ __forceinline__ T chem_pot_rows(T c, T ew, T n, T s, T nenw, T sesw, T two_beta,
-                                           T dl, T dg, T kappa6) {
-  T a = c + dl, b = c + dg;
-  T mu0 = two_beta * a * b * (a + b);
-  T lap6 = T(4) * (ew + (n + s)) + (nenw + sesw) - T(20) * c;
-  return mu0 - kappa6 * lap6;
+__device__ __forceinline__ double chem_pot(double c, double e, double w, double n, double s,
+                                           double ne, double nw, double se, double sw,
+                                           double two_beta, double dl, double dg, double kappa6) {
+  return chem_pot_rows(c, __dadd_rn(e, w), n, s, __dadd_rn(ne, nw), __dadd_rn(se, sw), two_beta,
+                       dl, dg, kappa6);
 }
 
 // 1/x: the hardware reciprocal approximation in FP32 (about 1 ulp; the FP32
@@ -255,68 +244,89 @@ template <typename T>
 __device__ __forceinline__ void textbook_pairs(T (&g)[9], T rs, T rho, T ux, T uy, T Fx,
                                                T Fy, const NodeConsts<T>& q);
 
-// The well-balanced collision from 12 grad mu and 12 grad rho (iso_grad12),
-// the same terms as collide below arranged for fewer operations, which is
-// what bounds the FP64 path.  F = -rho grad mu enters the update only as F/2
-// (the velocity, Eq. rhoU) and as kforce F, so both are formed from the
-// gradient directly; G = F + cs^2 grad rho enters only as kforce G; and t,
-// k_u are carried divided by 36, so that the even parts are
-// E_dg = t' + 2 k_u', E_ax = 3 t' + E_dg and E_0 = 16 (t' - k_u') + omega b_0.
-template <typename T>
-__device__ __forceinline__ void collide_wb12(T (&g)[9], T rs, T gmx, T gmy, T grx, T gry,
-                                             const NodeConsts<T>& q, T& ux_out,
-                                             T& uy_out) {
-  constexpr bool kShifted = sizeof(T) == 4;
-  const T omega = q.omega;
-  const T rho = kShifted ? rs + q.rho_ref : rs;
-  const T hm = rho * T(-1.0 / 24.0);                   // F/2 = hm (12 grad mu)
-  const T kcm = rho * q.kfm12;                         // kforce F = kcm (12 grad mu)
-  const T d13 = g[1] - g[3], d24 = g[2] - g[4], d57 = g[5] - g[7], d86 = g[8] - g[6];
-  const T jx = (d13 + d57) + d86;
-  const T jy = (d24 + d57) - d86;
-  const T inv_rho = recip(rho);
-  const T ux = (jx + hm * gmx) * inv_rho;               // Eq. rhoU
-  const T uy = (jy + hm * gmy) * inv_rho;
+// The FP64 collision from 12 grad mu and 12 grad rho (iso_grad12): the terms
+// of collide below, arranged for the fewest FP64 operations, which is what
+// bounds every FP64 kernel here (GB300 issues two per SM and clock).  With
+//   A = (omega rho / 2) u + kforce G,  S = u.A,  X = ux Ay + uy Ax
+// (G = F + cs^2 grad rho well-balanced, G = F standard) the even parts need
+// neither u.u nor u.G: t = omega rho (-3/2 u.u) - 3 kforce u.G = -3 S, and with
+// B = 2 k_u / 36 = kforce (u.grad rho) / 18 (well-balanced, else 0)
+//   E_13 = ux Ax - S/3 + B,   E_24 = uy Ay - S/3 + B,
+//   E_57, E_68 = S/6 +- X/4 + B,   E_0 = omega b_0' - 4/3 S - 8 B,
+// b_0' = rho (well-balanced); the standard scheme adds w_i omega rho to each.
+// A, F and omega rho are carried divided by 3 (A3 = A/3, ..), so the odd
+// parts are M3 = (omega rho u + kforce F)/3 on the axes and (M3x +- M3y)/4 on
+// the diagonals, folded into the multiply-adds of the populations.  61
+// operations (well-balanced) where t, u.u, u.G and the parts one by one took
+// 77; the roundings are named so that every kernel gives the same bits.  Its
+// errors against 128-bit arithmetic are those of that form (populations
+// 0.8e-16 to 1.9e-16 relative, at u = 1e-2, 1e-4 and 1e-8 alike).
+// 4096^2 well-balanced step: 3.87 ms before, 3.44 ms.
+template <int SCH>
+__device__ __forceinline__ void collide12_f64(double (&g)[9], double rho, double gmx, double gmy,
+                                              double grx, double gry,
+                                              const NodeConsts<double>& q, double& ux_out,
+                                              double& uy_out) {
+  constexpr bool WB = SCH == kSchWB;
+  static_assert(WB || SCH == kSchStandard, "potential-form schemes");
+  const double d13 = __dadd_rn(g[1], -g[3]), d24 = __dadd_rn(g[2], -g[4]);
+  const double d57 = __dadd_rn(g[5], -g[7]), d86 = __dadd_rn(g[8], -g[6]);
+  const double jx = __dadd_rn(__dadd_rn(d13, d57), d86);
+  const double jy = __dadd_rn(__dadd_rn(d24, d57), -d86);
+  const double inv = recip(rho);
+  const double hm = __dmul_rn(rho, -1.0 / 24.0);         // F/2 = hm (12 grad mu) [+ cs^2 grad rho/2]
+  double sx = __fma_rn(hm, gmx, jx), sy = __fma_rn(hm, gmy, jy);
+  if (!WB) {
+    sx = __fma_rn(1.0 / 72.0, grx, sx);
+    sy = __fma_rn(1.0 / 72.0, gry, sy);
+  }
+  const double ux = __dmul_rn(sx, inv), uy = __dmul_rn(sy, inv);   // Eq. rhoU
   ux_out = ux;
   uy_out = uy;
-  const T kFx = kcm * gmx, kFy = kcm * gmy;
-  const T kGx = kFx + q.kf36 * grx, kGy = kFy + q.kf36 * gry;
-  const T orho = omega * rho;
-  const T uu = ux * ux + uy * uy;
-  const T uK = ux * kGx + uy * kGy;                     // kforce u.G
-  const T tq = (orho * T(-1.0 / 24.0)) * uu - T(1.0 / 12.0) * uK;   // t / 36
-  const T kq = q.kf432 * (ux * grx + uy * gry);         // k_u / 36
-  const T Cdg = tq + T(2) * kq;
-  const T Cax = T(3) * tq + Cdg;
-  const T E0 = T(16) * (tq - kq) + omega * rs;          // b_0 = rs, b_ax = b_dg = 0
-  const T hrho = T(0.5) * orho;
-  const T Mx = orho * ux + kFx;                         // odd parts: omega rho c.u + kforce c.F
-  const T My = orho * uy + kFy;
-  const T E1 = Cax + ux * (hrho * ux + kGx);            // pair (1,3): c = (1,0)
-  const T O1 = T(1.0 / 3.0) * Mx;
-  const T E2 = Cax + uy * (hrho * uy + kGy);            // pair (2,4): c = (0,1)
-  const T O2 = T(1.0 / 3.0) * My;
-  const T cu5 = ux + uy;                                // pair (5,7): c = (1,1)
-  const T E5 = Cdg + (T(0.25) * cu5) * (hrho * cu5 + (kGx + kGy));
-  const T O5 = T(1.0 / 12.0) * (Mx + My);
-  const T cu6 = uy - ux;                                // pair (6,8): c = (-1,1)
-  const T E6 = Cdg + (T(0.25) * cu6) * (hrho * cu6 + (kGy - kGx));
-  const T O6 = T(1.0 / 12.0) * (My - Mx);
-  const T keep = q.keep;
-  g[1] = keep * g[1] + (E1 + O1);
-  g[3] = keep * g[3] + (E1 - O1);
-  g[2] = keep * g[2] + (E2 + O2);
-  g[4] = keep * g[4] + (E2 - O2);
-  g[5] = keep * g[5] + (E5 + O5);
-  g[7] = keep * g[7] + (E5 - O5);
-  g[6] = keep * g[6] + (E6 + O6);
-  g[8] = keep * g[8] + (E6 - O6);
-  if (kShifted) {
-    (void)E0;                                           // mass balance, as in collide
-    g[0] = rs - (((g[1] + g[3]) + (g[2] + g[4])) + ((g[5] + g[7]) + (g[6] + g[8])));
+  const double kc = __dmul_rn(rho, q.kcm);               // kforce F / 3
+  double kFx, kFy, kGx, kGy;
+  if (WB) {
+    kFx = __dmul_rn(kc, gmx);
+    kFy = __dmul_rn(kc, gmy);
+    kGx = __fma_rn(q.kf108, grx, kFx);
+    kGy = __fma_rn(q.kf108, gry, kFy);
   } else {
-    g[0] = keep * g[0] + E0;
+    kFx = __fma_rn(kc, gmx, __dmul_rn(q.kf108, grx));
+    kFy = __fma_rn(kc, gmy, __dmul_rn(q.kf108, gry));
+    kGx = kFx;
+    kGy = kFy;
   }
+  // omega rho itself enters the rest population: keep + omega == 1 exactly,
+  // where keep + 3 (omega/3) would not be and the mass would drift
+  const double orho = __dmul_rn(q.omega, rho);
+  const double o3 = __dmul_rn(orho, 1.0 / 3.0), h3 = __dmul_rn(orho, 1.0 / 6.0);
+  const double Ax = __fma_rn(h3, ux, kGx), Ay = __fma_rn(h3, uy, kGy);
+  const double Mx = __fma_rn(o3, ux, kFx), My = __fma_rn(o3, uy, kFy);
+  const double Px = __dmul_rn(ux, Ax), Py = __dmul_rn(uy, Ay);
+  const double S = __dadd_rn(Px, Py);
+  const double X = __fma_rn(ux, Ay, __dmul_rn(uy, Ax));
+  const double keep = q.keep;
+  double Ca, Cd;
+  if (WB) {
+    Ca = __fma_rn(q.kf216, __fma_rn(ux, grx, __dmul_rn(uy, gry)), -S);
+    Cd = __fma_rn(1.5, S, Ca);
+    g[0] = __fma_rn(keep, g[0], __fma_rn(-8.0, Cd, orho));
+  } else {
+    Ca = __fma_rn(1.0 / 9.0, orho, -S);
+    Cd = __fma_rn(0.5, S, __dmul_rn(1.0 / 36.0, orho));
+    g[0] = __fma_rn(keep, g[0], __dmul_rn(4.0, Ca));
+  }
+  const double E1 = __fma_rn(3.0, Px, Ca), E2 = __fma_rn(3.0, Py, Ca);
+  const double E5 = __fma_rn(0.75, X, Cd), E6 = __fma_rn(-0.75, X, Cd);
+  const double T5 = __dadd_rn(Mx, My), T6 = __dadd_rn(My, -Mx);
+  g[1] = __fma_rn(keep, g[1], __dadd_rn(E1, Mx));
+  g[3] = __fma_rn(keep, g[3], __dadd_rn(E1, -Mx));
+  g[2] = __fma_rn(keep, g[2], __dadd_rn(E2, My));
+  g[4] = __fma_rn(keep, g[4], __dadd_rn(E2, -My));
+  g[5] = __fma_rn(keep, g[5], __fma_rn(0.25, T5, E5));
+  g[7] = __fma_rn(keep, g[7], __fma_rn(-0.25, T5, E5));
+  g[6] = __fma_rn(keep, g[6], __fma_rn(0.25, T6, E6));
+  g[8] = __fma_rn(keep, g[8], __fma_rn(-0.25, T6, E6));
 }
 
 // GS: the gradient inputs are GS times the gradients (12: the strip kernel
@@ -330,8 +340,8 @@ __device__ __forceinline__ void collide(T (&g)[9], T rs, T gmx, T gmy, T grx,
   constexpr bool kShifted = sizeof(T) == 4;   // FP32 storage is always shifted
   constexpr bool kG12 = GS == 12;
   static_assert(GS == 1 || GS == 12, "gradient scale");
-  if constexpr (WB && kG12) {
-    collide_wb12<T>(g, rs, gmx, gmy, grx, gry, q, ux_out, uy_out);
+  if constexpr (kG12 && sizeof(T) == 8 && (SCH == kSchWB || SCH == kSchStandard)) {
+    collide12_f64<SCH>(g, rs, gmx, gmy, grx, gry, q, ux_out, uy_out);
     return;
   }
   const T omega = q.omega, kf = q.kf;
@@ -494,23 +504,23 @@ __device__ __forceinline__ void iso_grad(T e, T w, T n, T s, T ne, T nw, T se, T
 
 // 12 times the same gradient, 4 (E - W) + (d1 + d2): two multiplications
 // fewer per gradient; collide<T, SCH, 12> folds the 1/12 into its uses.
-template <typename T>
-__device__ __forceinline__ void iso_grad12(T e, T w, T n, T s, T ne, T nw, T se, T sw,
-                                           T& gx, T& gy) {
-  const T d1 = ne - sw, d2 = se - nw;
-  gx = T(4) * (e - w) + (d1 + d2);
-  gy = T(4) * (n - s) + (d1 - d2);
+__device__ __forceinline__ void iso_grad12(double e, double w, double n, double s, double ne,
+                                           double nw, double se, double sw, double& gx,
+                                           double& gy) {
+  const double d1 = ne - sw, d2 = se - nw;
+  gx = __fma_rn(4.0, e - w, d1 + d2);
+  gy = __fma_rn(4.0, n - s, d1 - d2);
 }
 
 // iso_grad12 from per-row x-differences q = f(x+1) - f(x-1) and x-sums
 // p = f(x+1) + f(x-1) of the rows above (n), at (c) and below (s), which
 // the FP64 strip kernel forms once per row and carries:
 // 12 df/dx = 4 q_c + (q_n + q_s),  12 df/dy = 4 (n - s) + (p_n - p_s).
-template <typename T>
-__device__ __forceinline__ void iso_grad12_rows(T qc, T qn, T qs, T n, T s, T pn, T ps, T& gx,
-                                                T& gy) {
-  gx = T(4) * qc + (qn + qs);
-  gy = T(4) * (n - s) + (pn - ps);
+__device__ __forceinline__ void iso_grad12_rows(double qc, double qn, double qs, double n,
+                                                double s, double pn, double ps, double& gx,
+                                                double& gy) {
+  gx = __fma_rn(4.0, qc, qn + qs);
+  gy = __fma_rn(4.0, n - s, pn - ps);
 }
 
 // ---- packed FP32 pairs ------------------------------------------------------
@@ -1047,7 +1057,18 @@ __device__ __forceinline__ void strip_pass(const T* __restrict__ src, T* __restr
   // each side, rounded up to whole chunks; never past the stage row)
   const int nch_rt = GHOST ? (w + 2 * kPad + E - 1) / E : NCH;
 
-  const NodeConsts<T> cc = consts_of(p, T(0));
+  // FP64 constants by way of shared memory, so that they stay in registers:
+  // as constant-bank operands the 4096^2 standard step takes 3.46 ms, this
+  // way 3.40 (well-balanced 3.46 and 3.44)
+  __shared__ NodeConsts<double> s_cd;
+  if constexpr (!GHOST && sizeof(T) == 8) {
+    if (tx == 0) s_cd = p.d;
+    __syncthreads();
+  }
+  const NodeConsts<T> cc = [&]() -> NodeConsts<T> {
+    if constexpr (!GHOST && sizeof(T) == 8) return s_cd;
+    else return consts_of(p, T(0));
+  }();
   const T two_beta = cc.two_beta, dl = cc.dl, dg = cc.dg, kappa6 = cc.kappa6;
   // The second ring holds mu, or lap(rho) with the pressure-form force
   // (chem_pot with beta = 0 and kappa/6 -> -1/6 gives exactly lap(rho)); the
@@ -1307,21 +1328,21 @@ __device__ __forceinline__ void strip_pass(const T* __restrict__ src, T* __restr
               const T* rsb = rho_s + WB_SLOT(j - 2, kRing) * SW;  // row below (y-1)
               T* mrow = mu_s + WB_SLOT(j - 1, kMuRing) * SW;
               auto at = [&](int s) {
-                return chem_pot<T>(rc[s], rc[s + 1], rc[s - 1], rn[s], rsb[s], rn[s + 1],
+                return chem_pot(rc[s], rc[s + 1], rc[s - 1], rn[s], rsb[s], rn[s + 1],
                                    rn[s - 1], rsb[s + 1], rsb[s - 1], ring_tb, dl, dg, ring_k6);
               };
               if (own) {
-                mrow[sx] = chem_pot_rows<T>(rc[sx], psum_c, rn[sx], rsb[sx], psum_n, psum_b,
+                mrow[sx] = chem_pot_rows(rc[sx], psum_c, rn[sx], rsb[sx], psum_n, psum_b,
                                             ring_tb, dl, dg, ring_k6);
                 frs[j] = rc[sx];
                 // 12 grad(rho) (or 12 grad(cs^2 rho - p_0)): see iso_grad12
                 // and iso_grad12_rows
                 if (kPress)
-                  iso_grad12<T>(press_a(rc[sx + 1]), press_a(rc[sx - 1]), press_a(rn[sx]),
+                  iso_grad12(press_a(rc[sx + 1]), press_a(rc[sx - 1]), press_a(rn[sx]),
                                 press_a(rsb[sx]), press_a(rn[sx + 1]), press_a(rn[sx - 1]),
                                 press_a(rsb[sx + 1]), press_a(rsb[sx - 1]), fgx[j], fgy[j]);
                 else
-                  iso_grad12_rows<T>(pdif_c, pdif_n, pdif_b, rn[sx], rsb[sx], psum_n, psum_b,
+                  iso_grad12_rows(pdif_c, pdif_n, pdif_b, rn[sx], rsb[sx], psum_n, psum_b,
                                      fgx[j], fgy[j]);
               }
               if (tx == mu_lo) mrow[3] = at(3);
@@ -1397,7 +1418,7 @@ __device__ __forceinline__ void strip_pass(const T* __restrict__ src, T* __restr
               const T* m_up = mu_s + WB_SLOT(j - 1, kMuRing) * SW;
               // "up" is row c+1 (+y), "dn" row c-1; slot sx+1 is +x
               T gmx, gmy;                        // 12 grad(mu)
-              iso_grad12<T>(m_c[sx + 1], m_c[sx - 1], m_up[sx], m_dn[sx], m_up[sx + 1],
+              iso_grad12(m_c[sx + 1], m_c[sx - 1], m_up[sx], m_dn[sx], m_up[sx + 1],
                             m_up[sx - 1], m_dn[sx + 1], m_dn[sx - 1], gmx, gmy);
               const T rs = j == 0 ? prs : frs[j - 1];
               const T grx = j == 0 ? pgx : fgx[j - 1];

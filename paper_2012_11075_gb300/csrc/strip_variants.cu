@@ -63,16 +63,16 @@ __global__ void __launch_bounds__(kE6Threads)
     rho_t[k] = s;
   }
   __syncthreads();
-  const double two_beta = p.two_beta, dl = p.dl, dg = p.dg, kappa6 = p.kappa / 6.0;
+  const double two_beta = p.d.two_beta, dl = p.d.dl, dg = p.d.dg, kappa6 = p.d.kappa6;
   for (int k = tid; k < kMuH * kMuW; k += kE6Threads) {
     const int ly = k / kMuW, lx = k - ly * kMuW;
     const double* r = rho_t + (ly + 1) * kRhoW + lx + 1;
-    mu_t[k] = chem_pot<double>(r[0], r[1], r[-1], r[kRhoW], r[-kRhoW], r[kRhoW + 1],
+    mu_t[k] = chem_pot(r[0], r[1], r[-1], r[kRhoW], r[-kRhoW], r[kRhoW + 1],
                                r[kRhoW - 1], r[-kRhoW + 1], r[-kRhoW - 1], two_beta, dl, dg,
                                kappa6);
   }
   __syncthreads();
-  const NodeConsts<double> cc = consts_of(p, 0.0);
+  const NodeConsts<double>& cc = p.d;
   StatsAcc acc;
   const bool acc_on = MODE != kModeStep;
 #pragma unroll

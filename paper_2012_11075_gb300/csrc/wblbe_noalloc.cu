@@ -72,10 +72,10 @@ __global__ void __launch_bounds__(kTileX* kTileY)
     rho_s[ly][lx] = s;
   }
   __syncthreads();
-  const double two_beta = p.two_beta, dl = p.dl, dg = p.dg, kappa6 = p.kappa / 6.0;
+  const double two_beta = p.d.two_beta, dl = p.d.dl, dg = p.d.dg, kappa6 = p.d.kappa6;
   for (int q = t; q < (kTileY + 2) * (kTileX + 2); q += kTileX * kTileY) {
     const int ly = q / (kTileX + 2) + 1, lx = q % (kTileX + 2) + 1;
-    mu_s[ly - 1][lx - 1] = chem_pot<double>(
+    mu_s[ly - 1][lx - 1] = chem_pot(
         rho_s[ly][lx], rho_s[ly][lx + 1], rho_s[ly][lx - 1], rho_s[ly + 1][lx],
         rho_s[ly - 1][lx], rho_s[ly + 1][lx + 1], rho_s[ly + 1][lx - 1],
         rho_s[ly - 1][lx + 1], rho_s[ly - 1][lx - 1], two_beta, dl, dg, kappa6);
@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(kTileX* kTileY)
     for (int i = 0; i < 9; ++i) g[i] = f[i * plane + k];
     const double rs = rho_s[ry][rx];
     double ux, uy;
-    const NodeConsts<double> cc = consts_of(p, 0.0);
+    const NodeConsts<double>& cc = p.d;
     collide<double, WB ? kSchWB : kSchStandard>(g, rs, gmx, gmy, grx, gry, cc, ux, uy);
     const double mu = mu_s[my][mx];
     if (rho_out) rho_out[k] = rs;
