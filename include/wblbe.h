@@ -127,7 +127,9 @@ typedef struct {
 
 /* Launch shape of the fused step kernel: tile_x lattice columns per CTA
  * (32, 64, 128 or 256) and rows_per_cta rows marched by each CTA (>= 1).
- * Results do not depend on it. */
+ * Results do not depend on it.  Lattices of up to about two million nodes
+ * (standard and well-balanced schemes) run in a two-dimensional tile kernel
+ * of their own until wblbe_set_launch asks for a shape. */
 typedef struct {
   int32_t tile_x;
   int32_t rows_per_cta;

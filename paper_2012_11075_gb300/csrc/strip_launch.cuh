@@ -44,23 +44,43 @@ cudaError_t allow_smem_scheme() {
   return e;
 }
 
+// Launch configuration of a step kernel; chained: the kernel may be placed
+// while the stream's previous kernel ends (it waits for it in chain_wait).
+// Consecutive steps of a lattice: 2048^2 FP32 61.0 -> 58.4 us per step, 128^2
+// FP32 2.8 -> 2.2 us.
+struct ChainedLaunch {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr{};
+  ChainedLaunch(dim3 grid, int block, size_t smem, cudaStream_t s, bool chained) {
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = chained ? 1 : 0;
+  }
+  ChainedLaunch(const ChainedLaunch&) = delete;
+};
+
 template <typename T, int SCH, int MOM, int TX>
 cudaError_t launch_tx(const void* src, void* dst, const KParams& kp, const MomentsOut& mo,
-                      cudaStream_t s) {
+                      cudaStream_t s, bool chained) {
   dim3 grid((kp.nx + TX - 1) / TX, (kp.row_hi - kp.row_lo + kp.rows - 1) / kp.rows);
-  lbm_strip_kernel<T, SCH, MOM, TX><<<grid, TX, strip_smem<T>(TX), s>>>(
-      static_cast<const T*>(src), static_cast<T*>(dst), kp, mo);
-  return cudaGetLastError();
+  ChainedLaunch l(grid, TX, strip_smem<T>(TX), s, chained);
+  return cudaLaunchKernelEx(&l.cfg, lbm_strip_kernel<T, SCH, MOM, TX>,
+                            static_cast<const T*>(src), static_cast<T*>(dst), kp, mo);
 }
 
 template <typename T, int SCH, int MOM>
 cudaError_t launch_strip(const void* src, void* dst, const KParams& kp, const MomentsOut& mo,
-                         int tile, cudaStream_t s) {
+                         int tile, cudaStream_t s, bool chained) {
   switch (tile) {
-    case 32: return launch_tx<T, SCH, MOM, 32>(src, dst, kp, mo, s);
-    case 64: return launch_tx<T, SCH, MOM, 64>(src, dst, kp, mo, s);
-    case 128: return launch_tx<T, SCH, MOM, 128>(src, dst, kp, mo, s);
-    case 256: return launch_tx<T, SCH, MOM, 256>(src, dst, kp, mo, s);
+    case 32: return launch_tx<T, SCH, MOM, 32>(src, dst, kp, mo, s, chained);
+    case 64: return launch_tx<T, SCH, MOM, 64>(src, dst, kp, mo, s, chained);
+    case 128: return launch_tx<T, SCH, MOM, 128>(src, dst, kp, mo, s, chained);
+    case 256: return launch_tx<T, SCH, MOM, 256>(src, dst, kp, mo, s, chained);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -68,19 +88,22 @@ cudaError_t launch_strip(const void* src, void* dst, const KParams& kp, const Mo
 // mode: a StripMode (step, moments, step with statistics)
 template <typename T, int SCH>
 cudaError_t launch_mode(int mode, const void* src, void* dst, const KParams& kp,
-                        const MomentsOut& mo, int tile, cudaStream_t s) {
+                        const MomentsOut& mo, int tile, cudaStream_t s, bool chained) {
   switch (mode) {
-    case kModeStep: return launch_strip<T, SCH, kModeStep>(src, dst, kp, mo, tile, s);
-    case kModeMoments: return launch_strip<T, SCH, kModeMoments>(src, dst, kp, mo, tile, s);
-    case kModeStepStats: return launch_strip<T, SCH, kModeStepStats>(src, dst, kp, mo, tile, s);
+    case kModeStep: return launch_strip<T, SCH, kModeStep>(src, dst, kp, mo, tile, s, chained);
+    case kModeMoments:
+      return launch_strip<T, SCH, kModeMoments>(src, dst, kp, mo, tile, s, chained);
+    case kModeStepStats:
+      return launch_strip<T, SCH, kModeStepStats>(src, dst, kp, mo, tile, s, chained);
     default: return cudaErrorInvalidValue;
   }
 }
 template <int SCH>
 cudaError_t launch_scheme(bool fp64, int mode, const void* src, void* dst,
-                          const KParams& kp, const MomentsOut& mo, int tile, cudaStream_t s) {
-  return fp64 ? launch_mode<double, SCH>(mode, src, dst, kp, mo, tile, s)
-              : launch_mode<float, SCH>(mode, src, dst, kp, mo, tile, s);
+                          const KParams& kp, const MomentsOut& mo, int tile, cudaStream_t s,
+                          bool chained = false) {
+  return fp64 ? launch_mode<double, SCH>(mode, src, dst, kp, mo, tile, s, chained)
+              : launch_mode<float, SCH>(mode, src, dst, kp, mo, tile, s, chained);
 }
 
 // Resident CTAs per SM of the step kernel at this tile width.
@@ -117,6 +140,13 @@ constexpr int kSchE6 = 4;
 cudaError_t launch_e6(int mode, const void* src, void* dst, const KParams& kp,
                       const MomentsOut& mo, cudaStream_t s);
 int e6_partials(int nx, int ny);
+// Tile kernel of small and medium lattices, schemes 0 and 1 (tile.cu): whether
+// a lattice takes it, the per-CTA records its statistics modes write (0: it
+// does not take it), and the launch.
+bool tile_path(int sch, bool fp64, int nx, int ny);
+int tile_records(bool fp64, int nx, int ny);
+cudaError_t launch_tile(int sch, bool fp64, int mode, const void* src, void* dst,
+                        const KParams& kp, const MomentsOut& mo, cudaStream_t s, bool chained);
 // Strip-kernel launches for scheme codes 0-3 without instantiating the
 // kernel templates again (defined in wblbe.cu; used by slabs.cu).
 cudaError_t launch_strip_any(int sch, bool fp64, int mode, const void* src, void* dst,
@@ -126,5 +156,6 @@ cudaError_t allow_smem_strip_all();
 // Bounds-check counts of the other translation units (bounds-checked build).
 unsigned int variants_bounds_errors(bool reset);
 unsigned int batch_bounds_errors(bool reset);
+unsigned int tile_bounds_errors(bool reset);
 
 }  // namespace wblbe

@@ -1,0 +1,332 @@
+// The step of small and medium lattices: one CTA per two-dimensional tile.
+//
+// The strip kernel marches each CTA up its rows, which streams a large
+// lattice at the least traffic but takes a fixed chain of row iterations
+// (load, barrier, mu, barrier, collide) one after another: with only a few
+// CTAs that chain is the whole step.  Here a CTA takes a TW x TH tile at
+// once: every population its nodes and their density frame pull is requested
+// before the first is used, and the step is three phases with two barriers,
+//   1. rho over the tile and two nodes around it      (shared memory)
+//   2. mu over the tile and one node around it        (shared memory),
+//      rho and grad rho of the own nodes              (registers)
+//   3. grad mu, the collision and the stores,
+// at the price of evaluating the frame's densities and chemical potentials
+// again in every tile (0.56 to 1.5 times the tile's densities).  The chain of
+// phases, not the traffic, bounds it up to about 256^2.  us per step with the
+// strip kernel and here: FP64 4 x 256 48.9 and 5.1, 100^2 49.2 and 5.7, 256^2
+// 51.2 and 18.2; FP32 100^2 8.1 and 2.0, 256^2 7.5 and 2.8, 512^2 8.7 and 5.4,
+// 1023 x 771 19.9 and 12.0, 1024^2 18.3 and 14.3.  Each node goes through the same device functions in
+// the same order as in the strip kernel, so the result is the same bit for
+// bit.
+#include <cuda_runtime.h>
+
+#include "lbm_kernels.cuh"
+#include "strip_launch.cuh"
+
+namespace wblbe {
+
+namespace {
+
+// A thread owns PR nodes of one column (rows ty * PR ..); the TW * TH / PR
+// owners come first, and the other threads of the CTA (if any) start on the
+// frame, whose work would otherwise follow the owners' own.
+template <typename T, int SCH, int MODE, int TW, int TH, int PR, int NT>
+__global__ void __launch_bounds__(NT)
+    lbm_tile_kernel(const T* __restrict__ src, T* __restrict__ dst, const KParams p,
+                    const MomentsOut mo) {
+  static_assert(SCH == kSchStandard || SCH == kSchWB, "potential-form schemes");
+  static_assert(sizeof(T) == 8 || PR == 2, "FP32 threads own a pair of rows");
+  constexpr bool STATS = MODE != kModeStep;
+  constexpr int FW = TW + 4, FH = TH + 4;       // the density frame
+  constexpr int NO = TW * TH / PR;              // owner threads
+  static_assert(NT >= NO && NT % 32 == 0 && TH % PR == 0 && TH % 2 == 0, "tile shape");
+  __shared__ T rho_s[FH][FW], mu_s[FH][FW];     // [2 + row][2 + column] of the tile
+
+  const int tid = threadIdx.x;
+  const int x0 = blockIdx.x * TW, y0 = blockIdx.y * TH;
+  const int nx = p.nx, ny = p.ny;
+  const bool owner = tid < NO;
+  const int tx = tid % TW, r0 = (tid / TW) * PR;
+  const int first_halo = tid >= NO ? tid - NO : tid + NT - NO;
+
+  auto ld = [&](int i, unsigned off) {
+    return WB_IN(off, p.plane) ? (src + i * p.plane)[off] : T(0);
+  };
+  // f_i(x) = P_i(x - c_i) from the wrapped columns (west, own, east) and row
+  // offsets (below, own, above)
+  auto pull = [&](T(&g)[9], unsigned xw, unsigned xc, unsigned xe, unsigned rb, unsigned rc,
+                  unsigned ra) {
+    g[0] = ld(0, rc + xc);
+    g[1] = ld(1, rc + xw);
+    g[2] = ld(2, rb + xc);
+    g[3] = ld(3, rc + xe);
+    g[4] = ld(4, ra + xc);
+    g[5] = ld(5, rb + xw);
+    g[6] = ld(6, rb + xe);
+    g[7] = ld(7, ra + xe);
+    g[8] = ld(8, ra + xw);
+  };
+  auto rho_of = [](const T(&g)[9]) {
+    if constexpr (sizeof(T) == 4)
+      return g[0] + (((g[1] + g[3]) + (g[2] + g[4])) + ((g[5] + g[7]) + (g[6] + g[8])));
+    else
+      return ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
+  };
+
+  chain_wait();
+  // ---- phase 1: densities ----
+  T g[PR][9];
+  if (owner) {
+    const int xc = wrap_index(x0 + tx, nx);
+    const int xw = xc == 0 ? nx - 1 : xc - 1, xe = xc == nx - 1 ? 0 : xc + 1;
+    int yr = wrap_index(y0 + r0, ny);
+    unsigned rb = (unsigned)((yr == 0 ? ny - 1 : yr - 1) * p.pitch);
+    unsigned rc = (unsigned)(yr * p.pitch);
+#pragma unroll
+    for (int r = 0; r < PR; ++r) {
+      yr = yr == ny - 1 ? 0 : yr + 1;
+      const unsigned ra = (unsigned)(yr * p.pitch);
+      pull(g[r], xw, xc, xe, rb, rc, ra);
+      rb = rc;
+      rc = ra;
+    }
+  }
+  // the frame: two rows below, two above, then two columns on each side
+  constexpr int kRowHalo = 2 * FW, kHaloN = 4 * FW + 4 * TH;
+  for (int h = first_halo; h < kHaloN; h += NT) {
+    int fx, fy;
+    if (h < 2 * kRowHalo) {
+      fy = h / FW;
+      fx = h - fy * FW;
+      if (fy >= 2) fy += TH;
+    } else {
+      const int q = h - 2 * kRowHalo;
+      fy = 2 + (q >> 2);
+      fx = q & 3;
+      if (fx >= 2) fx += TW;
+    }
+    const int xc = wrap_index(x0 - 2 + fx, nx), yc = wrap_index(y0 - 2 + fy, ny);
+    T f[9];
+    pull(f, xc == 0 ? nx - 1 : xc - 1, xc, xc == nx - 1 ? 0 : xc + 1,
+         (unsigned)((yc == 0 ? ny - 1 : yc - 1) * p.pitch), (unsigned)(yc * p.pitch),
+         (unsigned)((yc == ny - 1 ? 0 : yc + 1) * p.pitch));
+    rho_s[fy][fx] = rho_of(f);
+  }
+  T rs[PR];
+  const int fx = 2 + tx, fy = 2 + r0;
+  if (owner) {
+#pragma unroll
+    for (int r = 0; r < PR; ++r) {
+      rs[r] = rho_of(g[r]);
+      rho_s[fy + r][fx] = rs[r];
+    }
+  }
+  __syncthreads();
+
+  // ---- phase 2: chemical potential; grad rho of the own nodes ----
+  const NodeConsts<T> cc = consts_of(p, T(0));
+  const T two_beta = cc.two_beta, dl = cc.dl, dg = cc.dg, kappa6 = cc.kappa6;
+  T mu[PR], grx[PR], gry[PR];
+  if constexpr (sizeof(T) == 4) {
+    const float2 tb2 = splat(two_beta), dl2 = splat(dl), dg2 = splat(dg), k62 = splat(kappa6);
+    auto V = [](T lo, T hi) { return make_float2(lo, hi); };
+    // mu at frame positions (ax, ay) and (bx, by), one per lane
+    auto mu2 = [&](int ax, int ay, int bx, int by) {
+      auto at = [&](int dx, int dy) { return V(rho_s[ay + dy][ax + dx], rho_s[by + dy][bx + dx]); };
+      return chem_pot_x2(at(0, 0), at(1, 0), at(-1, 0), at(0, 1), at(0, -1), at(1, 1), at(-1, 1),
+                         at(1, -1), at(-1, -1), tb2, dl2, dg2, k62);
+    };
+    if (owner) {
+      const float2 m = mu2(fx, fy, fx, fy + 1);
+      auto at = [&](int dx, int dy) { return V(rho_s[fy + dy][fx + dx], rho_s[fy + 1 + dy][fx + dx]); };
+      float2 gx2, gy2;
+      iso_grad_x2(at(1, 0), at(-1, 0), at(0, 1), at(0, -1), at(1, 1), at(-1, 1), at(1, -1),
+                  at(-1, -1), gx2, gy2);
+      mu_s[fy][fx] = mu[0] = m.x;
+      mu_s[fy + 1][fx] = mu[1] = m.y;
+      grx[0] = gx2.x;
+      grx[1] = gx2.y;
+      gry[0] = gy2.x;
+      gry[1] = gy2.y;
+    }
+    // ring: the rows below and above (one per lane), then the two sides
+    for (int h = first_halo; h < TW + 2 + TH; h += NT) {
+      const int ax = h < TW + 2 ? 1 + h : 1, ay = h < TW + 2 ? 1 : h - TW;
+      const int bx = h < TW + 2 ? 1 + h : TW + 2, by = h < TW + 2 ? TH + 2 : h - TW;
+      const float2 m = mu2(ax, ay, bx, by);
+      mu_s[ay][ax] = m.x;
+      mu_s[by][bx] = m.y;
+    }
+  } else {
+    if (owner) {
+      T c[PR + 2], ps[PR + 2], pd[PR + 2];
+#pragma unroll
+      for (int r = 0; r < PR + 2; ++r) {
+        const T* row = rho_s[fy + r - 1];
+        c[r] = row[fx];
+        ps[r] = row[fx + 1] + row[fx - 1];
+        pd[r] = row[fx + 1] - row[fx - 1];
+      }
+#pragma unroll
+      for (int r = 0; r < PR; ++r) {
+        mu[r] = chem_pot_rows(c[r + 1], ps[r + 1], c[r + 2], c[r], ps[r + 2], ps[r], two_beta,
+                                 dl, dg, kappa6);
+        iso_grad12_rows(pd[r + 1], pd[r + 2], pd[r], c[r + 2], c[r], ps[r + 2], ps[r], grx[r],
+                           gry[r]);
+        mu_s[fy + r][fx] = mu[r];
+      }
+    }
+    for (int h = first_halo; h < 2 * (TW + 2) + 2 * TH; h += NT) {
+      int hx, hy;
+      if (h < 2 * (TW + 2)) {
+        hx = 1 + (h >= TW + 2 ? h - (TW + 2) : h);
+        hy = h >= TW + 2 ? TH + 2 : 1;
+      } else {
+        const int q = h - 2 * (TW + 2);
+        hx = (q & 1) ? TW + 2 : 1;
+        hy = 2 + (q >> 1);
+      }
+      const T *rn = rho_s[hy + 1], *rc = rho_s[hy], *rb = rho_s[hy - 1];
+      mu_s[hy][hx] = chem_pot(rc[hx], rc[hx + 1], rc[hx - 1], rn[hx], rb[hx], rn[hx + 1],
+                                 rn[hx - 1], rb[hx + 1], rb[hx - 1], two_beta, dl, dg, kappa6);
+    }
+  }
+  __syncthreads();
+
+  // ---- phase 3: collision ----
+  StatsAcc acc;
+  const int x = x0 + tx, y = y0 + r0;
+  if (owner && x < nx && y < ny) {
+    if constexpr (sizeof(T) == 4) {
+      auto at = [&](int dx, int dy) {
+        return make_float2(mu_s[fy + dy][fx + dx], mu_s[fy + 1 + dy][fx + dx]);
+      };
+      float2 gmx, gmy, ux, uy;
+      iso_grad_x2(at(1, 0), at(-1, 0), at(0, 1), at(0, -1), at(1, 1), at(-1, 1), at(1, -1),
+                  at(-1, -1), gmx, gmy);
+      float2 g2[9];
+#pragma unroll
+      for (int i = 0; i < 9; ++i) g2[i] = make_float2(g[0][i], g[1][i]);
+      const uint32_t ht = step_key(p.step + (p.step_base ? *p.step_base : 0LL));
+      const float2 rnd = pair_uniforms((uint32_t)y * (uint32_t)nx + (uint32_t)x, ht);
+      collide_x2<SCH>(g2, make_float2(rs[0], rs[1]), gmx, gmy, make_float2(grx[0], grx[1]),
+                      make_float2(gry[0], gry[1]), cc, ux, uy, rnd);
+      const T gl[9] = {g2[0].x, g2[1].x, g2[2].x, g2[3].x, g2[4].x,
+                       g2[5].x, g2[6].x, g2[7].x, g2[8].x};
+      emit_node<T, MODE, false>(p, mo, dst, y, x, x, false, false, gl, rs[0], mu[0], ux.x, uy.x,
+                                acc, STATS);
+      if (y + 1 < ny) {
+        const T gh[9] = {g2[0].y, g2[1].y, g2[2].y, g2[3].y, g2[4].y,
+                         g2[5].y, g2[6].y, g2[7].y, g2[8].y};
+        emit_node<T, MODE, false>(p, mo, dst, y + 1, x, x, false, false, gh, rs[1], mu[1], ux.y,
+                                  uy.y, acc, STATS);
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < PR; ++r) {
+        if (y + r < ny) {
+          const T *mn = mu_s[fy + r + 1], *mc = mu_s[fy + r], *mb = mu_s[fy + r - 1];
+          T gmx, gmy, ux, uy;
+          iso_grad12(mc[fx + 1], mc[fx - 1], mn[fx], mb[fx], mn[fx + 1], mn[fx - 1],
+                        mb[fx + 1], mb[fx - 1], gmx, gmy);
+          collide<T, SCH, 12>(g[r], rs[r], gmx, gmy, grx[r], gry[r], cc, ux, uy);
+          emit_node<T, MODE, false>(p, mo, dst, y + r, x, x, false, false, g[r], rs[r], mu[r], ux,
+                                    uy, acc, STATS);
+        }
+      }
+    }
+  }
+  if (STATS && mo.partials)
+    write_stats_record<NT>(acc, mo.partials +
+                                    (size_t)(blockIdx.y * gridDim.x + blockIdx.x) * kStatRec);
+  chain_signal();
+}
+
+template <typename T, int SCH, int MODE, int TW, int TH, int PR, int NT>
+cudaError_t launch_shape(const void* src, void* dst, const KParams& kp, const MomentsOut& mo,
+                         cudaStream_t s, bool chained) {
+  ChainedLaunch l(dim3((kp.nx + TW - 1) / TW, (kp.ny + TH - 1) / TH), NT, 0, s, chained);
+  return cudaLaunchKernelEx(&l.cfg, lbm_tile_kernel<T, SCH, MODE, TW, TH, PR, NT>,
+                            static_cast<const T*>(src), static_cast<T*>(dst), kp, mo);
+}
+
+// Tile shapes, smallest first (TW x TH, nodes per thread, threads), and the
+// largest number of tiles each is chosen for; us per step, GB300:
+//   FP64   8 x 4, 1,  96  up to 380 tiles: the FP64 chain of one node sets the
+//                         time, so every node has its own lane and the frame
+//                         other warps (4 x 256: 5.1, 16 x 8 5.9; 100^2: 5.7
+//                         and 6.0; 128^2, 512 tiles: 6.5 and 6.0)
+//         16 x 8, 1, 256  up to one tile per SM (128^2: 6.0, 16 x 16 10.7)
+//         16 x 16, 2, 128 the rest: row sums shared by two rows (256^2: 18.2,
+//                         16 x 8 18.6; 512^2: 59.2 and 60.8, 32 x 16 66.9)
+//   FP32  16 x 8, 2, 192  up to three tiles per SM (128^2: 2.2, 32 x 16 2.7;
+//                         256^2, 512 tiles: both 2.8)
+//         32 x 16, 2, 256 the rest (512^2: 5.4, 16 x 8 6.3; 1024^2 14.3 and
+//                         20.7, 64 x 16 15.7, 32 x 32 15.8)
+struct Shape { int tw, th; long long max_tiles; };
+constexpr long long kSMs = 152, kAny = 1LL << 40;
+constexpr Shape kShapes64[] = {{8, 4, 380}, {16, 8, kSMs}, {16, 16, kAny}};
+constexpr Shape kShapes32[] = {{16, 8, 3 * kSMs}, {32, 16, kAny}};
+// Above these many nodes the strip kernel reads less and is faster: FP64
+// 1500^2 490 us per step here and 492 there, 2048^2 894 and 865; FP32 1500^2
+// 35.8 and 38.3, 2048^2 62.6 and 58.4.
+constexpr long long kMaxNodes64 = 2250000, kMaxNodes32 = 3000000;
+
+long long tiles_of(const Shape& s, int nx, int ny) {
+  return (long long)((nx + s.tw - 1) / s.tw) * ((ny + s.th - 1) / s.th);
+}
+int shape_of(bool fp64, int nx, int ny) {
+  const Shape* s = fp64 ? kShapes64 : kShapes32;
+  int k = 0;
+  while (tiles_of(s[k], nx, ny) > s[k].max_tiles) ++k;
+  return k;
+}
+
+template <int SCH, int MODE>
+cudaError_t launch_mode_tile(bool fp64, const void* src, void* dst, const KParams& kp,
+                             const MomentsOut& mo, cudaStream_t s, bool ch) {
+  const int k = shape_of(fp64, kp.nx, kp.ny);
+  if (fp64) {
+    switch (k) {
+      case 0: return launch_shape<double, SCH, MODE, 8, 4, 1, 96>(src, dst, kp, mo, s, ch);
+      case 1: return launch_shape<double, SCH, MODE, 16, 8, 1, 256>(src, dst, kp, mo, s, ch);
+      default: return launch_shape<double, SCH, MODE, 16, 16, 2, 128>(src, dst, kp, mo, s, ch);
+    }
+  }
+  if (k == 0) return launch_shape<float, SCH, MODE, 16, 8, 2, 192>(src, dst, kp, mo, s, ch);
+  return launch_shape<float, SCH, MODE, 32, 16, 2, 256>(src, dst, kp, mo, s, ch);
+}
+
+template <int SCH>
+cudaError_t launch_scheme_tile(bool fp64, int mode, const void* src, void* dst, const KParams& kp,
+                               const MomentsOut& mo, cudaStream_t s, bool ch) {
+  switch (mode) {
+    case kModeStep: return launch_mode_tile<SCH, kModeStep>(fp64, src, dst, kp, mo, s, ch);
+    case kModeMoments: return launch_mode_tile<SCH, kModeMoments>(fp64, src, dst, kp, mo, s, ch);
+    case kModeStepStats:
+      return launch_mode_tile<SCH, kModeStepStats>(fp64, src, dst, kp, mo, s, ch);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+}  // namespace
+
+bool tile_path(int sch, bool fp64, int nx, int ny) {
+  return (sch == kSchStandard || sch == kSchWB) &&
+         (long long)nx * ny <= (fp64 ? kMaxNodes64 : kMaxNodes32) && (ny + 3) / 4 <= 65535;
+}
+
+int tile_records(bool fp64, int nx, int ny) {
+  if (!tile_path(kSchWB, fp64, nx, ny)) return 0;
+  return (int)tiles_of((fp64 ? kShapes64 : kShapes32)[shape_of(fp64, nx, ny)], nx, ny);
+}
+
+cudaError_t launch_tile(int sch, bool fp64, int mode, const void* src, void* dst,
+                        const KParams& kp, const MomentsOut& mo, cudaStream_t s, bool chained) {
+  return sch == kSchWB ? launch_scheme_tile<kSchWB>(fp64, mode, src, dst, kp, mo, s, chained)
+                       : launch_scheme_tile<kSchStandard>(fp64, mode, src, dst, kp, mo, s, chained);
+}
+
+unsigned int tile_bounds_errors(bool reset) { return read_bounds_errors(reset); }
+
+}  // namespace wblbe

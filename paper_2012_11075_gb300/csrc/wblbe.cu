@@ -75,10 +75,12 @@ Layout make_layout(const wblbe_params* p) {
   L.pops_bytes = align_up((size_t)9 * (size_t)L.plane * L.elem);
   // per-CTA records: the moments pass (32-column strips at the narrowest,
   // kMomentsRows rows) and a step with statistics in any default launch
-  // shape (at least 32 columns and 8 rows per CTA)
   const int strips = (p->nx + 31) / 32;
   const int runs = (p->ny + 7) / 8;
+  // shape (at least 32 columns and 8 rows per CTA), or the tile kernel's
   L.max_partials = strips * runs;
+  const int tiles = tile_records(p->precision == WBLBE_FP64, p->nx, p->ny);
+  if (tiles > L.max_partials) L.max_partials = tiles;
   size_t off = 0;
   L.off_a = off; off += L.pops_bytes;
   L.off_b = off; off += L.pops_bytes;
@@ -106,6 +108,7 @@ struct wblbe_ctx {
   double* stats_dev;
   long long* step_dev;           // step of the first step of a graph replay
   wblbe_launch launch;
+  bool launch_set;               // the caller chose the strip kernel's shape
   int64_t steps;
   int64_t launches;
   double mass0;
@@ -244,16 +247,27 @@ wblbe_launch default_launch(const wblbe_params& p) {
   return l;
 }
 
-// mode: kModeStep, kModeMoments or kModeStepStats (see StripMode)
+// Does this handle's lattice take the tile kernel?  Moments do by the lattice
+// alone; steps unless the caller chose a launch shape, which is one of the
+// strip kernel.
+bool takes_tiles(const wblbe_ctx* h, int mode) {
+  return (mode == kModeMoments || !h->launch_set) &&
+         tile_path(h->p.scheme, h->p.precision == WBLBE_FP64, h->p.nx, h->p.ny);
+}
+
+// mode: kModeStep, kModeMoments or kModeStepStats (see StripMode); chained:
+// see ChainedLaunch
 cudaError_t launch_any(const wblbe_ctx* h, int mode, const void* src,
                        void* dst, const KParams& kp, const MomentsOut& mo,
-                       int tile, cudaStream_t s) {
+                       int tile, cudaStream_t s, bool chained = false) {
   const bool fp64 = h->p.precision == WBLBE_FP64;
+  if (takes_tiles(h, mode))
+    return launch_tile(h->p.scheme, fp64, mode, src, dst, kp, mo, s, chained);
   switch (h->p.scheme) {
     case WBLBE_STANDARD:
-      return launch_scheme<kSchStandard>(fp64, mode, src, dst, kp, mo, tile, s);
+      return launch_scheme<kSchStandard>(fp64, mode, src, dst, kp, mo, tile, s, chained);
     case WBLBE_WELL_BALANCED:
-      return launch_scheme<kSchWB>(fp64, mode, src, dst, kp, mo, tile, s);
+      return launch_scheme<kSchWB>(fp64, mode, src, dst, kp, mo, tile, s, chained);
     case WBLBE_STANDARD_E6:
       return launch_e6(mode, src, dst, kp, mo, s);
     default:
@@ -264,6 +278,8 @@ cudaError_t launch_any(const wblbe_ctx* h, int mode, const void* src,
 // Per-CTA statistics records a step launch writes in the step-with-statistics
 // mode (the E6 tile kernel uses fixed 32 x 16 tiles).
 long long step_records(const wblbe_ctx* h) {
+  if (takes_tiles(h, kModeStepStats))
+    return tile_records(h->p.precision == WBLBE_FP64, h->p.nx, h->p.ny);
   if (h->p.scheme == WBLBE_STANDARD_E6) return e6_partials(h->p.nx, h->p.ny);
   const long long tx = h->launch.tile_x, rows = h->launch.rows_per_cta;
   return ((h->p.nx + tx - 1) / tx) * ((h->p.ny + rows - 1) / rows);
@@ -282,7 +298,7 @@ cudaError_t issue_step(wblbe_ctx* h, int from, cudaStream_t s, int graph_k = -1)
   }
   MomentsOut mo{};
   return launch_any(h, kModeStep, h->buf[from], h->buf[1 - from], kp, mo,
-                    h->launch.tile_x, s);
+                    h->launch.tile_x, s, true);
 }
 
 __global__ void set_step_kernel(long long* dst, long long v) { *dst = v; }
@@ -321,7 +337,9 @@ wblbe_status run_moments(wblbe_ctx* h, double* rho, double* ux, double* uy,
   KParams kp = make_kparams(h, kMomentsRows);
   MomentsOut mo{rho, ux, uy, mu, h->partials};
   CU(h, launch_any(h, kModeMoments, h->buf[h->cur], nullptr, kp, mo, tile, h->stream));
-  const int n = h->p.scheme == WBLBE_STANDARD_E6
+  const int n = takes_tiles(h, kModeMoments)
+                    ? tile_records(h->p.precision == WBLBE_FP64, h->p.nx, h->p.ny)
+                : h->p.scheme == WBLBE_STANDARD_E6
                     ? e6_partials(h->p.nx, h->p.ny)
                     : ((h->p.nx + tile - 1) / tile) * ((h->p.ny + kMomentsRows - 1) / kMomentsRows);
   stats_finalize_kernel<<<1, 256, 0, h->stream>>>(h->partials, n,
@@ -496,6 +514,7 @@ wblbe_status wblbe_set_launch(wblbe_handle h, const wblbe_launch* launch) {
   if (!h) return fail(nullptr, WBLBE_EINVAL, "handle is NULL");
   if (!launch_valid(launch)) return fail(h, WBLBE_EINVAL, "tile_x must be 32/64/128/256 and rows_per_cta >= 1");
   h->launch = *launch;
+  h->launch_set = true;
   drop_graph(h);
   return WBLBE_OK;
 }
@@ -869,7 +888,11 @@ extern "C" unsigned int wblbe_debug_bounds_errors(int32_t reset) {
   const unsigned int a = read_bounds_errors(reset != 0);
   const unsigned int b = batch_bounds_errors(reset != 0);
   const unsigned int c = variants_bounds_errors(reset != 0);
-  if (a == 0xFFFFFFFFu || b == 0xFFFFFFFFu || c == 0xFFFFFFFFu) return 0xFFFFFFFFu;
-  if (a == 0xFFFFFFFEu || b == 0xFFFFFFFEu || c == 0xFFFFFFFEu) return 0xFFFFFFFEu;
-  return a + b + c;
+  const unsigned int d = tile_bounds_errors(reset != 0);
+  unsigned int sum = 0;
+  for (unsigned int v : {a, b, c, d}) {
+    if (v == 0xFFFFFFFFu || v == 0xFFFFFFFEu) return v;
+    sum += v;
+  }
+  return sum;
 }
