@@ -11,8 +11,9 @@
 // grad(phi) = 3 sum_i w_i c_i phi(x + c_i) and
 // lap(phi) = 6 sum_i w_i (phi(x + c_i) - phi(x)).
 //
-// One step is three kernels on the caller's stream (in FP64 the FP64 pipe is
-// the limit, not memory traffic; in FP32 the traffic is):
+// An FP32 step is one kernel (d3_step_f32).  An FP64 step, and the moments of
+// both, are three kernels on the caller's stream (the FP64 pipe is the limit,
+// not memory traffic):
 //   d3_density:   rho(x) = sum_i P_i(x - c_i)           (pull, Eq. rhoU)
 //   d3_chem_pot:  mu = mu_0(rho) - kappa lap(rho)        (Sec. II)
 //   d3_collide:   the pulled populations, grad rho and grad mu, the force,
@@ -33,6 +34,7 @@
 
 #include "../../include/wblbe.h"
 #include "lbm_kernels.cuh"
+#include "strip_launch.cuh"
 
 using namespace wblbe;
 
@@ -84,24 +86,11 @@ __device__ __forceinline__ T moving_sum3(const T (&g)[19]) {
   return ax + ((xy + xz) + yz);
 }
 
-// Single-node forms of the FP32 exact-mass rounding of the 2D kernel:
-// TwoSum (Knuth), a uniform draw in [0, 1) on a 2^-23 grid from the node key
-// k and the step key ht (MurmurHash3's finalizer), and the stochastic
-// rounding of h + e to h or its neighbour on the side of e with probability
-// |e| / gap.
-__device__ __forceinline__ void two_sum1(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  const float bv = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bv)), __fsub_rn(b, bv));
-}
+// A uniform draw in [0, 1) on a 2^-23 grid from the node key k and the step
+// key ht (MurmurHash3's finalizer), for the rounding of the 2D kernel.
 __device__ __forceinline__ float node_uniform(uint32_t k, uint32_t ht) {
   return __fsub_rn(__uint_as_float(0x3f800000u | (fmix32(k + ht) >> 9)), 1.0f);
 }
-__device__ __forceinline__ float round_stochastic1(float h, float e, float u) {
-  const float n = next_toward(h, e);
-  return fabsf(__fmul_rn(u, __fsub_rn(n, h))) < fabsf(e) ? n : h;
-}
-
 template <typename T>
 __device__ __forceinline__ NodeConsts<T> consts3(const P3& p) {
   if constexpr (sizeof(T) == 4) {
@@ -202,6 +191,18 @@ __global__ void __launch_bounds__(kBlock3) d3_chem_pot(const T* __restrict__ rho
   mu[at3(p, x, y, z)] = mu3(ax, ed, c, consts3<T>(p));
 }
 
+// 12 grad(phi) from v(dx, dy, dz) = phi(x + (dx, dy, dz)); see grad3x12.
+template <typename T, typename V>
+__device__ __forceinline__ void grad3_sums(const V& v, T& gx, T& gy, T& gz) {
+  const T axx = v(1, 0, 0) - v(-1, 0, 0), axy = v(0, 1, 0) - v(0, -1, 0),
+          axz = v(0, 0, 1) - v(0, 0, -1);
+  const T exy1 = v(1, 1, 0) - v(-1, -1, 0), exy2 = v(1, -1, 0) - v(-1, 1, 0);
+  const T exz1 = v(1, 0, 1) - v(-1, 0, -1), exz2 = v(1, 0, -1) - v(-1, 0, 1);
+  const T eyz1 = v(0, 1, 1) - v(0, -1, -1), eyz2 = v(0, 1, -1) - v(0, -1, 1);
+  gx = fma(T(2), axx, (exy1 + exy2) + (exz1 + exz2));
+  gy = fma(T(2), axy, (exy1 - exy2) + (eyz1 + eyz2));
+  gz = fma(T(2), axz, (exz1 - exz2) + (eyz1 - eyz2));
+}
 // 12 grad(phi) = 36 sum_i w_i c_i phi(x + c_i): 2 (axis differences) +
 // (edge differences); the factor 1/12 is folded into the constants that
 // use the gradients.
@@ -211,14 +212,7 @@ __device__ __forceinline__ void grad3x12(const T* __restrict__ phi, const P3& p,
   auto v = [&](int dx, int dy, int dz) {
     return __ldg(phi + at3(p, wrap3(x + dx, p.nx), wrap3(y + dy, p.ny), wrap3(z + dz, p.nz)));
   };
-  const T axx = v(1, 0, 0) - v(-1, 0, 0), axy = v(0, 1, 0) - v(0, -1, 0),
-          axz = v(0, 0, 1) - v(0, 0, -1);
-  const T exy1 = v(1, 1, 0) - v(-1, -1, 0), exy2 = v(1, -1, 0) - v(-1, 1, 0);
-  const T exz1 = v(1, 0, 1) - v(-1, 0, -1), exz2 = v(1, 0, -1) - v(-1, 0, 1);
-  const T eyz1 = v(0, 1, 1) - v(0, -1, -1), eyz2 = v(0, 1, -1) - v(0, -1, 1);
-  gx = fma(T(2), axx, (exy1 + exy2) + (exz1 + exz2));
-  gy = fma(T(2), axy, (exy1 - exy2) + (eyz1 + eyz2));
-  gz = fma(T(2), axz, (exz1 - exz2) + (eyz1 - eyz2));
+  grad3_sums<T>(v, gx, gy, gz);
 }
 
 // One component of F from 12 grad mu and 12 grad rho, nr = -rho / 12:
@@ -239,65 +233,132 @@ __device__ __forceinline__ float vel3(float j, float F, float inv) {
   return __fmul_rn(__fmaf_rn(0.5f, F, j), inv);
 }
 
-// a x + b y + c z, the first product of the innermost sum fused
-__device__ __forceinline__ float dot3(float ax, float bx, float ay, float by, float az, float bz) {
-  return __fmaf_rn(az, bz, __fmaf_rn(ax, bx, __fmul_rn(ay, by)));
+// Momentum from the differences of opposite pairs (each edge difference
+// serves two components).
+template <typename T>
+__device__ __forceinline__ void momentum3(const T (&g)[19], T& jx, T& jy, T& jz) {
+  const T d12 = g[1] - g[2], d34 = g[3] - g[4], d56 = g[5] - g[6];
+  const T d78 = g[7] - g[8], d910 = g[9] - g[10], d1112 = g[11] - g[12];
+  const T d1314 = g[13] - g[14], d1516 = g[15] - g[16], d1718 = g[17] - g[18];
+  jx = ((d12 + d78) + (d910 + d1112)) + d1314;
+  jy = ((d34 + d78) - (d910 - d1516)) + d1718;
+  jz = ((d56 + d1112) - (d1314 - d1516)) - d1718;
 }
 
-// The FP32 update of one node's populations (the terms of d3_collide below):
-// F the force, gr 12 grad rho, key the node's number and ht the step's key
-// (the draw of the rest population's rounding).
+// ---- FP32 on pairs of nodes -------------------------------------------------
+// (a pair's lanes are two nodes; every rounding is named, as in the scalar
+// functions above, whose operations these are in the same order)
+__device__ __forceinline__ float2 moving_sum3_x2(const float2 (&g)[19]) {
+  const float2 ax = add2(add2(add2(g[1], g[2]), add2(g[3], g[4])), add2(g[5], g[6]));
+  const float2 xy = add2(add2(g[7], g[8]), add2(g[9], g[10]));
+  const float2 xz = add2(add2(g[11], g[12]), add2(g[13], g[14]));
+  const float2 yz = add2(add2(g[15], g[16]), add2(g[17], g[18]));
+  return add2(ax, add2(add2(xy, xz), yz));
+}
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 mu3_x2(float2 ax, float2 ed, float2 c,
+                                         const NodeConsts<float>& q) {
+  const float2 lap = fma2(splat(1.0f / 3.0f), fma2(splat(-6.0f), c, ax),
+                          mul2(splat(1.0f / 6.0f), fma2(splat(-12.0f), c, ed)));
+  const float2 a = add2(c, splat(q.dl)), b = add2(c, splat(q.dg));
+  return fma2(mul2(mul2(splat(q.two_beta), a), b), add2(a, b), neg2(mul2(splat(q.kappa), lap)));
+}
+// 12 grad(phi) of rows y and y + 1 from three shared-memory planes (below, at,
+// above) at [y][x]
+template <int W>
+__device__ __forceinline__ void grad3_planes(const float (*b)[W], const float (*c)[W],
+                                             const float (*a)[W], int x, int y, float2& gx,
+                                             float2& gy, float2& gz) {
+  auto v = [&](int dx, int dy, int dz) {
+    const float(*r)[W] = dz < 0 ? b : (dz == 0 ? c : a);
+    return make_float2(r[y + dy][x + dx], r[y + 1 + dy][x + dx]);
+  };
+  const float2 axx = sub2(v(1, 0, 0), v(-1, 0, 0)), axy = sub2(v(0, 1, 0), v(0, -1, 0)),
+               axz = sub2(v(0, 0, 1), v(0, 0, -1));
+  const float2 exy1 = sub2(v(1, 1, 0), v(-1, -1, 0)), exy2 = sub2(v(1, -1, 0), v(-1, 1, 0));
+  const float2 exz1 = sub2(v(1, 0, 1), v(-1, 0, -1)), exz2 = sub2(v(1, 0, -1), v(-1, 0, 1));
+  const float2 eyz1 = sub2(v(0, 1, 1), v(0, -1, -1)), eyz2 = sub2(v(0, 1, -1), v(0, -1, 1));
+  gx = fma2(splat(2.0f), axx, add2(add2(exy1, exy2), add2(exz1, exz2)));
+  gy = fma2(splat(2.0f), axy, add2(sub2(exy1, exy2), add2(eyz1, eyz2)));
+  gz = fma2(splat(2.0f), axz, add2(sub2(exz1, exz2), sub2(eyz1, eyz2)));
+}
+// a x + b y + c z, the first product of the innermost sum fused
+__device__ __forceinline__ float2 dot3_x2(float2 ax, float2 bx, float2 ay, float2 by, float2 az,
+                                          float2 bz) {
+  return fma2(az, bz, fma2(ax, bx, mul2(ay, by)));
+}
+
+// The FP32 update of a pair of nodes (the terms of d3_collide below): rs the
+// stored densities, (mx, my, mz) 12 grad mu, (rx, ry, rz) 12 grad rho; key_a,
+// key_b the nodes' numbers and ht the step's key (the draws of the rest
+// populations' roundings).
 template <bool WB>
-__device__ __forceinline__ void update3_f32(float (&g)[19], float rs, float r, float Fx, float Fy,
-                                            float Fz, float grx, float gry, float grz, float ux,
-                                            float uy, float uz, const NodeConsts<float>& q,
-                                            uint32_t key, uint32_t ht) {
-  const float om = q.omega, kf = q.kf, keep = q.keep, c36 = 1.0f / 36.0f;
-  const float m_in = moving_sum3(g);
-  const float Gx = WB ? __fmaf_rn(c36, grx, Fx) : Fx;     // F + cs^2 grad rho
-  const float Gy = WB ? __fmaf_rn(c36, gry, Fy) : Fy;
-  const float Gz = WB ? __fmaf_rn(c36, grz, Fz) : Fz;
-  const float orho = __fmul_rn(om, r);
-  const float t = __fmaf_rn(__fmul_rn(-1.5f, orho), dot3(ux, ux, uy, uy, uz, uz),
-                            -__fmul_rn(__fmul_rn(3.0f, kf), dot3(ux, Gx, uy, Gy, uz, Gz)));
-  float Ca, Ce;
+__device__ __forceinline__ void update3_x2(float2 (&g)[19], float2 rs, float2 mx, float2 my,
+                                           float2 mz, float2 rx, float2 ry, float2 rz,
+                                           const NodeConsts<float>& q, uint32_t key_a,
+                                           uint32_t key_b, uint32_t ht) {
+  const float2 om = splat(q.omega), keep = splat(q.keep), c36 = splat(1.0f / 36.0f);
+  const float2 r = add2(rs, splat(q.rho_ref));
+  const float2 nr = mul2(r, splat(-1.0f / 12.0f));
+  auto force = [&](float2 gm, float2 gr) {
+    return WB ? mul2(nr, gm) : fma2(nr, gm, mul2(c36, gr));
+  };
+  const float2 Fx = force(mx, rx), Fy = force(my, ry), Fz = force(mz, rz);
+  const float2 d12 = sub2(g[1], g[2]), d34 = sub2(g[3], g[4]), d56 = sub2(g[5], g[6]);
+  const float2 d78 = sub2(g[7], g[8]), d910 = sub2(g[9], g[10]), d1112 = sub2(g[11], g[12]);
+  const float2 d1314 = sub2(g[13], g[14]), d1516 = sub2(g[15], g[16]), d1718 = sub2(g[17], g[18]);
+  const float2 jx = add2(add2(add2(d12, d78), add2(d910, d1112)), d1314);
+  const float2 jy = add2(sub2(add2(d34, d78), sub2(d910, d1516)), d1718);
+  const float2 jz = sub2(sub2(add2(d56, d1112), sub2(d1314, d1516)), d1718);
+  const float2 inv = make_float2(recip(r.x), recip(r.y)), half = splat(0.5f);
+  const float2 ux = mul2(fma2(half, Fx, jx), inv), uy = mul2(fma2(half, Fy, jy), inv),
+               uz = mul2(fma2(half, Fz, jz), inv);
+  const float2 m_in = WB ? moving_sum3_x2(g) : make_float2(0.f, 0.f);
+  const float2 Gx = WB ? fma2(c36, rx, Fx) : Fx;          // F + cs^2 grad rho
+  const float2 Gy = WB ? fma2(c36, ry, Fy) : Fy;
+  const float2 Gz = WB ? fma2(c36, rz, Fz) : Fz;
+  const float2 orho = mul2(om, r);
+  const float2 t = fma2(mul2(splat(-1.5f), orho), dot3_x2(ux, ux, uy, uy, uz, uz),
+                        neg2(mul2(splat(__fmul_rn(3.0f, q.kf)), dot3_x2(ux, Gx, uy, Gy, uz, Gz))));
+  float2 Ca, Ce;
   if (WB) {
-    const float ku = __fmul_rn(__fmul_rn(kf, 1.0f / 12.0f), dot3(ux, grx, uy, gry, uz, grz));
-    Ca = __fmul_rn(1.0f / 18.0f, t);
-    Ce = __fmul_rn(c36, __fmaf_rn(1.5f, ku, t));
+    const float2 ku = mul2(splat(__fmul_rn(q.kf, 1.0f / 12.0f)), dot3_x2(ux, rx, uy, ry, uz, rz));
+    Ca = mul2(splat(1.0f / 18.0f), t);
+    Ce = mul2(c36, fma2(splat(1.5f), ku, t));
   } else {
-    const float b = __fmaf_rn(om, rs, t);
-    Ca = __fmul_rn(1.0f / 18.0f, b);
-    Ce = __fmul_rn(c36, b);
+    const float2 b = fma2(om, rs, t);
+    Ca = mul2(splat(1.0f / 18.0f), b);
+    Ce = mul2(c36, b);
   }
-  const float Aa = __fmul_rn(0.25f, orho), Ae = __fmul_rn(0.125f, orho);
-  const float kh = __fmul_rn(0.5f, kf), kq = __fmul_rn(0.25f, kf), k6 = __fmul_rn(kf, 1.0f / 6.0f);
-  const float o6 = __fmul_rn(orho, 1.0f / 6.0f);
-  const float Mx = __fmaf_rn(k6, Fx, __fmul_rn(o6, ux));
-  const float My = __fmaf_rn(k6, Fy, __fmul_rn(o6, uy));
-  const float Mz = __fmaf_rn(k6, Fz, __fmul_rn(o6, uz));
-  const float Key = __fmul_rn(kq, Gy), Kez = __fmul_rn(kq, Gz);
-  auto axis = [&](int i, int j, float cu, float G, float M) {
-    const float E = __fmaf_rn(cu, __fmaf_rn(kh, G, __fmul_rn(Aa, cu)), Ca);
-    g[i] = __fmaf_rn(keep, g[i], __fadd_rn(E, M));
-    g[j] = __fmaf_rn(keep, g[j], __fsub_rn(E, M));
+  const float2 Aa = mul2(splat(0.25f), orho), Ae = mul2(splat(0.125f), orho);
+  const float2 kh = splat(__fmul_rn(0.5f, q.kf)), kq = splat(__fmul_rn(0.25f, q.kf));
+  const float2 k6 = splat(__fmul_rn(q.kf, 1.0f / 6.0f));
+  const float2 o6 = mul2(orho, splat(1.0f / 6.0f));
+  const float2 Mx = fma2(k6, Fx, mul2(o6, ux));
+  const float2 My = fma2(k6, Fy, mul2(o6, uy));
+  const float2 Mz = fma2(k6, Fz, mul2(o6, uz));
+  const float2 Key = mul2(kq, Gy), Kez = mul2(kq, Gz);
+  auto axis = [&](int i, int j, float2 cu, float2 G, float2 M) {
+    const float2 E = fma2(cu, fma2(kh, G, mul2(Aa, cu)), Ca);
+    g[i] = fma2(keep, g[i], add2(E, M));
+    g[j] = fma2(keep, g[j], sub2(E, M));
     return E;
   };
-  auto edge = [&](int i, int j, float cu, float K, float S) {
-    const float E = __fmaf_rn(cu, __fmaf_rn(Ae, cu, K), Ce);
-    g[i] = __fmaf_rn(keep, g[i], __fmaf_rn(0.5f, S, E));
-    g[j] = __fmaf_rn(keep, g[j], __fmaf_rn(-0.5f, S, E));
+  auto edge = [&](int i, int j, float2 cu, float2 K, float2 S) {
+    const float2 E = fma2(cu, fma2(Ae, cu, K), Ce);
+    g[i] = fma2(keep, g[i], fma2(half, S, E));
+    g[j] = fma2(keep, g[j], fma2(splat(-0.5f), S, E));
     return E;
   };
-  const float Ea1 = axis(1, 2, ux, Gx, Mx);
-  const float Ea2 = axis(3, 4, uy, Gy, My);
-  const float Ea3 = axis(5, 6, uz, Gz, Mz);
-  const float Ee1 = edge(7, 8, __fadd_rn(ux, uy), __fmaf_rn(kq, Gx, Key), __fadd_rn(Mx, My));
-  const float Ee2 = edge(9, 10, __fsub_rn(ux, uy), __fmaf_rn(kq, Gx, -Key), __fsub_rn(Mx, My));
-  const float Ee3 = edge(11, 12, __fadd_rn(ux, uz), __fmaf_rn(kq, Gx, Kez), __fadd_rn(Mx, Mz));
-  const float Ee4 = edge(13, 14, __fsub_rn(ux, uz), __fmaf_rn(kq, Gx, -Kez), __fsub_rn(Mx, Mz));
-  const float Ee5 = edge(15, 16, __fadd_rn(uy, uz), __fadd_rn(Key, Kez), __fadd_rn(My, Mz));
-  const float Ee6 = edge(17, 18, __fsub_rn(uy, uz), __fsub_rn(Key, Kez), __fsub_rn(My, Mz));
+  const float2 Ea1 = axis(1, 2, ux, Gx, Mx);
+  const float2 Ea2 = axis(3, 4, uy, Gy, My);
+  const float2 Ea3 = axis(5, 6, uz, Gz, Mz);
+  const float2 Ee1 = edge(7, 8, add2(ux, uy), fma2(kq, Gx, Key), add2(Mx, My));
+  const float2 Ee2 = edge(9, 10, sub2(ux, uy), fma2(kq, Gx, neg2(Key)), sub2(Mx, My));
+  const float2 Ee3 = edge(11, 12, add2(ux, uz), fma2(kq, Gx, Kez), add2(Mx, Mz));
+  const float2 Ee4 = edge(13, 14, sub2(ux, uz), fma2(kq, Gx, neg2(Kez)), sub2(Mx, Mz));
+  const float2 Ee5 = edge(15, 16, add2(uy, uz), add2(Key, Kez), add2(My, Mz));
+  const float2 Ee6 = edge(17, 18, sub2(uy, uz), sub2(Key, Kez), sub2(My, Mz));
   if (WB) {
     // The collision conserves the node's mass, so the rest population
     // follows from the balance: g_0' = g_0 + omega m_in - 2 sum E (the
@@ -305,12 +366,14 @@ __device__ __forceinline__ void update3_f32(float (&g)[19], float rs, float r, f
     // part would be lost in rounding g_0 ~ rho - rho_ref to float; TwoSum
     // keeps the remainder and a zero-mean rounding, seeded by the node and
     // the step, takes it into account.
-    const float sE = ((Ea1 + Ea2) + Ea3) + (((Ee1 + Ee2) + (Ee3 + Ee4)) + (Ee5 + Ee6));
-    float hsum, err;
-    two_sum1(g[0], __fmaf_rn(-2.0f, sE, __fmul_rn(om, m_in)), hsum, err);
-    g[0] = round_stochastic1(hsum, err, node_uniform(key, ht));
+    const float2 sE = add2(add2(add2(Ea1, Ea2), Ea3),
+                           add2(add2(add2(Ee1, Ee2), add2(Ee3, Ee4)), add2(Ee5, Ee6)));
+    float2 hsum, err;
+    two_sum2(g[0], fma2(splat(-2.0f), sE, mul2(om, m_in)), hsum, err);
+    g[0] = round_stochastic2(hsum, err,
+                             make_float2(node_uniform(key_a, ht), node_uniform(key_b, ht)));
   } else {
-    g[0] = __fsub_rn(rs, moving_sum3(g));      // the standard scheme: the mass balance
+    g[0] = sub2(rs, moving_sum3_x2(g));        // the standard scheme: the mass balance
   }
 }
 
@@ -351,18 +414,12 @@ __global__ void __launch_bounds__(kBlock3) d3_collide(const T* __restrict__ src,
     const T nr = r * T(-1.0 / 12.0);
     const T Fx = force3<WB>(nr, gmx, grx), Fy = force3<WB>(nr, gmy, gry),
             Fz = force3<WB>(nr, gmz, grz);
-    // momentum from the differences of opposite pairs (each edge difference
-    // serves two components)
-    const T d12 = g[1] - g[2], d34 = g[3] - g[4], d56 = g[5] - g[6];
-    const T d78 = g[7] - g[8], d910 = g[9] - g[10], d1112 = g[11] - g[12];
-    const T d1314 = g[13] - g[14], d1516 = g[15] - g[16], d1718 = g[17] - g[18];
-    const T jx = ((d12 + d78) + (d910 + d1112)) + d1314;
-    const T jy = ((d34 + d78) - (d910 - d1516)) + d1718;
-    const T jz = ((d56 + d1112) - (d1314 - d1516)) - d1718;
+    T jx, jy, jz;
+    momentum3(g, jx, jy, jz);
     const T inv = recip(r);
     const T ux = vel3(jx, Fx, inv), uy = vel3(jy, Fy, inv), uz = vel3(jz, Fz, inv);  // Eq. rhoU
     const T muc = mu[k];
-    if (MOMENTS) {
+    if constexpr (MOMENTS) {
       const double rd = kShifted ? (double)rs + p.rho_ref : (double)r;
       const double uxd = ux, uyd = uy, uzd = uz, mud = muc;
       if (out.rho) out.rho[(size_t)(z * p.ny + y) * p.nx + x] = rd;
@@ -379,11 +436,8 @@ __global__ void __launch_bounds__(kBlock3) d3_collide(const T* __restrict__ src,
       st[5] = (!isfinite(rd) || !isfinite(mud) || !isfinite(u2)) ? 1.0 : 0.0;
     } else {
       const NodeConsts<T> q = consts3<T>(p);
-      if constexpr (kShifted) {
-        const uint32_t key = (uint32_t)(((long long)z * p.ny + y) * p.nx + x);
-        update3_f32<WB>(g, rs, r, Fx, Fy, Fz, grx, gry, grz, ux, uy, uz, q, key,
-                        step_key(p.step));
-      } else {
+      static_assert(MOMENTS || !kShifted, "FP32 steps run in d3_step_f32");
+      {
         const T om = q.omega, kf = q.kf, keep = q.keep;
         T Gx = Fx, Gy = Fy, Gz = Fz;
         if (WB) {
@@ -477,6 +531,179 @@ __global__ void __launch_bounds__(kBlock3) d3_collide(const T* __restrict__ src,
       for (int q = 0; q < kStatRec; ++q) o[q] = r[q];
     }
   }
+}
+
+// The whole FP32 step in one kernel: a CTA owns TX x TY columns and marches a
+// run of planes along z; a thread owns two rows of a column, whose arithmetic
+// runs on packed pairs.  Per plane, with the front plane f:
+//   A. rho of plane f over the tile and two columns around it (the nineteen
+//      pulled populations of each node), into a ring of planes;
+//   B. mu of plane f - 1 over the tile and one column around it, into a second
+//      ring; rho and grad rho of the own nodes stay in registers;
+//   C. grad mu, the collision and the stores of plane f - 2.
+// The three kernels read the populations twice from DRAM and write and read
+// two fields, 248 bytes per update for 152 algorithmic ones; here the second
+// read of the own populations (requested before B's arithmetic) and the frame
+// come from L2.  The latency of the pulls bounds it (11 warps per SM; DRAM 46 %,
+// issue 40 % busy).  us per step in three kernels and here: 256^3 985 and 708,
+// 128^3 130 and 97, 101 x 67 x 75 42 and 37, 64^3 27 and 20.  Measured and not kept, 256^3:
+// one node per thread 782; all pulls of an iteration requested at once 844;
+// populations staged by 4-byte asynchronous copies 1178; plane addresses from
+// the constant bank 775; four resident CTAs 714, 32 x 16 tiles 728.
+constexpr int kTX3 = 32, kTY3 = 8, kNT3 = kTX3 * kTY3 / 2;
+constexpr int kMinB3 = 3;          // resident CTAs (164 registers)
+
+template <bool WB>
+__global__ void __launch_bounds__(kNT3, kMinB3)
+    d3_step_f32(const float* __restrict__ src, float* __restrict__ dst, const P3 p, int run) {
+  constexpr int TX = kTX3, TY = kTY3;
+  constexpr int FW = TX + 4, FH = TY + 4, MW = TX + 2, MH = TY + 2;
+  __shared__ float rho_s[4][FH][FW];           // [f & 3][2 + y][2 + x]
+  __shared__ float mu_s[4][MH][MW];            // [f & 3][1 + y][1 + x]
+  const int tid = threadIdx.x, tx = tid % TX, ty = 2 * (tid / TX);
+  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+  const int z0 = blockIdx.z * run, z1 = min(z0 + run, p.nz);
+  chain_wait();
+
+  // element offsets of a column's west, own and east elements and of four
+  // rows: below the pair, the pair, above it
+  struct Col { unsigned x[3], y[4]; };
+  auto column = [&](int x, int y) {
+    Col c;
+    const int xc = wrap_index(x, p.nx);
+    c.x[0] = (unsigned)(xc == 0 ? p.nx - 1 : xc - 1);
+    c.x[1] = (unsigned)xc;
+    c.x[2] = (unsigned)(xc == p.nx - 1 ? 0 : xc + 1);
+    int yr = wrap_index(y - 1, p.ny);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      c.y[k] = (unsigned)p.pitch * (unsigned)yr;
+      yr = yr == p.ny - 1 ? 0 : yr + 1;
+    }
+    return c;
+  };
+  const Col own = column(x0 + tx, y0 + ty);
+  // the frame in pairs of rows: the two rows below, the two above, and two
+  // columns on each side
+  constexpr int kFrame = 2 * FW + 2 * TY;
+  const bool has_frame = tid < kFrame;
+  static_assert(kFrame <= kNT3, "one pair of the frame per thread");
+  int hx, hy;
+  if (tid < 2 * FW) {
+    hx = tid < FW ? tid : tid - FW;
+    hy = tid < FW ? 0 : TY + 2;
+  } else {
+    const int k = tid - 2 * FW;
+    hx = (k & 3) < 2 ? (k & 3) : TX + (k & 3);
+    hy = 2 + 2 * (k >> 2);
+  }
+  const Col frame = column(x0 - 2 + hx, y0 - 2 + hy);
+  // mu's ring: the rows below and above (one per lane), then the two sides
+  constexpr int kRing = MW + TY;
+  static_assert(kRing <= kNT3, "one pair of the ring per thread");
+  const bool has_ring = tid < kRing;
+  const bool rows = tid < MW;
+  const int rax = rows ? tid : 0, ray = rows ? 0 : 1 + tid - MW;
+  const int rbx = rows ? tid : MW - 1, rby = rows ? MH - 1 : 1 + tid - MW;
+
+  // g_i(x) = P_i(x - c_i) of a pair of rows; z: offsets of the planes below,
+  // at and above
+  auto pull = [&](float2(&g)[19], const Col& c, unsigned zb, unsigned zc, unsigned za) {
+#pragma unroll
+    for (int i = 0; i < kQ3; ++i) {
+      const unsigned xz = (cz3(i) == 1 ? zb : (cz3(i) == 0 ? zc : za)) + c.x[1 - cx3(i)];
+      const float* pl = src + i * p.plane;
+      g[i] = make_float2(pl[xz + c.y[1 - cy3(i)]], pl[xz + c.y[2 - cy3(i)]]);
+    }
+  };
+  const unsigned layer = (unsigned)p.pitch * (unsigned)p.ny;
+  auto zoff = [&](int z) { return layer * (unsigned)wrap_index(z, p.nz); };
+  int f = z0 - 2;
+  // planes f - 3 .. f + 1
+  unsigned zm3 = 0, zm2 = 0, zm1 = zoff(f - 1), zc = zoff(f), zp = zoff(f + 1);
+  int znext = wrap_index(f + 1, p.nz);
+
+  const NodeConsts<float> q = p.f;
+  const uint32_t ht = step_key(p.step);
+  const bool mine_a = x0 + tx < p.nx && y0 + ty < p.ny, mine_b = mine_a && y0 + ty + 1 < p.ny;
+  const float2 zero = make_float2(0.f, 0.f);
+  float2 prs = zero, pgx = zero, pgy = zero, pgz = zero;   // rho - rho_ref, 12 grad rho of f - 2
+  for (; f < z1 + 2; ++f) {
+    const int c = f - 2;                        // the plane to collide
+    const bool upd = mine_a && c >= z0;
+    {
+      float2 a[19];
+      pull(a, own, zm1, zc, zp);
+      const float2 r = add2(a[0], moving_sum3_x2(a));
+      rho_s[f & 3][2 + ty][2 + tx] = r.x;
+      rho_s[f & 3][3 + ty][2 + tx] = r.y;
+      if (has_frame) {
+        pull(a, frame, zm1, zc, zp);
+        const float2 v = add2(a[0], moving_sum3_x2(a));
+        rho_s[f & 3][hy][hx] = v.x;
+        rho_s[f & 3][hy + 1][hx] = v.y;
+      }
+    }
+    __syncthreads();
+    float2 g[19];
+    if (upd) pull(g, own, zm3, zm2, zm1);
+    float2 rs = zero, gx = zero, gy = zero, gz = zero;
+    if (f >= z0) {
+      const float(*rb)[FW] = rho_s[(f + 2) & 3], (*rc)[FW] = rho_s[(f + 3) & 3],
+                 (*ra)[FW] = rho_s[f & 3];
+      // mu at two nodes of the frame, from the neighbours' sums in the
+      // direction order of d3_chem_pot
+      auto mu_at = [&](int ax, int ay, int bx, int by) {
+        auto v = [&](int dx, int dy, int dz) {
+          const float(*r)[FW] = dz < 0 ? rb : (dz == 0 ? rc : ra);
+          return make_float2(r[ay + dy][ax + dx], r[by + dy][bx + dx]);
+        };
+        float2 sa = v(1, 0, 0), se = v(1, 1, 0);
+#pragma unroll
+        for (int i = 2; i < 7; ++i) sa = add2(sa, v(cx3(i), cy3(i), cz3(i)));
+#pragma unroll
+        for (int i = 8; i < kQ3; ++i) se = add2(se, v(cx3(i), cy3(i), cz3(i)));
+        return mu3_x2(sa, se, v(0, 0, 0), q);
+      };
+      const int x = 2 + tx, y = 2 + ty;
+      const float2 m = mu_at(x, y, x, y + 1);
+      mu_s[(f + 3) & 3][1 + ty][1 + tx] = m.x;
+      mu_s[(f + 3) & 3][2 + ty][1 + tx] = m.y;
+      rs = make_float2(rc[y][x], rc[y + 1][x]);
+      grad3_planes(rb, rc, ra, x, y, gx, gy, gz);
+      if (has_ring) {
+        const float2 h = mu_at(rax + 1, ray + 1, rbx + 1, rby + 1);
+        mu_s[(f + 3) & 3][ray][rax] = h.x;
+        mu_s[(f + 3) & 3][rby][rbx] = h.y;
+      }
+    }
+    __syncthreads();
+    if (upd) {
+      float2 mx, my, mz;
+      grad3_planes(mu_s[(f + 1) & 3], mu_s[(f + 2) & 3], mu_s[(f + 3) & 3], 1 + tx, 1 + ty, mx, my,
+                   mz);
+      const uint32_t key = (uint32_t)(((long long)c * p.ny + y0 + ty) * p.nx + x0 + tx);
+      update3_x2<WB>(g, prs, mx, my, mz, pgx, pgy, pgz, q, key, key + (uint32_t)p.nx, ht);
+      float* da = dst + (zm2 + own.x[1] + own.y[1]);
+      float* db = dst + (zm2 + own.x[1] + own.y[2]);
+#pragma unroll
+      for (int i = 0; i < kQ3; ++i) {
+        da[i * p.plane] = g[i].x;
+        if (mine_b) db[i * p.plane] = g[i].y;
+      }
+    }
+    prs = rs;
+    pgx = gx;
+    pgy = gy;
+    pgz = gz;
+    zm3 = zm2;
+    zm2 = zm1;
+    zm1 = zc;
+    zc = zp;
+    znext = znext == p.nz - 1 ? 0 : znext + 1;
+    zp = layer * (unsigned)znext;
+  }
+  chain_signal();
 }
 
 // f = f^eq(rho, 0) stored for the pull: P_i(x) = f_i^eq(rho(x + c_i)) - s_i.
@@ -640,14 +867,51 @@ void pass3_typed(wblbe3_ctx* h, bool moments, const Out3& out, const P3& q, dim3
   if (moments) {
     if (wb) d3_collide<T, true, true><<<g, kBlock3, 0, h->stream>>>(src, nullptr, rho, mu, q, out);
     else d3_collide<T, false, true><<<g, kBlock3, 0, h->stream>>>(src, nullptr, rho, mu, q, out);
-  } else {
+  } else if constexpr (sizeof(T) == 8) {
     if (wb) d3_collide<T, true, false><<<g, kBlock3, 0, h->stream>>>(src, dst, rho, mu, q, out);
     else d3_collide<T, false, false><<<g, kBlock3, 0, h->stream>>>(src, dst, rho, mu, q, out);
   }
 }
 
+// Planes per CTA of the fused FP32 step: the run whose waves of resident CTAs
+// take the fewest plane iterations in all (a run of n planes takes n + 4, of
+// which the first four store nothing).
+int fused_run(const wblbe3_ctx* h) {
+  const long long tiles = (long long)((h->p.nx + kTX3 - 1) / kTX3) * ((h->p.ny + kTY3 - 1) / kTY3);
+  const long long resident = 152LL * kMinB3;
+  int best = h->p.nz;
+  long long cost = -1;
+  for (int segs = 1; segs <= h->p.nz && segs <= 65535; ++segs) {
+    const int run = (h->p.nz + segs - 1) / segs;
+    const long long n = tiles * ((h->p.nz + run - 1) / run);
+    const long long c = (n + resident - 1) / resident * (run + 4);
+    if (cost < 0 || c < cost) {
+      cost = c;
+      best = run;
+    }
+  }
+  return best;
+}
+
+cudaError_t fused_step(wblbe3_ctx* h, const P3& q) {
+  const int run = fused_run(h);
+  ChainedLaunch l(dim3((h->p.nx + kTX3 - 1) / kTX3, (h->p.ny + kTY3 - 1) / kTY3,
+                       (h->p.nz + run - 1) / run),
+                  kNT3, 0, h->stream, true);
+  const float* src = static_cast<const float*>(h->buf[h->cur]);
+  float* dst = static_cast<float*>(h->buf[1 - h->cur]);
+  return h->p.scheme == WBLBE_WELL_BALANCED
+             ? cudaLaunchKernelEx(&l.cfg, d3_step_f32<true>, src, dst, q, run)
+             : cudaLaunchKernelEx(&l.cfg, d3_step_f32<false>, src, dst, q, run);
+}
+
 wblbe_status pass3(wblbe3_ctx* h, bool moments, const Out3& out) {
   const P3 q = p3_of(h);
+  if (!moments && h->p.precision == WBLBE_FP32_SHIFTED) {
+    CU3(h, fused_step(h, q));
+    h->launches += 1;
+    return WBLBE_OK;
+  }
   const dim3 g = grid3(h);
   if (h->p.precision == WBLBE_FP64)
     pass3_typed<double>(h, moments, out, q, g);

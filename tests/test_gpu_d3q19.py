@@ -240,3 +240,26 @@ def test_d3q19_fp32_droplet_follows_fp64():
     assert abs(j32 - j64) < 1e-3
     assert abs(s32["mass_drift_rel"]) < 1e-6
     assert abs(s32["umax"] - s64["umax"]) < 0.05 * s64["umax"]
+
+
+@pytest.mark.parametrize("scheme", [wblbe.STANDARD, wblbe.WELL_BALANCED])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (2, 3, 5), (9, 8, 32), (3, 9, 33), (40, 7, 31),
+                                   (5, 17, 65)])
+def test_d3q19_fp32_one_kernel_step_at_tile_edges(shape, scheme):
+    """The one-kernel FP32 step (32 x 8 columns, pairs of rows, runs of
+    planes) at lattices smaller than its frame and one node around its tile:
+    5 steps against FP64.  Populations are O(1), so the float storage and
+    arithmetic of 5 steps stay within 40 ulps of 1 (2^-24 each)."""
+    nz, ny, nx = shape
+    rng = np.random.default_rng(nx * 100 + ny * 10 + nz)
+    rho = 0.6 + 0.1 * rng.uniform(-1, 1, shape)
+    out = []
+    for precision in (wblbe.FP64, wblbe.FP32_SHIFTED):
+        s = wblbe.Solver3(wblbe.Params3(nx, ny, nz, 0.9, 0.01, 0.005, 1.0, 0.2, scheme=scheme,
+                                        precision=precision))
+        s.init_rho(rho)
+        s.step(5)
+        out.append((s.get_populations(), s.stats()["mass"]))
+        s.close()
+    assert np.max(np.abs(out[0][0] - out[1][0])) < 40 * 2.0 ** -24
+    assert abs(out[0][1] - out[1][1]) < 40 * 2.0 ** -24 * nx * ny * nz
