@@ -261,7 +261,9 @@ typedef struct wblbe_batch* wblbe_batch_handle;
 
 typedef struct {
   int32_t tile_x;            /* 32, 64, 128 or 256                         */
-  int32_t rows_per_tile;     /* >= 4; rows are split into near-equal runs  */
+  int32_t rows_per_tile;     /* >= 4; rows are split into near-equal runs,
+                              * shorter ones where the running cases' tiles
+                              * would not occupy the device               */
   int32_t steps_per_launch;  /* >= 1 lattice steps per persistent launch   */
 } wblbe_batch_config;
 

@@ -440,6 +440,8 @@ LayoutParams case_layout(const wblbe_batch::Case& c) {
   return lp;
 }
 
+int resident_ctas(const wblbe_batch* b);
+
 // Does the periodic interval [a - h, b + h) (mod n) meet [c, d) (0 <= c < d <= n)?
 bool periodic_meet(int a, int b, int c, int d, int h, int n) {
   const int len = (b - a) + 2 * h;
@@ -450,59 +452,84 @@ bool periodic_meet(int a, int b, int c, int d, int h, int n) {
 }
 
 // Tiles of a case: strips of tile_x columns (x0 a multiple of tile_x) and
-// near-equal runs of about rows_per_tile rows.
-void case_tiles(const wblbe_batch::Case& c, int case_idx, const wblbe_batch_config& cfg,
-                std::vector<TileDev>& out) {
-  const int nx = c.p.nx, ny = c.p.ny;
-  const int nseg = std::max(1, ny / std::max(cfg.rows_per_tile, 4));
-  // run boundaries on even rows (the FP32 stochastic rounding draws one hash
-  // per pair of rows 2j, 2j + 1; see pair_uniforms)
-  auto bound = [&](int s) { return s >= nseg ? ny : (int)((long long)s * ny / nseg) & ~1; };
-  for (int s = 0; s < nseg; ++s) {
-    const int y0 = bound(s), y1 = bound(s + 1);
-    for (int x0 = 0; x0 < nx; x0 += cfg.tile_x) {
-      TileDev t{};
-      t.c = case_idx;
-      t.x0 = x0;
-      t.y0 = y0;
-      t.y1 = y1;
-      for (int q = 0; q < kMaxNb; ++q) t.nb[q] = -1;
-      out.push_back(t);
-    }
-  }
+// near-equal runs of about `rows` rows.
+int run_count(const wblbe_batch::Case& c, int rows) { return std::max(1, c.p.ny / std::max(rows, 4)); }
+long long tile_count(const wblbe_batch::Case& c, int tile_x, int rows) {
+  return (long long)run_count(c, rows) * ((c.p.nx + tile_x - 1) / tile_x);
 }
 
-// Cut a case into tiles for the current configuration and find, for every
-// tile, the tiles of the same case its halo reads (local indices).  Cached
-// until the configuration changes.
-wblbe_status ensure_case_tiles(wblbe_batch* b, wblbe_batch::Case& c) {
-  if (c.tiles_tx == b->cfg.tile_x && c.tiles_rows == b->cfg.rows_per_tile && !c.tiles.empty())
-    return WBLBE_OK;
+// Cut a case into tiles of at most tile_x columns by about `rows` rows and
+// find, for every tile, the tiles of the same case its halo reads (local
+// indices): the product of the runs its rows meet and the strips its columns
+// meet.  Cached until the cut changes.
+wblbe_status ensure_case_tiles(wblbe_batch* b, wblbe_batch::Case& c, int rows) {
+  const int tile_x = b->cfg.tile_x;
+  if (c.tiles_tx == tile_x && c.tiles_rows == rows && !c.tiles.empty()) return WBLBE_OK;
   c.tiles.clear();
-  case_tiles(c, 0, b->cfg, c.tiles);
-  const int nt = (int)c.tiles.size();
-  for (int a = 0; a < nt; ++a) {
-    TileDev& ta = c.tiles[a];
-    const int wa = std::min(b->cfg.tile_x, c.p.nx - ta.x0);
-    int n = 0;
-    for (int q = 0; q < nt; ++q) {
-      if (q == a) continue;
-      const TileDev& tq = c.tiles[q];
-      const int wq = std::min(b->cfg.tile_x, c.p.nx - tq.x0);
-      if (periodic_meet(ta.x0, ta.x0 + wa, tq.x0, tq.x0 + wq, kHaloReach, c.p.nx) &&
-          periodic_meet(ta.y0, ta.y1, tq.y0, tq.y1, kHaloReach, c.p.ny)) {
-        if (n == kMaxNb) {
-          c.tiles.clear();
-          return bfail(b, WBLBE_EINVAL, "a tile of case %lld has more than %d neighbours; "
-                       "use larger tiles", (long long)c.id, kMaxNb);
+  c.tiles_tx = c.tiles_rows = 0;
+  const int nx = c.p.nx, ny = c.p.ny;
+  const int nrun = run_count(c, rows), nstrip = (nx + tile_x - 1) / tile_x;
+  // run boundaries on even rows (the FP32 stochastic rounding draws one hash
+  // per pair of rows 2j, 2j + 1; see pair_uniforms)
+  auto ybound = [&](int s) { return s >= nrun ? ny : (int)((long long)s * ny / nrun) & ~1; };
+  auto xbound = [&](int s) { return std::min(nx, s * tile_x); };
+  // indices of the parts whose interval the halo of part a reaches
+  auto meets = [](int n, int a, int len, auto bound, std::vector<int>& out) {
+    out.clear();
+    for (int q = 0; q < n; ++q)
+      if (periodic_meet(bound(a), bound(a + 1), bound(q), bound(q + 1), kHaloReach, len))
+        out.push_back(q);
+  };
+  std::vector<std::vector<int>> cols(nstrip);
+  for (int x = 0; x < nstrip; ++x) meets(nstrip, x, nx, xbound, cols[x]);
+  std::vector<int> runs;
+  for (int s = 0; s < nrun; ++s) {
+    meets(nrun, s, ny, ybound, runs);
+    for (int x = 0; x < nstrip; ++x) {
+      TileDev t{};
+      t.x0 = xbound(x);
+      t.y0 = ybound(s);
+      t.y1 = ybound(s + 1);
+      for (int q = 0; q < kMaxNb; ++q) t.nb[q] = -1;
+      int n = 0;
+      for (int rs : runs)
+        for (int cs : cols[x]) {
+          if (rs == s && cs == x) continue;
+          if (n == kMaxNb) {
+            c.tiles.clear();
+            return bfail(b, WBLBE_EINVAL, "a tile of case %lld has more than %d neighbours; "
+                         "use larger tiles", (long long)c.id, kMaxNb);
+          }
+          t.nb[n++] = rs * nstrip + cs;
         }
-        ta.nb[n++] = q;
-      }
+      c.tiles.push_back(t);
     }
   }
-  c.tiles_tx = b->cfg.tile_x;
-  c.tiles_rows = b->cfg.rows_per_tile;
+  c.tiles_tx = tile_x;
+  c.tiles_rows = rows;
   return WBLBE_OK;
+}
+
+// Rows per tile for the running cases: the configured ones, halved (down to
+// 8) while that leaves fewer than two tiles per resident CTA and the tile
+// table holds the finer cut.  With less than that, CTAs idle while the
+// longest tile of each step marches its rows: a tile's row takes about 0.7 us
+// whatever runs beside it.  us per step of 64-step launches, 128-column
+// tiles, rows 128 / 64 / 32 / 16 / 8: 32 cases of 64-300 columns (50 to 979
+// tiles) 141 / 73 / 37 / 23 / 18; 128 cases of 64-512 (432 to 7480) 188 / 121
+// / 107 / 118 / 139; 400 (1292 to 22771) 303 / 297 / 316 / 352 / 417.
+// Results do not depend on the cut.
+int effective_rows(const wblbe_batch* b) {
+  auto total = [&](int rows) {
+    long long n = 0;
+    for (const auto& c : b->cases)
+      if (c.used && c.running) n += tile_count(c, b->cfg.tile_x, rows);
+    return n;
+  };
+  const long long want = 2LL * resident_ctas(b);
+  int rows = b->cfg.rows_per_tile;
+  while (rows >= 16 && total(rows) < want && total(rows / 2) <= b->max_tiles) rows /= 2;
+  return rows;
 }
 
 wblbe_status upload_case_entry(wblbe_batch* b, int ci) {
@@ -522,10 +549,11 @@ wblbe_status upload_case_entry(wblbe_batch* b, int ci) {
 wblbe_status rebuild_tiles(wblbe_batch* b) {
   std::vector<TileDev> tiles;
   b->run_host.clear();
+  const int rows = effective_rows(b);
   for (size_t ci = 0; ci < b->cases.size(); ++ci) {
     auto& c = b->cases[ci];
     if (!c.used || !c.running) continue;
-    wblbe_status st = ensure_case_tiles(b, c);
+    wblbe_status st = ensure_case_tiles(b, c, rows);
     if (st != WBLBE_OK) return st;
     RunCase rc{};
     rc.c = (int)ci;
@@ -602,6 +630,15 @@ int batch_grid(int tile) {
   }
 }
 
+// CTAs of the persistent kernel at the batch's tile width that are resident
+// at once (also its grid).
+int resident_ctas(const wblbe_batch* b) {
+  const bool wb = b->scheme == WBLBE_WELL_BALANCED;
+  const int tx = b->cfg.tile_x;
+  return b->precision == WBLBE_FP64 ? (wb ? batch_grid<double, true>(tx) : batch_grid<double, false>(tx))
+                                    : (wb ? batch_grid<float, true>(tx) : batch_grid<float, false>(tx));
+}
+
 template <typename T, bool WB>
 cudaError_t batch_launch(const BatchDev& d, int tile, int grid, cudaStream_t s) {
   switch (tile) {
@@ -653,10 +690,7 @@ void drop_batch_graph(wblbe_batch* b) {
 wblbe_status build_batch_graph(wblbe_batch* b) {
   drop_batch_graph(b);
   // attributes and occupancy queries outside the capture
-  const bool wb = b->scheme == WBLBE_WELL_BALANCED;
-  const int grid = b->precision == WBLBE_FP64
-                       ? (wb ? batch_grid<double, true>(b->cfg.tile_x) : batch_grid<double, false>(b->cfg.tile_x))
-                       : (wb ? batch_grid<float, true>(b->cfg.tile_x) : batch_grid<float, false>(b->cfg.tile_x));
+  const int grid = resident_ctas(b);
   BCU(b, cudaGetLastError());
   cudaGraph_t g = nullptr;
   BCU(b, cudaStreamBeginCapture(b->capture_stream, cudaStreamCaptureModeThreadLocal));
@@ -899,22 +933,18 @@ wblbe_status wblbe_batch_admit(wblbe_batch_handle b, const wblbe_params* params,
   for (int i = 0; i < b->max_cases; ++i)
     if (!b->cases[i].used) { slot = i; break; }
   if (slot < 0) return bfail(b, WBLBE_ENOMEM, "no free case slot (%d in use)", b->max_cases);
-  // tiles this case adds (running cases' tile lists are cached per config)
+  // tiles this case adds
   wblbe_batch::Case& c = b->cases[slot];
   c = wblbe_batch::Case();
   c.p = *params;
   c.id = b->next_id;
   {
-    wblbe_status st = ensure_case_tiles(b, c);
+    const int rows = b->cfg.rows_per_tile;
+    wblbe_status st = ensure_case_tiles(b, c, rows);
     if (st != WBLBE_OK) { c = wblbe_batch::Case(); return st; }
-    long long ntiles = (long long)c.tiles.size();
-    for (size_t ci = 0; ci < b->cases.size(); ++ci) {
-      auto& o = b->cases[ci];
-      if ((int)ci == slot || !o.used || !o.running) continue;
-      st = ensure_case_tiles(b, o);
-      if (st != WBLBE_OK) { c = wblbe_batch::Case(); return st; }
-      ntiles += (long long)o.tiles.size();
-    }
+    long long ntiles = 0;
+    for (const auto& o : b->cases)
+      if (&o == &c || (o.used && o.running)) ntiles += tile_count(o, b->cfg.tile_x, rows);
     if (ntiles > b->max_tiles) {
       c = wblbe_batch::Case();
       return bfail(b, WBLBE_ENOMEM, "tile table full (%lld > %d)", ntiles, b->max_tiles);
@@ -1115,7 +1145,7 @@ wblbe_status wblbe_batch_counts(wblbe_batch_handle b, int32_t* resident, int32_t
     ++res;
     if (c.running) {
       ++run;
-      if (ensure_case_tiles(b, c) == WBLBE_OK) nt += (int)c.tiles.size();
+      nt += (int)tile_count(c, b->cfg.tile_x, b->cfg.rows_per_tile);
     }
   }
   size_t fr = 0;
