@@ -66,10 +66,10 @@ __host__ __device__ constexpr double w3(int i) {
 struct P3 {
   int nx, ny, nz, pitch;
   long long plane;                 // elements per population plane / field
-  double omega, kforce, kappa, two_beta;
-  // storage shift density (0 in FP64) and rho_ref - rho_l, rho_ref - rho_g
-  double rho_ref, dl, dg;
-  NodeConsts<float> f;             // the FP32 constants, converted on the host
+  double rho_ref;                  // storage shift density, 0 in FP64
+  NodeConsts<double> d;            // the update's constants in both types
+  NodeConsts<float> f;
+  double kc72, kf288;              // -kforce/72, kforce/288 (update3_f64)
   long long step;                  // the step being taken (FP32 rounding draws)
 };
 
@@ -91,22 +91,8 @@ __device__ __forceinline__ T moving_sum3(const T (&g)[19]) {
 __device__ __forceinline__ float node_uniform(uint32_t k, uint32_t ht) {
   return __fsub_rn(__uint_as_float(0x3f800000u | (fmix32(k + ht) >> 9)), 1.0f);
 }
-template <typename T>
-__device__ __forceinline__ NodeConsts<T> consts3(const P3& p) {
-  if constexpr (sizeof(T) == 4) {
-    return p.f;
-  } else {
-    NodeConsts<double> q{};
-    q.omega = p.omega;
-    q.keep = 1.0 - p.omega;
-    q.kf = p.kforce;
-    q.kappa = p.kappa;
-    q.two_beta = p.two_beta;
-    q.dl = p.dl;
-    q.dg = p.dg;
-    return q;
-  }
-}
+__device__ __forceinline__ const NodeConsts<float>& consts3(const P3& p, float) { return p.f; }
+__device__ __forceinline__ const NodeConsts<double>& consts3(const P3& p, double) { return p.d; }
 
 struct Out3 {
   double* rho;                     // [nz][ny][nx] fields (may be null)
@@ -123,6 +109,27 @@ __device__ __forceinline__ long long at3(const P3& p, int x, int y, int z) {
   return ((long long)z * p.ny + y) * p.pitch + x;
 }
 
+// Element offsets of a node's wrapped neighbour columns, rows and planes
+// (below, own, above): 32 bits, a plane has fewer than 2^32 elements.
+struct Nbr3 {
+  unsigned x[3], y[3], z[3];
+  __device__ __forceinline__ Nbr3(const P3& p, int xx, int yy, int zz) {
+    const unsigned row = (unsigned)p.pitch, layer = row * (unsigned)p.ny;
+    x[0] = (unsigned)(xx == 0 ? p.nx - 1 : xx - 1);
+    x[1] = (unsigned)xx;
+    x[2] = (unsigned)(xx == p.nx - 1 ? 0 : xx + 1);
+    y[0] = row * (unsigned)(yy == 0 ? p.ny - 1 : yy - 1);
+    y[1] = row * (unsigned)yy;
+    y[2] = row * (unsigned)(yy == p.ny - 1 ? 0 : yy + 1);
+    z[0] = layer * (unsigned)(zz == 0 ? p.nz - 1 : zz - 1);
+    z[1] = layer * (unsigned)zz;
+    z[2] = layer * (unsigned)(zz == p.nz - 1 ? 0 : zz + 1);
+  }
+  __device__ __forceinline__ unsigned at(int dx, int dy, int dz) const {
+    return x[1 + dx] + y[1 + dy] + z[1 + dz];
+  }
+};
+
 // rho = sum_i f_i with f_i(x) = P_i(x - c_i): in FP64 summed from i = 0 to
 // 18; in FP32 the stored deviation rs = rho - rho_ref = g_0 + the
 // mirror-symmetric moving sum (the collision repeats that sum for the exact
@@ -132,21 +139,19 @@ __global__ void __launch_bounds__(kBlock3) d3_density(const T* __restrict__ src,
                                                       T* __restrict__ rho, const P3 p) {
   const int x = blockIdx.x * kBlock3 + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
   if (x >= p.nx) return;
+  const Nbr3 nb(p, x, y, z);
+  T g[kQ3];
+#pragma unroll
+  for (int i = 0; i < kQ3; ++i) g[i] = (src + i * p.plane)[nb.at(-cx3(i), -cy3(i), -cz3(i))];
+  T s;
   if (sizeof(T) == 8) {
-    T s = src[at3(p, x, y, z)];                   // f_0 (c_0 = 0)
+    s = g[0];                                     // f_0 (c_0 = 0)
 #pragma unroll
-    for (int i = 1; i < kQ3; ++i)
-      s += src[i * p.plane + at3(p, wrap3(x - cx3(i), p.nx), wrap3(y - cy3(i), p.ny),
-                                 wrap3(z - cz3(i), p.nz))];
-    rho[at3(p, x, y, z)] = s;
+    for (int i = 1; i < kQ3; ++i) s += g[i];
   } else {
-    T g[kQ3];
-#pragma unroll
-    for (int i = 0; i < kQ3; ++i)
-      g[i] = src[i * p.plane + at3(p, wrap3(x - cx3(i), p.nx), wrap3(y - cy3(i), p.ny),
-                                   wrap3(z - cz3(i), p.nz))];
-    rho[at3(p, x, y, z)] = g[0] + moving_sum3(g);
+    s = g[0] + moving_sum3(g);
   }
+  rho[nb.at(0, 0, 0)] = s;
 }
 
 // mu from the sums of the axis and edge neighbours' densities and the own
@@ -154,9 +159,11 @@ __global__ void __launch_bounds__(kBlock3) d3_density(const T* __restrict__ src,
 // grad3_from, force3, update3_f32): a result then does not depend on which
 // multiply-adds the compiler contracts in one kernel or another.
 __device__ __forceinline__ double mu3(double ax, double ed, double c, const NodeConsts<double>& q) {
-  const double lap = (1.0 / 3.0) * (ax - 6.0 * c) + (1.0 / 6.0) * (ed - 12.0 * c);
-  const double a = c + q.dl, b = c + q.dg;
-  return q.two_beta * a * b * (a + b) - q.kappa * lap;
+  const double lap = __fma_rn(1.0 / 3.0, __fma_rn(-6.0, c, ax),
+                              __dmul_rn(1.0 / 6.0, __fma_rn(-12.0, c, ed)));
+  const double a = __dadd_rn(c, q.dl), b = __dadd_rn(c, q.dg);
+  return __fma_rn(__dmul_rn(__dmul_rn(q.two_beta, a), b), __dadd_rn(a, b),
+                  -__dmul_rn(q.kappa, lap));
 }
 __device__ __forceinline__ float mu3(float ax, float ed, float c, const NodeConsts<float>& q) {
   const float lap = __fmaf_rn(1.0f / 3.0f, __fmaf_rn(-6.0f, c, ax),
@@ -175,20 +182,17 @@ __global__ void __launch_bounds__(kBlock3) d3_chem_pot(const T* __restrict__ rho
                                                        T* __restrict__ mu, const P3 p) {
   const int x = blockIdx.x * kBlock3 + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
   if (x >= p.nx) return;
-  const T c = rho[at3(p, x, y, z)];
+  const Nbr3 nb(p, x, y, z);
   // sums of the axis and edge neighbours, then the centre's share taken off
   // once per sum (rather than from every neighbour): 6 (ax/18 + ed/36)
-  auto nbr = [&](int i) {
-    return __ldg(rho + at3(p, wrap3(x + cx3(i), p.nx), wrap3(y + cy3(i), p.ny),
-                           wrap3(z + cz3(i), p.nz)));
-  };
+  auto nbr = [&](int i) { return __ldg(rho + nb.at(cx3(i), cy3(i), cz3(i))); };
   T ax = nbr(1), ed = nbr(7);
 #pragma unroll
   for (int i = 2; i < kQ3; ++i) {
     if (i == 7) continue;
     if (i < 7) ax += nbr(i); else ed += nbr(i);
   }
-  mu[at3(p, x, y, z)] = mu3(ax, ed, c, consts3<T>(p));
+  mu[nb.at(0, 0, 0)] = mu3(ax, ed, rho[nb.at(0, 0, 0)], consts3(p, T(0)));
 }
 
 // 12 grad(phi) from v(dx, dy, dz) = phi(x + (dx, dy, dz)); see grad3x12.
@@ -207,29 +211,24 @@ __device__ __forceinline__ void grad3_sums(const V& v, T& gx, T& gy, T& gz) {
 // (edge differences); the factor 1/12 is folded into the constants that
 // use the gradients.
 template <typename T>
-__device__ __forceinline__ void grad3x12(const T* __restrict__ phi, const P3& p, int x, int y,
-                                         int z, T& gx, T& gy, T& gz) {
-  auto v = [&](int dx, int dy, int dz) {
-    return __ldg(phi + at3(p, wrap3(x + dx, p.nx), wrap3(y + dy, p.ny), wrap3(z + dz, p.nz)));
-  };
-  grad3_sums<T>(v, gx, gy, gz);
+__device__ __forceinline__ void grad3x12(const T* __restrict__ phi, const Nbr3& nb, T& gx, T& gy,
+                                         T& gz) {
+  grad3_sums<T>([&](int dx, int dy, int dz) { return __ldg(phi + nb.at(dx, dy, dz)); }, gx, gy, gz);
 }
 
-// One component of F from 12 grad mu and 12 grad rho, nr = -rho / 12:
-// -rho grad mu (Eq. mF), or the potential form of the standard scheme.
+// One component of u = (j + F/2) / rho (Eq. rhoU) from 12 grad mu and 12 grad
+// rho, inv = 1/rho: F = -rho grad mu (Eq. mF), plus cs^2 grad rho in the
+// potential form of the standard scheme.
 template <bool WB>
-__device__ __forceinline__ double force3(double nr, double gm, double gr) {
-  return WB ? nr * gm : (1.0 / 36.0) * gr + nr * gm;
+__device__ __forceinline__ double vel3(double j, double rho, double gm, double gr, double inv) {
+  double s = __fma_rn(__dmul_rn(rho, -1.0 / 24.0), gm, j);
+  if (!WB) s = __fma_rn(1.0 / 72.0, gr, s);
+  return __dmul_rn(s, inv);
 }
 template <bool WB>
-__device__ __forceinline__ float force3(float nr, float gm, float gr) {
-  return WB ? __fmul_rn(nr, gm) : __fmaf_rn(nr, gm, __fmul_rn(1.0f / 36.0f, gr));
-}
-// (j + F/2) / rho
-__device__ __forceinline__ double vel3(double j, double F, double inv) {
-  return (j + 0.5 * F) * inv;
-}
-__device__ __forceinline__ float vel3(float j, float F, float inv) {
+__device__ __forceinline__ float vel3(float j, float rho, float gm, float gr, float inv) {
+  const float nr = __fmul_rn(rho, -1.0f / 12.0f);
+  const float F = WB ? __fmul_rn(nr, gm) : __fmaf_rn(nr, gm, __fmul_rn(1.0f / 36.0f, gr));
   return __fmul_rn(__fmaf_rn(0.5f, F, j), inv);
 }
 
@@ -288,7 +287,7 @@ __device__ __forceinline__ float2 dot3_x2(float2 ax, float2 bx, float2 ay, float
   return fma2(az, bz, fma2(ax, bx, mul2(ay, by)));
 }
 
-// The FP32 update of a pair of nodes (the terms of d3_collide below): rs the
+// The FP32 update of a pair of nodes (the terms of update3_f64 below): rs the
 // stored densities, (mx, my, mz) 12 grad mu, (rx, ry, rz) 12 grad rho; key_a,
 // key_b the nodes' numbers and ht the step's key (the draws of the rest
 // populations' roundings).
@@ -377,160 +376,146 @@ __device__ __forceinline__ void update3_x2(float2 (&g)[19], float2 rs, float2 mx
   }
 }
 
-// The collision of one node, and its stores (MOMENTS: fields and stats
-// instead).  For an opposite pair (i, i') the even part E and the odd part
-// O of omega f^eq + kforce F_i are shared, g_i' = keep g_i + E + O,
-// g_i'' = keep g_i' + E - O, with
-//   E = w (t + cu (omega rho 9/2 cu + 9 kforce cG) + kforce h (u.grad rho))
-//       [+ omega w rho for the standard equilibrium],
-//   O = 3 w (omega rho cu + kforce cF),
-//   t = -3/2 omega rho u.u - 3 kforce u.G,
+// The FP64 update of one node's populations.  For an opposite pair (i, i') the
+// even part E and the odd part O of omega f^eq + kforce F_i are shared,
+// g_i' = keep g_i + E + O, g_i'' = keep g_i' + E - O, with
+//   E = w (9 (c.u)(c.A) - 3 S + kforce h (u.grad rho)) [+ omega w rho, standard],
+//   O = 3 w c.M,   A = (omega rho / 2) u + kforce G,   S = u.A,
+//   M = omega rho u + kforce F,
 // G = F + cs^2 grad rho and h = (3|c|^2 - 3)/2 (Eq. mFi, D = 3) for the
-// well-balanced scheme, G = F and h = 0 for the standard one (Eq. Fi).
-template <typename T, bool WB, bool MOMENTS>
-__global__ void __launch_bounds__(kBlock3) d3_collide(const T* __restrict__ src,
-                                                      T* __restrict__ dst,
-                                                      const T* __restrict__ rho,
-                                                      const T* __restrict__ mu,
-                                                      const P3 p, const Out3 out) {
-  constexpr bool kShifted = sizeof(T) == 4;    // FP32 stores g_i = f_i - s_i
-  const int x = blockIdx.x * kBlock3 + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
-  const bool own = x < p.nx;
-  double st[kStatRec] = {0.0, 0.0, 0.0, 1e300, -1e300, 0.0};
-  if (own) {
-    T g[kQ3];
+// well-balanced scheme, G = F and h = 0 for the standard one (Eq. Fi).  On an
+// axis (c.u)(c.A) is a product P = u_a A_a, on an edge (a, b) it is
+// P_a + P_b +- X_ab with X_ab = u_a A_b + u_b A_a, and P_a + P_b = S - P_c, so
+// u.u and u.G are not needed.  A, P, S, X, kforce F and omega rho are carried
+// divided by 6: E_axis = 3 P - S, E_edge = S - 3/2 P_c + B +- 3/2 X,
+// B = kforce (u.grad rho) / 24, O_axis = M, O_edge = (M_a +- M_b) / 2.
+// 161 FP64 operations with both gradients (191 with u.u, u.G and the pairs'
+// sums formed one by one); the FP64 pipe is what bounds the kernel.  128^3
+// well-balanced: 940 us per step before, 824 us; errors against 128-bit
+// arithmetic as before (WB: populations 0.8e-16 to 1.9e-16 relative).
+template <bool WB>
+__device__ __forceinline__ void update3_f64(double (&g)[19], double r, double gmx, double gmy,
+                                            double gmz, double grx, double gry, double grz,
+                                            double ux, double uy, double uz,
+                                            const P3& p) {
+  const NodeConsts<double>& q = p.d;
+  const double kc = __dmul_rn(r, p.kc72), keep = q.keep;
+  auto kforce = [&](double gm, double gr) {             // kforce F / 6
+    return WB ? __dmul_rn(kc, gm) : __fma_rn(kc, gm, __dmul_rn(q.kf216, gr));
+  };
+  const double kFx = kforce(gmx, grx), kFy = kforce(gmy, gry), kFz = kforce(gmz, grz);
+  const double kGx = WB ? __fma_rn(q.kf216, grx, kFx) : kFx;
+  const double kGy = WB ? __fma_rn(q.kf216, gry, kFy) : kFy;
+  const double kGz = WB ? __fma_rn(q.kf216, grz, kFz) : kFz;
+  const double orho = __dmul_rn(q.omega, r);
+  const double o6 = __dmul_rn(orho, 1.0 / 6.0), h6 = __dmul_rn(orho, 1.0 / 12.0);
+  const double Ax = __fma_rn(h6, ux, kGx), Ay = __fma_rn(h6, uy, kGy), Az = __fma_rn(h6, uz, kGz);
+  const double Mx = __fma_rn(o6, ux, kFx), My = __fma_rn(o6, uy, kFy), Mz = __fma_rn(o6, uz, kFz);
+  const double Px = __dmul_rn(ux, Ax), Py = __dmul_rn(uy, Ay), Pz = __dmul_rn(uz, Az);
+  const double S = __dadd_rn(__dadd_rn(Px, Py), Pz);
+  double Ca, Ce;
+  if (WB) {
+    const double D = __fma_rn(uz, grz, __fma_rn(ux, grx, __dmul_rn(uy, gry)));
+    Ca = -S;
+    Ce = __fma_rn(p.kf288, D, S);
+    // E_0 = omega rho - 6 (S + 2 B): rest equilibrium rho - (rho/2) u.u, F_0 of Eq. mFi
+    g[0] = __fma_rn(keep, g[0], __fma_rn(-6.0, __fma_rn(2.0, Ce, -S), orho));
+  } else {
+    Ca = __fma_rn(1.0 / 18.0, orho, -S);
+    Ce = __fma_rn(1.0 / 36.0, orho, S);
+    g[0] = __fma_rn(keep, g[0], __dmul_rn(6.0, Ca));
+  }
+  auto axis = [&](int i, int j, double P, double M) {
+    const double E = __fma_rn(3.0, P, Ca);
+    g[i] = __fma_rn(keep, g[i], __dadd_rn(E, M));
+    g[j] = __fma_rn(keep, g[j], __dadd_rn(E, -M));
+  };
+  // the four pairs of the edges in the plane of components a, b (P: the
+  // third component's product)
+  auto edges = [&](int i, int j, int k, int l, double ua, double Aa, double ub, double Ab, double P,
+                   double Ma, double Mb) {
+    const double X = __fma_rn(ua, Ab, __dmul_rn(ub, Aa)), E0 = __fma_rn(-1.5, P, Ce);
+    const double Ep = __fma_rn(1.5, X, E0), Em = __fma_rn(-1.5, X, E0);
+    const double Tp = __dadd_rn(Ma, Mb), Tm = __dadd_rn(Ma, -Mb);
+    g[i] = __fma_rn(keep, g[i], __fma_rn(0.5, Tp, Ep));
+    g[j] = __fma_rn(keep, g[j], __fma_rn(-0.5, Tp, Ep));
+    g[k] = __fma_rn(keep, g[k], __fma_rn(0.5, Tm, Em));
+    g[l] = __fma_rn(keep, g[l], __fma_rn(-0.5, Tm, Em));
+  };
+  axis(1, 2, Px, Mx);
+  axis(3, 4, Py, My);
+  axis(5, 6, Pz, Mz);
+  edges(7, 8, 9, 10, ux, Ax, uy, Ay, Pz, Mx, My);
+  edges(11, 12, 13, 14, ux, Ax, uz, Az, Py, Mx, Mz);
+  edges(15, 16, 17, 18, uy, Ay, uz, Az, Px, My, Mz);
+}
+
+// One node: its pulled populations, 12 grad mu, 12 grad rho and u.
+template <typename T, bool WB>
+struct Node3 {
+  T g[kQ3], rs, r, gmx, gmy, gmz, grx, gry, grz, ux, uy, uz;
+  __device__ __forceinline__ Node3(const T* __restrict__ src, const T* __restrict__ rho,
+                                   const T* __restrict__ mu, const P3& p, const Nbr3& nb) {
 #pragma unroll
-    for (int i = 0; i < kQ3; ++i)
-      g[i] = src[i * p.plane + at3(p, wrap3(x - cx3(i), p.nx), wrap3(y - cy3(i), p.ny),
-                                   wrap3(z - cz3(i), p.nz))];
-    const long long k = at3(p, x, y, z);
-    const T rs = rho[k];                         // rho - rho_ref (rho in FP64)
-    const T r = kShifted ? rs + consts3<T>(p).rho_ref : rs;
-    // 12 grad mu, 12 grad rho; F = -rho grad mu (Eq. mF), or the potential
-    // form cs^2 grad rho - rho grad mu of the standard scheme
-    T gmx, gmy, gmz, grx, gry, grz;
-    grad3x12<T>(mu, p, x, y, z, gmx, gmy, gmz);
-    grad3x12<T>(rho, p, x, y, z, grx, gry, grz);
-    const T nr = r * T(-1.0 / 12.0);
-    const T Fx = force3<WB>(nr, gmx, grx), Fy = force3<WB>(nr, gmy, gry),
-            Fz = force3<WB>(nr, gmz, grz);
+    for (int i = 0; i < kQ3; ++i) g[i] = (src + i * p.plane)[nb.at(-cx3(i), -cy3(i), -cz3(i))];
+    rs = rho[nb.at(0, 0, 0)];                  // rho - rho_ref (rho in FP64)
+    r = sizeof(T) == 4 ? rs + consts3(p, T(0)).rho_ref : rs;
+    grad3x12<T>(mu, nb, gmx, gmy, gmz);
+    grad3x12<T>(rho, nb, grx, gry, grz);
     T jx, jy, jz;
     momentum3(g, jx, jy, jz);
     const T inv = recip(r);
-    const T ux = vel3(jx, Fx, inv), uy = vel3(jy, Fy, inv), uz = vel3(jz, Fz, inv);  // Eq. rhoU
-    const T muc = mu[k];
-    if constexpr (MOMENTS) {
-      const double rd = kShifted ? (double)rs + p.rho_ref : (double)r;
-      const double uxd = ux, uyd = uy, uzd = uz, mud = muc;
-      if (out.rho) out.rho[(size_t)(z * p.ny + y) * p.nx + x] = rd;
-      if (out.ux) out.ux[(size_t)(z * p.ny + y) * p.nx + x] = uxd;
-      if (out.uy) out.uy[(size_t)(z * p.ny + y) * p.nx + x] = uyd;
-      if (out.uz) out.uz[(size_t)(z * p.ny + y) * p.nx + x] = uzd;
-      if (out.mu) out.mu[(size_t)(z * p.ny + y) * p.nx + x] = mud;
-      const double u2 = uxd * uxd + uyd * uyd + uzd * uzd;
-      st[0] = rd;
-      st[1] = 0.5 * rd * u2;
-      st[2] = u2;
-      st[3] = mud;
-      st[4] = mud;
-      st[5] = (!isfinite(rd) || !isfinite(mud) || !isfinite(u2)) ? 1.0 : 0.0;
-    } else {
-      const NodeConsts<T> q = consts3<T>(p);
-      static_assert(MOMENTS || !kShifted, "FP32 steps run in d3_step_f32");
-      {
-        const T om = q.omega, kf = q.kf, keep = q.keep;
-        T Gx = Fx, Gy = Fy, Gz = Fz;
-        if (WB) {
-          Gx = Fx + T(1.0 / 36.0) * grx;                          // G = F + cs^2 grad rho
-          Gy = Fy + T(1.0 / 36.0) * gry;
-          Gz = Fz + T(1.0 / 36.0) * grz;
-        }
-        const T orho = om * r;
-        const T obase = om * rs;                   // omega (rho - rho_ref): the stored base
-        const T t = T(-1.5) * orho * (ux * ux + uy * uy + uz * uz) -
-                    T(3.0) * kf * (ux * Gx + uy * Gy + uz * Gz);
-        const T ku = WB ? (kf * T(1.0 / 12.0)) * (ux * grx + uy * gry + uz * grz) : T(0);
-        // per-node constants of the pairs, with the weights folded in
-        // (w_ax = 1/18, w_edge = 1/36): E = C + cu (A cu + K.c), O = 3 w c.M
-        const T Ca = WB ? T(1.0 / 18.0) * t : T(1.0 / 18.0) * (t + obase);
-        const T Ce = WB ? T(1.0 / 36.0) * (t + T(1.5) * ku) : T(1.0 / 36.0) * (t + obase);
-        const T Aa = T(0.25) * orho, Ae = T(0.125) * orho;         // w 9/2 omega rho
-        const T kh = T(0.5) * kf, kq = T(0.25) * kf, k6 = kf * T(1.0 / 6.0);
-        const T Kax = kh * Gx, Kay = kh * Gy, Kaz = kh * Gz;       // 9 w_ax kforce G
-        const T Kex = kq * Gx, Key = kq * Gy, Kez = kq * Gz;       // 9 w_edge kforce G
-        const T o6 = orho * T(1.0 / 6.0);                          // 3 w_ax (omega rho u + kforce F)
-        const T Mx = o6 * ux + k6 * Fx, My = o6 * uy + k6 * Fy, Mz = o6 * uz + k6 * Fz;
-        auto axis = [&](int i, int j, T cu, T K, T M) {
-          const T E = Ca + cu * (Aa * cu + K);
-          g[i] = keep * g[i] + (E + M);
-          g[j] = keep * g[j] + (E - M);
-          return E;
-        };
-        // edge pair: 3 w_edge c.M = (Ma + Mb) / 2 for c = a + b
-        auto edge = [&](int i, int j, T cu, T K, T S) {
-          const T E = Ce + cu * (Ae * cu + K);
-          g[i] = keep * g[i] + (E + T(0.5) * S);
-          g[j] = keep * g[j] + (E - T(0.5) * S);
-          return E;
-        };
-        const T Ea1 = axis(1, 2, ux, Kax, Mx);
-        const T Ea2 = axis(3, 4, uy, Kay, My);
-        const T Ea3 = axis(5, 6, uz, Kaz, Mz);
-        const T Ee1 = edge(7, 8, ux + uy, Kex + Key, Mx + My);
-        const T Ee2 = edge(9, 10, ux - uy, Kex - Key, Mx - My);
-        const T Ee3 = edge(11, 12, ux + uz, Kex + Kez, Mx + Mz);
-        const T Ee4 = edge(13, 14, ux - uz, Kex - Kez, Mx - Mz);
-        const T Ee5 = edge(15, 16, uy + uz, Key + Kez, My + Mz);
-        const T Ee6 = edge(17, 18, uy - uz, Key - Kez, My - Mz);
-        // rest: WB f_0^eq - s_0 = rho - w_0 3/2 rho u.u, F_0 = w_0 (-3 u.G - 3/2 u.grad rho);
-        // standard f_0^eq = w_0 rho (1 - 3/2 u.u), F_0 = w_0 (-3 u.G)
-        const T w0 = T(1.0 / 3.0);
-        g[0] = keep * g[0] + (WB ? obase + w0 * (t - T(1.5) * ku) : w0 * (t + obase));
-      }
-#pragma unroll
-      for (int i = 0; i < kQ3; ++i) dst[i * p.plane + k] = g[i];
-    }
+    ux = vel3<WB>(jx, r, gmx, grx, inv);
+    uy = vel3<WB>(jy, r, gmy, gry, inv);
+    uz = vel3<WB>(jz, r, gmz, grz, inv);
   }
-  if (MOMENTS && out.partials) {
-    __shared__ double red[kBlock3 / 32][kStatRec];
+};
+
+// FP64 step: the collision of one node, and its stores.
+template <bool WB>
+__global__ void __launch_bounds__(kBlock3) d3_collide(const double* __restrict__ src,
+                                                      double* __restrict__ dst,
+                                                      const double* __restrict__ rho,
+                                                      const double* __restrict__ mu, const P3 p) {
+  const int x = blockIdx.x * kBlock3 + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
+  if (x >= p.nx) return;
+  const Nbr3 nb(p, x, y, z);
+  Node3<double, WB> n(src, rho, mu, p, nb);
+  update3_f64<WB>(n.g, n.r, n.gmx, n.gmy, n.gmz, n.grx, n.gry, n.grz, n.ux, n.uy, n.uz, p);
+  const unsigned k = nb.at(0, 0, 0);
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      const double o0 = __shfl_down_sync(0xffffffffu, st[0], off);
-      const double o1 = __shfl_down_sync(0xffffffffu, st[1], off);
-      const double o2 = __shfl_down_sync(0xffffffffu, st[2], off);
-      const double o3 = __shfl_down_sync(0xffffffffu, st[3], off);
-      const double o4 = __shfl_down_sync(0xffffffffu, st[4], off);
-      const double o5 = __shfl_down_sync(0xffffffffu, st[5], off);
-      st[0] += o0;
-      st[1] += o1;
-      st[2] = fmax(st[2], o2);
-      st[3] = fmin(st[3], o3);
-      st[4] = fmax(st[4], o4);
-      st[5] = fmax(st[5], o5);
-    }
-    const int warp = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0)
-#pragma unroll
-      for (int q = 0; q < kStatRec; ++q) red[warp][q] = st[q];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double r[kStatRec];
-#pragma unroll
-      for (int q = 0; q < kStatRec; ++q) r[q] = red[0][q];
-      for (int w = 1; w < kBlock3 / 32; ++w) {
-        r[0] += red[w][0];
-        r[1] += red[w][1];
-        r[2] = fmax(r[2], red[w][2]);
-        r[3] = fmin(r[3], red[w][3]);
-        r[4] = fmax(r[4], red[w][4]);
-        r[5] = fmax(r[5], red[w][5]);
-      }
-      double* o = out.partials +
-                  (size_t)((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * kStatRec;
-#pragma unroll
-      for (int q = 0; q < kStatRec; ++q) o[q] = r[q];
-    }
+  for (int i = 0; i < kQ3; ++i) (dst + i * p.plane)[k] = n.g[i];
+}
+
+// Fields and statistics of kMomPlanes3 planes per CTA: one record for all of
+// them, so that the reduction's shuffles and the final pass over the records
+// (one CTA) are shared by several nodes of each thread.
+constexpr int kMomPlanes3 = 8;
+template <typename T, bool WB>
+__global__ void __launch_bounds__(kBlock3) d3_moments(const T* __restrict__ src,
+                                                      const T* __restrict__ rho,
+                                                      const T* __restrict__ mu, const P3 p,
+                                                      const Out3 out) {
+  const int x = blockIdx.x * kBlock3 + threadIdx.x, y = blockIdx.y;
+  const int z0 = blockIdx.z * kMomPlanes3, z1 = min(z0 + kMomPlanes3, p.nz);
+  StatsAcc<T> acc;
+  for (int z = z0; z < z1 && x < p.nx; ++z) {
+    const Nbr3 nb(p, x, y, z);
+    const Node3<T, WB> n(src, rho, mu, p, nb);
+    const double rd = sizeof(T) == 4 ? widen(n.rs) + p.rho_ref : (double)n.r;
+    const double ux = widen(n.ux), uy = widen(n.uy), uz = widen(n.uz);
+    const T muc = mu[nb.at(0, 0, 0)];
+    const size_t k = ((size_t)z * p.ny + y) * p.nx + x;
+    if (out.rho) out.rho[k] = rd;
+    if (out.ux) out.ux[k] = ux;
+    if (out.uy) out.uy[k] = uy;
+    if (out.uz) out.uz[k] = uz;
+    if (out.mu) out.mu[k] = widen(muc);
+    acc.add(rd, muc, __fma_rn(uz, uz, __fma_rn(ux, ux, __dmul_rn(uy, uy))));
   }
+  write_stats_record<kBlock3>(
+      acc, out.partials + (size_t)((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) *
+                              kStatRec);
 }
 
 // The whole FP32 step in one kernel: a CTA owns TX x TY columns and marches a
@@ -753,7 +738,8 @@ Layout3 layout3(const wblbe3_params* p) {
   L.plane = (long long)L.pitch * p->ny * p->nz;
   const size_t pops = align3((size_t)kQ3 * L.plane * elem3(p));
   const size_t field = align3((size_t)L.plane * elem3(p));
-  L.records = (long long)((p->nx + kBlock3 - 1) / kBlock3) * p->ny * p->nz;
+  L.records = (long long)((p->nx + kBlock3 - 1) / kBlock3) * p->ny *
+              ((p->nz + kMomPlanes3 - 1) / kMomPlanes3);
   size_t off = 0;
   L.off_a = off; off += pops;
   L.off_b = off; off += pops;
@@ -830,13 +816,12 @@ P3 p3_of(const wblbe3_ctx* h) {
   q.plane = h->L.plane;
   // FP32 stores deviations from the rest equilibrium at rho_ref = rho_g
   q.rho_ref = h->p.precision == WBLBE_FP64 ? 0.0 : h->p.rho_g;
-  q.omega = 1.0 / h->p.tau;
-  q.kforce = 1.0 - 1.0 / (2.0 * h->p.tau);
-  q.kappa = h->p.kappa;
-  q.two_beta = 2.0 * h->p.beta;
-  q.dl = q.rho_ref - h->p.rho_l;
-  q.dg = q.rho_ref - h->p.rho_g;
-  q.f.set(q.omega, q.kforce, q.kappa, q.two_beta, q.dl, q.dg, q.rho_ref);
+  const double om = 1.0 / h->p.tau, kf = 1.0 - 1.0 / (2.0 * h->p.tau), tb = 2.0 * h->p.beta;
+  const double dl = q.rho_ref - h->p.rho_l, dg = q.rho_ref - h->p.rho_g;
+  q.d.set(om, kf, h->p.kappa, tb, dl, dg, q.rho_ref);
+  q.f.set(om, kf, h->p.kappa, tb, dl, dg, q.rho_ref);
+  q.kc72 = -kf / 72.0;
+  q.kf288 = kf / 288.0;
   q.step = h->steps;
   return q;
 }
@@ -853,23 +838,21 @@ double shift3(const wblbe3_params& p, int i) {
   return i == 0 ? rr - (1.0 - w3(0)) * p.rho0 : w3(i) * p.rho0;
 }
 
-// density and chemical potential of the current state, then the collision
-// (step: into the other buffer) or the moments (fields and stats).
-template <typename T>
+// Density and chemical potential of the current state, then the moments
+// (fields and statistics), or in FP64 the collision into the other buffer.
+template <typename T, bool WB>
 void pass3_typed(wblbe3_ctx* h, bool moments, const Out3& out, const P3& q, dim3 g) {
   const T* src = static_cast<const T*>(h->buf[h->cur]);
-  T* dst = static_cast<T*>(h->buf[1 - h->cur]);
   T* rho = static_cast<T*>(h->rho);
   T* mu = static_cast<T*>(h->mu);
   d3_density<T><<<g, kBlock3, 0, h->stream>>>(src, rho, q);
   d3_chem_pot<T><<<g, kBlock3, 0, h->stream>>>(rho, mu, q);
-  const bool wb = h->p.scheme == WBLBE_WELL_BALANCED;
   if (moments) {
-    if (wb) d3_collide<T, true, true><<<g, kBlock3, 0, h->stream>>>(src, nullptr, rho, mu, q, out);
-    else d3_collide<T, false, true><<<g, kBlock3, 0, h->stream>>>(src, nullptr, rho, mu, q, out);
+    const dim3 gm(g.x, g.y, (h->p.nz + kMomPlanes3 - 1) / kMomPlanes3);
+    d3_moments<T, WB><<<gm, kBlock3, 0, h->stream>>>(src, rho, mu, q, out);
   } else if constexpr (sizeof(T) == 8) {
-    if (wb) d3_collide<T, true, false><<<g, kBlock3, 0, h->stream>>>(src, dst, rho, mu, q, out);
-    else d3_collide<T, false, false><<<g, kBlock3, 0, h->stream>>>(src, dst, rho, mu, q, out);
+    d3_collide<WB><<<g, kBlock3, 0, h->stream>>>(src, static_cast<T*>(h->buf[1 - h->cur]), rho, mu,
+                                                 q);
   }
 }
 
@@ -913,10 +896,13 @@ wblbe_status pass3(wblbe3_ctx* h, bool moments, const Out3& out) {
     return WBLBE_OK;
   }
   const dim3 g = grid3(h);
+  const bool wb = h->p.scheme == WBLBE_WELL_BALANCED;
   if (h->p.precision == WBLBE_FP64)
-    pass3_typed<double>(h, moments, out, q, g);
+    wb ? pass3_typed<double, true>(h, moments, out, q, g)
+       : pass3_typed<double, false>(h, moments, out, q, g);
   else
-    pass3_typed<float>(h, moments, out, q, g);
+    wb ? pass3_typed<float, true>(h, moments, out, q, g)
+       : pass3_typed<float, false>(h, moments, out, q, g);
   CU3(h, cudaGetLastError());
   h->launches += 3;
   return WBLBE_OK;

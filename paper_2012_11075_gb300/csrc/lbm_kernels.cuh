@@ -904,53 +904,90 @@ enum StripMode {
   kModeStepStats = 2   // store, and accumulate per-CTA stats of f(t)
 };
 
-// Per-CTA statistics of the collided nodes (FP64 accumulators).
+// (double)v on the integer units: the exponent rebased and the mantissa
+// shifted, exact.  The hardware's conversion runs on the FP64 pipe, which has
+// two lanes per SM and clock; it is left to subnormal and non-finite values.
+__device__ __forceinline__ double widen(float v) {
+  const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
+  if (m - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+  return m == 0 ? __hiloint2double((int)b, 0) : (double)v;
+}
+__device__ __forceinline__ double widen(double v) { return v; }
+
+__device__ __forceinline__ bool finite_bits(double v) {
+  return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000;
+}
+
+// Per-thread statistics of the nodes, sums in FP64.  In FP32 the extrema stay
+// off the FP64 pipe, where a comparison costs as much as an addition: mu's in
+// float, max |u|^2 (never negative) by its bits.  NaNs are left out of the
+// extrema, as fmin and fmax do.  FP32 moments of the 4096^2 lattice (16
+// rows per CTA): 663 us with conversions and extrema on the FP64 pipe, 317 us.
+template <typename T>
 struct StatsAcc {
-  double mass = 0.0, kin = 0.0, u2 = 0.0, mumin = 1e300, mumax = -1e300;
+  double mass = 0.0, kin2 = 0.0, u2 = 0.0;   // sum rho, sum rho |u|^2, max |u|^2
+  T mumin = T(INFINITY), mumax = T(-INFINITY);
   int bad = 0;
+
+  __device__ __forceinline__ void max_u2(double v) {
+    if constexpr (sizeof(T) == 8) {
+      u2 = fmax(u2, v);
+    } else {
+      const long long k = __double_as_longlong(v);
+      if (k > __double_as_longlong(u2) && k <= 0x7ff0000000000000LL) u2 = v;
+    }
+  }
+  __device__ __forceinline__ void add(double rho, T mu, double speed2) {
+    mass += rho;
+    kin2 = __fma_rn(rho, speed2, kin2);
+    max_u2(speed2);
+    mumin = min(mumin, mu);
+    mumax = max(mumax, mu);
+    if (!finite_bits(rho) || !isfinite(mu) || !finite_bits(speed2)) bad = 1;
+  }
+  __device__ __forceinline__ void fold(const StatsAcc& o) {
+    mass += o.mass;
+    kin2 += o.kin2;
+    max_u2(o.u2);
+    mumin = min(mumin, o.mumin);
+    mumax = max(mumax, o.mumax);
+    bad |= o.bad;
+  }
+  __device__ __forceinline__ StatsAcc from_lane(int off) const {
+    StatsAcc o;
+    o.mass = __shfl_down_sync(0xffffffffu, mass, off);
+    o.kin2 = __shfl_down_sync(0xffffffffu, kin2, off);
+    o.u2 = __shfl_down_sync(0xffffffffu, u2, off);
+    o.mumin = __shfl_down_sync(0xffffffffu, mumin, off);
+    o.mumax = __shfl_down_sync(0xffffffffu, mumax, off);
+    o.bad = __shfl_down_sync(0xffffffffu, bad, off);
+    return o;
+  }
 };
 
 // One CTA's statistics record from its threads' accumulators (every thread of
 // the CTA calls it): warp shuffles, then thread 0 over the warps; a fixed
 // order, so the record does not vary from run to run.
-template <int NT>
-__device__ __forceinline__ void write_stats_record(const StatsAcc& acc, double* rec) {
-  __shared__ double red[NT / 32][kStatRec];
-  double v[kStatRec] = {acc.mass, acc.kin, acc.u2, acc.mumin, acc.mumax, (double)acc.bad};
+template <int NT, typename T>
+__device__ __forceinline__ void write_stats_record(StatsAcc<T> acc, double* rec) {
+  __shared__ __align__(8) unsigned char raw[NT / 32 * sizeof(StatsAcc<T>)];
+  StatsAcc<T>* red = reinterpret_cast<StatsAcc<T>*>(raw);
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    double o0 = __shfl_down_sync(0xffffffffu, v[0], off);
-    double o1 = __shfl_down_sync(0xffffffffu, v[1], off);
-    double o2 = __shfl_down_sync(0xffffffffu, v[2], off);
-    double o3 = __shfl_down_sync(0xffffffffu, v[3], off);
-    double o4 = __shfl_down_sync(0xffffffffu, v[4], off);
-    double o5 = __shfl_down_sync(0xffffffffu, v[5], off);
-    v[0] += o0;
-    v[1] += o1;
-    v[2] = fmax(v[2], o2);
-    v[3] = fmin(v[3], o3);
-    v[4] = fmax(v[4], o4);
-    v[5] = fmax(v[5], o5);
-  }
-  const int tx = threadIdx.x, warp = tx >> 5, lane = tx & 31;
-  if (lane == 0)
-#pragma unroll
-    for (int q = 0; q < kStatRec; ++q) red[warp][q] = v[q];
+  for (int off = 16; off > 0; off >>= 1) acc.fold(acc.from_lane(off));
+  const int tx = threadIdx.x;
+  if ((tx & 31) == 0) red[tx >> 5] = acc;
   __syncthreads();
   if (tx == 0) {
-    double r[kStatRec];
-#pragma unroll
-    for (int q = 0; q < kStatRec; ++q) r[q] = red[0][q];
-    for (int q = 1; q < NT / 32; ++q) {
-      r[0] += red[q][0];
-      r[1] += red[q][1];
-      r[2] = fmax(r[2], red[q][2]);
-      r[3] = fmin(r[3], red[q][3]);
-      r[4] = fmax(r[4], red[q][4]);
-      r[5] = fmax(r[5], red[q][5]);
-    }
-#pragma unroll
-    for (int q = 0; q < kStatRec; ++q) rec[q] = r[q];
+    StatsAcc<T> r = red[0];
+    for (int q = 1; q < NT / 32; ++q) r.fold(red[q]);
+    const bool any = r.mumin <= r.mumax;     // else the records' neutral values
+    rec[0] = r.mass;
+    rec[1] = 0.5 * r.kin2;
+    rec[2] = r.u2;
+    rec[3] = any ? (double)r.mumin : 1e300;
+    rec[4] = any ? (double)r.mumax : -1e300;
+    rec[5] = (double)r.bad;
   }
 }
 
@@ -961,7 +998,7 @@ template <typename T, int MODE, bool GHOST>
 __device__ __forceinline__ void emit_node(const KParams& p, const MomentsOut& mo, T* dst, int c,
                                           int xcol, int xm, bool ghost_r, bool ghost_l,
                                           const T (&gv)[9], T rs, T muc, T ux, T uy,
-                                          StatsAcc& acc, bool acc_on) {
+                                          StatsAcc<T>& acc, bool acc_on) {
   constexpr bool MOMENTS = MODE == kModeMoments;
   constexpr bool STATS = MODE != kModeStep;
   if (!MOMENTS && WB_IN(c, p.ny) && WB_IN(xcol, p.pitch)) {
@@ -987,9 +1024,9 @@ __device__ __forceinline__ void emit_node(const KParams& p, const MomentsOut& mo
     }
   }
   if (STATS && acc_on) {
-    const double rho = (double)rs + p.rho_ref;
-    const double mu = (double)muc;
-    const double dux = (double)ux, duy = (double)uy;
+    const double rho = sizeof(T) == 4 ? widen(rs) + p.rho_ref : (double)rs;
+    const double mu = widen(muc);
+    const double dux = widen(ux), duy = widen(uy);
     if (MOMENTS && WB_IN(c, p.ny) && WB_IN(xm, p.nx)) {
       const unsigned kk = (unsigned)((c + p.y_offset) * p.nx + xm);
       if (mo.rho) mo.rho[kk] = rho;
@@ -997,13 +1034,7 @@ __device__ __forceinline__ void emit_node(const KParams& p, const MomentsOut& mo
       if (mo.uy) mo.uy[kk] = duy;
       if (mo.mu) mo.mu[kk] = mu;
     }
-    const double u2 = __fma_rn(dux, dux, __dmul_rn(duy, duy));
-    acc.mass += rho;
-    acc.kin = __fma_rn(__dmul_rn(0.5, rho), u2, acc.kin);
-    acc.u2 = fmax(acc.u2, u2);
-    acc.mumin = fmin(acc.mumin, mu);
-    acc.mumax = fmax(acc.mumax, mu);
-    if (!isfinite(rho) || !isfinite(mu) || !isfinite(u2)) acc.bad = 1;
+    acc.add(rho, muc, __fma_rn(dux, dux, __dmul_rn(duy, duy)));
   }
 }
 
@@ -1204,7 +1235,7 @@ __device__ __forceinline__ void strip_pass(const T* __restrict__ src, T* __restr
   cp_async_wait<PDG - 1>();                // first group landed (this thread)
   __syncthreads();                         // ... and everyone else's
 
-  StatsAcc acc;
+  StatsAcc<T> acc;
   const int xm = x0 + tx;                  // column of the moment fields
   // statistics are gathered only into a record (a uniform, runtime choice in
   // the step-and-statistics mode, so that one instantiation serves both)

@@ -45,7 +45,6 @@ __global__ void __launch_bounds__(kE6Threads)
                    const MomentsOut mo) {
   __shared__ double rho_t[kRhoH * kRhoW];
   __shared__ double mu_t[kMuH * kMuW];
-  __shared__ double red[kE6Threads / 32][kStatRec];
   constexpr int CX[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
   constexpr int CY[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
   const int tid = threadIdx.x;
@@ -73,7 +72,7 @@ __global__ void __launch_bounds__(kE6Threads)
   }
   __syncthreads();
   const NodeConsts<double>& cc = p.d;
-  StatsAcc acc;
+  StatsAcc<double> acc;
   const bool acc_on = MODE != kModeStep;
 #pragma unroll
   for (int half = 0; half < 2; ++half) {
@@ -94,44 +93,9 @@ __global__ void __launch_bounds__(kE6Threads)
           acc, acc_on);
     }
   }
-  if (MODE != kModeStep && mo.partials) {
-    double v[kStatRec] = {acc.mass, acc.kin, acc.u2, acc.mumin, acc.mumax, (double)acc.bad};
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      const double o0 = __shfl_down_sync(0xffffffffu, v[0], off);
-      const double o1 = __shfl_down_sync(0xffffffffu, v[1], off);
-      const double o2 = __shfl_down_sync(0xffffffffu, v[2], off);
-      const double o3 = __shfl_down_sync(0xffffffffu, v[3], off);
-      const double o4 = __shfl_down_sync(0xffffffffu, v[4], off);
-      const double o5 = __shfl_down_sync(0xffffffffu, v[5], off);
-      v[0] += o0;
-      v[1] += o1;
-      v[2] = fmax(v[2], o2);
-      v[3] = fmin(v[3], o3);
-      v[4] = fmax(v[4], o4);
-      v[5] = fmax(v[5], o5);
-    }
-    if ((tid & 31) == 0)
-#pragma unroll
-      for (int q = 0; q < kStatRec; ++q) red[tid >> 5][q] = v[q];
-    __syncthreads();
-    if (tid == 0) {
-      double r[kStatRec];
-#pragma unroll
-      for (int q = 0; q < kStatRec; ++q) r[q] = red[0][q];
-      for (int w = 1; w < kE6Threads / 32; ++w) {
-        r[0] += red[w][0];
-        r[1] += red[w][1];
-        r[2] = fmax(r[2], red[w][2]);
-        r[3] = fmin(r[3], red[w][3]);
-        r[4] = fmax(r[4], red[w][4]);
-        r[5] = fmax(r[5], red[w][5]);
-      }
-      double* out = mo.partials + (size_t)(blockIdx.y * gridDim.x + blockIdx.x) * kStatRec;
-#pragma unroll
-      for (int q = 0; q < kStatRec; ++q) out[q] = r[q];
-    }
-  }
+  if (MODE != kModeStep && mo.partials)
+    write_stats_record<kE6Threads>(
+        acc, mo.partials + (size_t)(blockIdx.y * gridDim.x + blockIdx.x) * kStatRec);
 }
 
 }  // namespace

@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(NT)
   __syncthreads();
 
   // ---- phase 3: collision ----
-  StatsAcc acc;
+  StatsAcc<T> acc;
   const int x = x0 + tx, y = y0 + r0;
   if (owner && x < nx && y < ny) {
     if constexpr (sizeof(T) == 4) {

@@ -25,7 +25,6 @@ namespace {
 
 constexpr size_t kAlign = 256;
 constexpr int kGraphSteps = 32;          // steps per captured graph (even)
-constexpr int kMomentsRows = 16;         // rows per CTA of the moments kernel
 constexpr int kNumSMs = 152;
 
 thread_local char g_thread_error[256] = "";
@@ -73,11 +72,11 @@ Layout make_layout(const wblbe_params* p) {
   L.pitch = (p->nx + align_elems - 1) / align_elems * align_elems;
   L.plane = (long long)L.pitch * p->ny;
   L.pops_bytes = align_up((size_t)9 * (size_t)L.plane * L.elem);
-  // per-CTA records: the moments pass (32-column strips at the narrowest,
-  // kMomentsRows rows) and a step with statistics in any default launch
+  // per-CTA records: the moments pass and a step with statistics in any
+  // default launch shape (at least 32 columns and 8 rows per CTA), or the
+  // tile kernel's
   const int strips = (p->nx + 31) / 32;
   const int runs = (p->ny + 7) / 8;
-  // shape (at least 32 columns and 8 rows per CTA), or the tile kernel's
   L.max_partials = strips * runs;
   const int tiles = tile_records(p->precision == WBLBE_FP64, p->nx, p->ny);
   if (tiles > L.max_partials) L.max_partials = tiles;
@@ -109,6 +108,7 @@ struct wblbe_ctx {
   long long* step_dev;           // step of the first step of a graph replay
   wblbe_launch launch;
   bool launch_set;               // the caller chose the strip kernel's shape
+  wblbe_launch moments;          // the default shape, of the moments pass
   int64_t steps;
   int64_t launches;
   double mass0;
@@ -333,15 +333,17 @@ wblbe_status build_graph(wblbe_ctx* h) {
 // and its statistics record (stats_out, or the handle's record).
 wblbe_status run_moments(wblbe_ctx* h, double* rho, double* ux, double* uy,
                          double* mu, double* stats_out = nullptr) {
-  const int tile = h->p.nx >= 128 ? 128 : (h->p.nx > 32 ? 64 : 32);
-  KParams kp = make_kparams(h, kMomentsRows);
+  // the strip kernel's default shape, one wave of long runs (4096^2, with the
+  // fields: FP32 16 rows per CTA 317 us, one wave 264; FP64 2304 and 2123)
+  const int tile = h->moments.tile_x, rows = h->moments.rows_per_cta;
+  KParams kp = make_kparams(h, rows);
   MomentsOut mo{rho, ux, uy, mu, h->partials};
   CU(h, launch_any(h, kModeMoments, h->buf[h->cur], nullptr, kp, mo, tile, h->stream));
   const int n = takes_tiles(h, kModeMoments)
                     ? tile_records(h->p.precision == WBLBE_FP64, h->p.nx, h->p.ny)
                 : h->p.scheme == WBLBE_STANDARD_E6
                     ? e6_partials(h->p.nx, h->p.ny)
-                    : ((h->p.nx + tile - 1) / tile) * ((h->p.ny + kMomentsRows - 1) / kMomentsRows);
+                    : ((h->p.nx + tile - 1) / tile) * ((h->p.ny + rows - 1) / rows);
   stats_finalize_kernel<<<1, 256, 0, h->stream>>>(h->partials, n,
                                                   stats_out ? stats_out : h->stats_dev);
   CU(h, cudaGetLastError());
@@ -484,6 +486,7 @@ wblbe_status wblbe_create(const wblbe_params* params, void* dev_workspace,
   h->step_dev = reinterpret_cast<long long*>(h->ws + h->L.off_step);
   h->cur = 0;
   h->launch = default_launch(*params);
+  h->moments = h->launch;
   *out = h;
   return WBLBE_OK;
 }
