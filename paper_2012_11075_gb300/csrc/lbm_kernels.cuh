@@ -1090,13 +1090,18 @@ __device__ __forceinline__ void strip_pass(const T* __restrict__ src, T* __restr
   const bool own = tx < w;
   __syncthreads();                         // a previous pass may still read smem
   const int sx = tx + kPad;                // slot of the own column
-  // Halo work: threads 0-3 take the densities of slots 2, 3 (x0-2, x0-1)
-  // and w+4, w+5 (x0+w, x0+w+1); threads mu_lo and mu_hi (warp 1 when there
-  // is one) take mu at slots 3 and w+4.  Each halo branch runs in one warp,
-  // and the two are in different warps so that no warp carries both.
-  const bool halo = tx < 4;
-  const int hs = tx < 2 ? 2 + tx : w + 2 + tx;
-  constexpr int mu_lo = TX >= 64 ? 32 : 0, mu_hi = mu_lo + 1;
+  // Halo work: four lanes of one warp take the densities of slots 2, 3 (x0-2,
+  // x0-1) and w+4, w+5 (x0+w, x0+w+1), two lanes of another the mu of slots 3
+  // and w+4.  In FP64 the two warps change with every iteration: a warp's
+  // place in its CTA decides its SM sub-partition, so a fixed warp would put
+  // the halo instructions of all resident CTAs on one FP64 pipe (23 FP64
+  // instructions a row beside 96; 4096^2 FP64: 3392 us with fixed warps, 3284
+  // us).  FP32 is not bound by issue: 2048^2 58.5 us fixed, 59.3 changing.
+  constexpr int NW = TX / 32;
+  constexpr bool kTurn = sizeof(T) == 8;
+  constexpr int mu_lo = TX >= 64 ? 32 : 0, mu_hi = mu_lo + 1;   // fixed threads
+  const int lane = kTurn ? tx & 31 : tx, wid = tx >> 5;
+  const int hs = lane < 2 ? 2 + lane : w + 2 + lane;
   const bool use_vec = GHOST || ((w == TX) && (p.nx % 4 == 0));
   // 16-byte chunks per plane row this strip needs (its columns plus 4 on
   // each side, rounded up to whole chunks; never past the stage row)
@@ -1263,6 +1268,10 @@ __device__ __forceinline__ void strip_pass(const T* __restrict__ src, T* __restr
       const int n0 = n + ph * R;           // density front, relative to kfirst
       if (live && n0 > nlast) live = false;
       if (live) {
+        const bool halo = lane < 4 && (!kTurn || wid == ph % NW);
+        const bool mu_halo =
+            kTurn ? lane < 2 && wid == (ph + NW / 2) % NW : tx == mu_lo || tx == mu_hi;
+        const int mu_slot = (kTurn ? lane == 0 : tx == mu_lo) ? 3 : w + 4;
         // slot of the row at relative offset d from this iteration's front
         // (ph * R + d, taken modulo the ring; compile-time after unrolling)
 #define WB_SLOT(d, ring) ((ph * R + (d) + 4 * (ring)) % (ring))
@@ -1350,8 +1359,8 @@ __device__ __forceinline__ void strip_pass(const T* __restrict__ src, T* __restr
               m0[sx] = mu.x;
               m1[sx] = mu.y;
             }
-            if (tx == mu_lo || tx == mu_hi) {   // halo mu at slots 3 and w+4
-              const int s = tx == mu_lo ? 3 : w + 4;
+            if (mu_halo) {                      // halo mu at slots 3 and w+4
+              const int s = mu_slot;
               const float2 mu = at2(s);
               if (WB_IN(s, SW)) {
                 m0[s] = mu.x;
@@ -1390,8 +1399,9 @@ __device__ __forceinline__ void strip_pass(const T* __restrict__ src, T* __restr
                   iso_grad12_rows(pdif_c, pdif_n, pdif_b, rn[sx], rsb[sx], psum_n, psum_b,
                                      fgx[j], fgy[j]);
               }
-              if (tx == mu_lo) mrow[3] = at(3);
-              if (tx == mu_hi && WB_IN(w + 4, SW)) mrow[w + 4] = at(w + 4);
+              if (mu_halo) {
+                if (WB_IN(mu_slot, SW)) mrow[mu_slot] = at(mu_slot);
+              }
             }
             psum_b = psum_c;
             psum_c = psum_n;
