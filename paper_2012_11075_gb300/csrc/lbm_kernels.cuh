@@ -840,15 +840,22 @@ template <> struct Staging<float> {
   static constexpr int kRows = 2;
   static constexpr int kAhead = 2;
   static constexpr int kStages = 2 + kRows + kRows * kAhead;     // 8
-  __host__ __device__ static constexpr int min_blocks(int tx) { return 640 / tx > 1 ? 640 / tx : 1; }
-  // the batched kernel (case parameters in shared memory) fits the same budget
-  __host__ __device__ static constexpr int min_blocks_batch(int tx) { return min_blocks(tx); }
+  // Five CTAs of 128 threads are resident by shared memory.  The well-balanced
+  // step gets a budget of four (93 registers, still five resident; at 86 its
+  // schedule is tighter: 4096^2 218.1 and 217.3 us, 3000^2 126.6 and 123.3,
+  // 2048^2 58.8 and 57.7), the others one of five (standard 4096^2 219.5 and,
+  // with four, 222.6; the batched kernel 105.0 and 110.5 us per step).
+  __host__ __device__ static constexpr int min_blocks(int tx, bool wb_step) {
+    const int threads = wb_step ? 512 : 640;
+    return threads / tx > 1 ? threads / tx : 1;
+  }
+  __host__ __device__ static constexpr int min_blocks_batch(int tx) { return min_blocks(tx, false); }
 };
 template <> struct Staging<double> {
   static constexpr int kRows = 1;
   static constexpr int kAhead = 1;
   static constexpr int kStages = 2 + kRows + kRows * kAhead;     // 4
-  __host__ __device__ static constexpr int min_blocks(int tx) { return 65536 / (tx * 128); }
+  __host__ __device__ static constexpr int min_blocks(int tx, bool) { return 65536 / (tx * 128); }
   __host__ __device__ static constexpr int min_blocks_batch(int tx) { return 65536 / (tx * 128); }
 };
 
@@ -1507,7 +1514,7 @@ __device__ __forceinline__ void strip_pass(const T* __restrict__ src, T* __restr
 // statistics (a step that also reduces the stats of the state it starts
 // from), write the per-CTA stats record.
 template <typename T, int SCH, int MODE, int TX>
-__global__ void __launch_bounds__(TX, Staging<T>::min_blocks(TX))
+__global__ void __launch_bounds__(TX, Staging<T>::min_blocks(TX, SCH == kSchWB && MODE == kModeStep))
     lbm_strip_kernel(const T* __restrict__ src, T* __restrict__ dst,
                      const KParams p, const MomentsOut mo) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
