@@ -262,18 +262,20 @@ __device__ __forceinline__ void textbook_pairs(T (&g)[9], T rs, T rho, T ux, T u
 // errors against 128-bit arithmetic are those of that form (populations
 // 0.8e-16 to 1.9e-16 relative, at u = 1e-2, 1e-4 and 1e-8 alike).
 // 4096^2 well-balanced step: 3.87 ms before, 3.44 ms.
-template <int SCH>
-__device__ __forceinline__ void collide12_f64(double (&g)[9], double rho, double gmx, double gmy,
-                                              double grx, double gry,
-                                              const NodeConsts<double>& q, double& ux_out,
-                                              double& uy_out) {
-  constexpr bool WB = SCH == kSchWB;
-  static_assert(WB || SCH == kSchStandard, "potential-form schemes");
+// inv = 1/rho and the momentum j come from the caller (momentum_f64).
+__device__ __forceinline__ void momentum_f64(const double (&g)[9], double& jx, double& jy) {
   const double d13 = __dadd_rn(g[1], -g[3]), d24 = __dadd_rn(g[2], -g[4]);
   const double d57 = __dadd_rn(g[5], -g[7]), d86 = __dadd_rn(g[8], -g[6]);
-  const double jx = __dadd_rn(__dadd_rn(d13, d57), d86);
-  const double jy = __dadd_rn(__dadd_rn(d24, d57), -d86);
-  const double inv = recip(rho);
+  jx = __dadd_rn(__dadd_rn(d13, d57), d86);
+  jy = __dadd_rn(__dadd_rn(d24, d57), -d86);
+}
+template <int SCH>
+__device__ __forceinline__ void collide12_f64(double (&g)[9], double rho, double jx, double jy,
+                                              double inv, double gmx, double gmy, double grx,
+                                              double gry, const NodeConsts<double>& q,
+                                              double& ux_out, double& uy_out) {
+  constexpr bool WB = SCH == kSchWB;
+  static_assert(WB || SCH == kSchStandard, "potential-form schemes");
   const double hm = __dmul_rn(rho, -1.0 / 24.0);         // F/2 = hm (12 grad mu) [+ cs^2 grad rho/2]
   double sx = __fma_rn(hm, gmx, jx), sy = __fma_rn(hm, gmy, jy);
   if (!WB) {
@@ -341,7 +343,9 @@ __device__ __forceinline__ void collide(T (&g)[9], T rs, T gmx, T gmy, T grx,
   constexpr bool kG12 = GS == 12;
   static_assert(GS == 1 || GS == 12, "gradient scale");
   if constexpr (kG12 && sizeof(T) == 8 && (SCH == kSchWB || SCH == kSchStandard)) {
-    collide12_f64<SCH>(g, rs, gmx, gmy, grx, gry, q, ux_out, uy_out);
+    T jx, jy;
+    momentum_f64(g, jx, jy);
+    collide12_f64<SCH>(g, rs, jx, jy, recip(rs), gmx, gmy, grx, gry, q, ux_out, uy_out);
     return;
   }
   const T omega = q.omega, kf = q.kf;

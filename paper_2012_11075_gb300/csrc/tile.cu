@@ -242,6 +242,119 @@ __global__ void __launch_bounds__(NT)
   chain_signal();
 }
 
+// FP64 step of the smallest lattices, at most two 8 x 4 tiles per SM.  An FP64
+// warp instruction occupies its SM sub-partition for 64 cycles however few of
+// its lanes are active, so the time is the longest warp's instruction count,
+// and the tile's arithmetic is dealt out to four warps: two hold the same 32
+// nodes and take, one after another, {rho, momentum}, {mu, grad rho and 1/rho}
+// and, after a common part, {rest and axis populations, diagonal ones}; the
+// other two take the frame (rho) and its ring (mu).  About 70 instructions on
+// the longest warp where one warp of lbm_tile_kernel has 111, but a fifth more
+// in all: us per step there and here, 4 x 256 5.1 and 3.9, 96 x 100 (2 tiles on
+// every SM) 5.3 and 4.9, 100^2 (3 on some) 5.6 and 6.2.
+template <int SCH>
+__global__ void __launch_bounds__(128)
+    lbm_tile_split_kernel(const double* __restrict__ src, double* __restrict__ dst,
+                          const KParams p) {
+  constexpr int TW = 8, TH = 4, FW = TW + 4, FH = TH + 4;
+  static_assert(TW * TH == 32 && FW * FH - 32 == 64 && (TW + 2) * (TH + 2) - 32 <= 32,
+                "a warp's nodes, two warps' frame and one warp's ring");
+  __shared__ double rho_s[FH][FW], mu_s[FH][FW];
+  __shared__ double part_s[5][32];              // jx, jy, 1/rho, 12 grad rho of each node
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int x0 = blockIdx.x * TW, y0 = blockIdx.y * TH;
+  const int nx = p.nx, ny = p.ny;
+  // frame position: the nodes (warps 0 and 1), or the two rows below and above
+  // and the two columns on each side (warps 2 and 3)
+  int fx, fy;
+  if (wid < 2) {
+    fx = 2 + lane % TW;
+    fy = 2 + lane / TW;
+  } else {
+    const int h = (wid - 2) * 32 + lane;
+    if (h < 4 * FW) {
+      fy = h / FW;
+      fx = h - fy * FW;
+      if (fy >= 2) fy += TH;
+    } else {
+      const int q = h - 4 * FW;
+      fy = 2 + (q >> 2);
+      fx = q & 3;
+      if (fx >= 2) fx += TW;
+    }
+  }
+  const int xc = wrap_index(x0 - 2 + fx, nx), yc = wrap_index(y0 - 2 + fy, ny);
+  const unsigned xw = xc == 0 ? nx - 1 : xc - 1, xe = xc == nx - 1 ? 0 : xc + 1;
+  const unsigned rb = (unsigned)((yc == 0 ? ny - 1 : yc - 1) * p.pitch);
+  const unsigned rc = (unsigned)(yc * p.pitch);
+  const unsigned ra = (unsigned)((yc == ny - 1 ? 0 : yc + 1) * p.pitch);
+  const NodeConsts<double>& cc = p.d;
+  chain_wait();
+  auto ld = [&](int i, unsigned off) {
+    return WB_IN(off, p.plane) ? (src + i * p.plane)[off] : 0.0;
+  };
+  double g[9] = {ld(0, rc + xc), ld(1, rc + xw), ld(2, rb + xc), ld(3, rc + xe), ld(4, ra + xc),
+                 ld(5, rb + xw), ld(6, rb + xe), ld(7, ra + xe), ld(8, ra + xw)};
+  if (wid == 1) {
+    double jx, jy;
+    momentum_f64(g, jx, jy);
+    part_s[0][lane] = jx;
+    part_s[1][lane] = jy;
+  } else {
+    rho_s[fy][fx] = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
+  }
+  __syncthreads();
+  if (wid == 1) {
+    const double *rn = rho_s[fy + 1], *rm = rho_s[fy], *rs = rho_s[fy - 1];
+    double gx, gy;
+    iso_grad12_rows(rm[fx + 1] - rm[fx - 1], rn[fx + 1] - rn[fx - 1], rs[fx + 1] - rs[fx - 1],
+                    rn[fx], rs[fx], rn[fx + 1] + rn[fx - 1], rs[fx + 1] + rs[fx - 1], gx, gy);
+    part_s[2][lane] = recip(rm[fx]);
+    part_s[3][lane] = gx;
+    part_s[4][lane] = gy;
+  } else if (wid == 0 || wid == 2) {
+    int x = fx, y = fy;
+    if (wid == 2) {                             // the ring: rows below and above, sides
+      const int h = lane < 2 * (TW + 2) ? lane : min(lane - 2 * (TW + 2), 2 * TH - 1);
+      if (lane < 2 * (TW + 2)) {
+        x = 1 + (h >= TW + 2 ? h - (TW + 2) : h);
+        y = h >= TW + 2 ? TH + 2 : 1;
+      } else {
+        x = (h & 1) ? TW + 2 : 1;
+        y = 2 + (h >> 1);
+      }
+    }
+    const double *rn = rho_s[y + 1], *rm = rho_s[y], *rs = rho_s[y - 1];
+    mu_s[y][x] = chem_pot(rm[x], rm[x + 1], rm[x - 1], rn[x], rs[x], rn[x + 1], rn[x - 1],
+                          rs[x + 1], rs[x - 1], cc.two_beta, cc.dl, cc.dg, cc.kappa6);
+  }
+  __syncthreads();
+  const int x = x0 - 2 + fx, y = y0 - 2 + fy;
+  if (wid < 2 && x < nx && y < ny) {
+    const double *mn = mu_s[fy + 1], *mc = mu_s[fy], *mb = mu_s[fy - 1];
+    double gmx, gmy, ux, uy;
+    iso_grad12(mc[fx + 1], mc[fx - 1], mn[fx], mb[fx], mn[fx + 1], mn[fx - 1], mb[fx + 1],
+               mb[fx - 1], gmx, gmy);
+    const double rho = rho_s[fy][fx], jx = part_s[0][lane], jy = part_s[1][lane];
+    const double inv = part_s[2][lane], grx = part_s[3][lane], gry = part_s[4][lane];
+    const unsigned off = (unsigned)(y * p.pitch + x);
+    const bool in = WB_IN(y, ny) && WB_IN(x, p.pitch);
+    // each branch keeps only what its stores need
+    if (wid == 0) {
+      collide12_f64<SCH>(g, rho, jx, jy, inv, gmx, gmy, grx, gry, cc, ux, uy);
+#pragma unroll
+      for (int i = 0; i < 5; ++i)
+        if (in) (dst + i * p.plane)[off] = g[i];
+    } else {
+      collide12_f64<SCH>(g, rho, jx, jy, inv, gmx, gmy, grx, gry, cc, ux, uy);
+#pragma unroll
+      for (int i = 5; i < 9; ++i)
+        if (in) (dst + i * p.plane)[off] = g[i];
+    }
+  }
+  chain_signal();
+}
+
 template <typename T, int SCH, int MODE, int TW, int TH, int PR, int NT>
 cudaError_t launch_shape(const void* src, void* dst, const KParams& kp, const MomentsOut& mo,
                          cudaStream_t s, bool chained) {
@@ -286,6 +399,11 @@ template <int SCH, int MODE>
 cudaError_t launch_mode_tile(bool fp64, const void* src, void* dst, const KParams& kp,
                              const MomentsOut& mo, cudaStream_t s, bool ch) {
   const int k = shape_of(fp64, kp.nx, kp.ny);
+  if (fp64 && MODE == kModeStep && k == 0 && tiles_of(kShapes64[0], kp.nx, kp.ny) <= 2 * kSMs) {
+    ChainedLaunch l(dim3((kp.nx + 7) / 8, (kp.ny + 3) / 4), 128, 0, s, ch);
+    return cudaLaunchKernelEx(&l.cfg, lbm_tile_split_kernel<SCH>, static_cast<const double*>(src),
+                              static_cast<double*>(dst), kp);
+  }
   if (fp64) {
     switch (k) {
       case 0: return launch_shape<double, SCH, MODE, 8, 4, 1, 96>(src, dst, kp, mo, s, ch);
