@@ -11,8 +11,8 @@
 // grad(phi) = 3 sum_i w_i c_i phi(x + c_i) and
 // lap(phi) = 6 sum_i w_i (phi(x + c_i) - phi(x)).
 //
-// An FP32 step is one kernel (d3_step_f32).  An FP64 step, and the moments of
-// both, are three kernels on the caller's stream (the FP64 pipe is the limit,
+// An FP32 step is two kernels (d3_density, d3_step_f32).  An FP64 step, and the
+// moments of both, are three kernels on the caller's stream (the FP64 pipe is the limit,
 // not memory traffic):
 //   d3_density:   rho(x) = sum_i P_i(x - c_i)           (pull, Eq. rhoU)
 //   d3_chem_pot:  mu = mu_0(rho) - kappa lap(rho)        (Sec. II)
@@ -138,6 +138,7 @@ template <typename T>
 __global__ void __launch_bounds__(kBlock3) d3_density(const T* __restrict__ src,
                                                       T* __restrict__ rho, const P3 p) {
   const int x = blockIdx.x * kBlock3 + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
+  chain_wait();
   if (x >= p.nx) return;
   const Nbr3 nb(p, x, y, z);
   T g[kQ3];
@@ -152,6 +153,7 @@ __global__ void __launch_bounds__(kBlock3) d3_density(const T* __restrict__ src,
     s = g[0] + moving_sum3(g);
   }
   rho[nb.at(0, 0, 0)] = s;
+  chain_signal();
 }
 
 // mu from the sums of the axis and edge neighbours' densities and the own
@@ -518,29 +520,32 @@ __global__ void __launch_bounds__(kBlock3) d3_moments(const T* __restrict__ src,
                               kStatRec);
 }
 
-// The whole FP32 step in one kernel: a CTA owns TX x TY columns and marches a
+// The FP32 step after the density: a CTA owns TX x TY columns and marches a
 // run of planes along z; a thread owns two rows of a column, whose arithmetic
 // runs on packed pairs.  Per plane, with the front plane f:
-//   A. rho of plane f over the tile and two columns around it (the nineteen
-//      pulled populations of each node), into a ring of planes;
+//   A. rho of plane f over the tile and two columns around it, read from the
+//      density field into a ring of planes (the next plane's values are
+//      requested an iteration ahead);
 //   B. mu of plane f - 1 over the tile and one column around it, into a second
-//      ring; rho and grad rho of the own nodes stay in registers;
+//      ring; rho and grad rho of the own nodes stay in registers; the
+//      populations of plane f - 2 are requested before the arithmetic;
 //   C. grad mu, the collision and the stores of plane f - 2.
-// The three kernels read the populations twice from DRAM and write and read
-// two fields, 248 bytes per update for 152 algorithmic ones; here the second
-// read of the own populations (requested before B's arithmetic) and the frame
-// come from L2.  The latency of the pulls bounds it (11 warps per SM; DRAM 46 %,
-// issue 40 % busy).  us per step in three kernels and here: 256^3 985 and 708,
-// 128^3 130 and 97, 101 x 67 x 75 42 and 37, 64^3 27 and 20.  Measured and not kept, 256^3:
-// one node per thread 782; all pulls of an iteration requested at once 844;
-// populations staged by 4-byte asynchronous copies 1178; plane addresses from
-// the constant bank 775; four resident CTAs 714, 32 x 16 tiles 728.
+// With the density kernel a step moves 236 bytes per update at DRAM speed
+// (256^3: 94 % of the measured copy bandwidth; 152 algorithmic).  us per step
+// of the three kernels before and of the two, well-balanced: 256^3 985 and 633,
+// 192^3 463 and 283, 128^3 130 and 90, 101 x 67 x 75 42 and 29, 64^3 27 and
+// 16.5.  Measured and not kept, 256^3: the density formed here too, from the
+// populations of the tile and its frame (152 bytes from DRAM, the rest from
+// L2; bound by the latency of its pulls), 716; the same with one node per
+// thread 782, with all pulls of an iteration at once 844, with populations
+// staged by 4-byte asynchronous copies 1178; three resident CTAs 663, five 689.
 constexpr int kTX3 = 32, kTY3 = 8, kNT3 = kTX3 * kTY3 / 2;
-constexpr int kMinB3 = 3;          // resident CTAs (164 registers)
+constexpr int kMinB3 = 4;          // resident CTAs (128 registers)
 
 template <bool WB>
 __global__ void __launch_bounds__(kNT3, kMinB3)
-    d3_step_f32(const float* __restrict__ src, float* __restrict__ dst, const P3 p, int run) {
+    d3_step_f32(const float* __restrict__ src, float* __restrict__ dst,
+                const float* __restrict__ rho, const P3 p, int run) {
   constexpr int TX = kTX3, TY = kTY3;
   constexpr int FW = TX + 4, FH = TY + 4, MW = TX + 2, MH = TY + 2;
   __shared__ float rho_s[4][FH][FW];           // [f & 3][2 + y][2 + x]
@@ -613,21 +618,22 @@ __global__ void __launch_bounds__(kNT3, kMinB3)
   const bool mine_a = x0 + tx < p.nx && y0 + ty < p.ny, mine_b = mine_a && y0 + ty + 1 < p.ny;
   const float2 zero = make_float2(0.f, 0.f);
   float2 prs = zero, pgx = zero, pgy = zero, pgz = zero;   // rho - rho_ref, 12 grad rho of f - 2
+  auto ld2 = [&](const Col& c, unsigned z) {
+    return make_float2(rho[z + c.y[1] + c.x[1]], rho[z + c.y[2] + c.x[1]]);
+  };
+  float2 nr = ld2(own, zc), nh = has_frame ? ld2(frame, zc) : zero;
   for (; f < z1 + 2; ++f) {
     const int c = f - 2;                        // the plane to collide
     const bool upd = mine_a && c >= z0;
-    {
-      float2 a[19];
-      pull(a, own, zm1, zc, zp);
-      const float2 r = add2(a[0], moving_sum3_x2(a));
-      rho_s[f & 3][2 + ty][2 + tx] = r.x;
-      rho_s[f & 3][3 + ty][2 + tx] = r.y;
-      if (has_frame) {
-        pull(a, frame, zm1, zc, zp);
-        const float2 v = add2(a[0], moving_sum3_x2(a));
-        rho_s[f & 3][hy][hx] = v.x;
-        rho_s[f & 3][hy + 1][hx] = v.y;
-      }
+    rho_s[f & 3][2 + ty][2 + tx] = nr.x;
+    rho_s[f & 3][3 + ty][2 + tx] = nr.y;
+    if (has_frame) {
+      rho_s[f & 3][hy][hx] = nh.x;
+      rho_s[f & 3][hy + 1][hx] = nh.y;
+    }
+    if (f + 1 < z1 + 2) {
+      nr = ld2(own, zp);
+      if (has_frame) nh = ld2(frame, zp);
     }
     __syncthreads();
     float2 g[19];
@@ -856,10 +862,10 @@ void pass3_typed(wblbe3_ctx* h, bool moments, const Out3& out, const P3& q, dim3
   }
 }
 
-// Planes per CTA of the fused FP32 step: the run whose waves of resident CTAs
+// Planes per CTA of the FP32 step kernel: the run whose waves of resident CTAs
 // take the fewest plane iterations in all (a run of n planes takes n + 4, of
 // which the first four store nothing).
-int fused_run(const wblbe3_ctx* h) {
+int step_run(const wblbe3_ctx* h) {
   const long long tiles = (long long)((h->p.nx + kTX3 - 1) / kTX3) * ((h->p.ny + kTY3 - 1) / kTY3);
   const long long resident = 152LL * kMinB3;
   int best = h->p.nz;
@@ -876,23 +882,27 @@ int fused_run(const wblbe3_ctx* h) {
   return best;
 }
 
-cudaError_t fused_step(wblbe3_ctx* h, const P3& q) {
-  const int run = fused_run(h);
+cudaError_t fp32_step(wblbe3_ctx* h, const P3& q) {
+  const int run = step_run(h);
   ChainedLaunch l(dim3((h->p.nx + kTX3 - 1) / kTX3, (h->p.ny + kTY3 - 1) / kTY3,
                        (h->p.nz + run - 1) / run),
                   kNT3, 0, h->stream, true);
   const float* src = static_cast<const float*>(h->buf[h->cur]);
   float* dst = static_cast<float*>(h->buf[1 - h->cur]);
+  float* rho = static_cast<float*>(h->rho);
+  ChainedLaunch d(grid3(h), kBlock3, 0, h->stream, true);
+  const cudaError_t e = cudaLaunchKernelEx(&d.cfg, d3_density<float>, src, rho, q);
+  if (e != cudaSuccess) return e;
   return h->p.scheme == WBLBE_WELL_BALANCED
-             ? cudaLaunchKernelEx(&l.cfg, d3_step_f32<true>, src, dst, q, run)
-             : cudaLaunchKernelEx(&l.cfg, d3_step_f32<false>, src, dst, q, run);
+             ? cudaLaunchKernelEx(&l.cfg, d3_step_f32<true>, src, dst, (const float*)rho, q, run)
+             : cudaLaunchKernelEx(&l.cfg, d3_step_f32<false>, src, dst, (const float*)rho, q, run);
 }
 
 wblbe_status pass3(wblbe3_ctx* h, bool moments, const Out3& out) {
   const P3 q = p3_of(h);
   if (!moments && h->p.precision == WBLBE_FP32_SHIFTED) {
-    CU3(h, fused_step(h, q));
-    h->launches += 1;
+    CU3(h, fp32_step(h, q));
+    h->launches += 2;
     return WBLBE_OK;
   }
   const dim3 g = grid3(h);

@@ -245,8 +245,8 @@ def test_d3q19_fp32_droplet_follows_fp64():
 @pytest.mark.parametrize("scheme", [wblbe.STANDARD, wblbe.WELL_BALANCED])
 @pytest.mark.parametrize("shape", [(1, 1, 1), (2, 3, 5), (9, 8, 32), (3, 9, 33), (40, 7, 31),
                                    (5, 17, 65)])
-def test_d3q19_fp32_one_kernel_step_at_tile_edges(shape, scheme):
-    """The one-kernel FP32 step (32 x 8 columns, pairs of rows, runs of
+def test_d3q19_fp32_marching_step_at_tile_edges(shape, scheme):
+    """The marching FP32 step kernel (32 x 8 columns, pairs of rows, runs of
     planes) at lattices smaller than its frame and one node around its tile:
     5 steps against FP64.  Populations are O(1), so the float storage and
     arithmetic of 5 steps stay within 40 ulps of 1 (2^-24 each)."""
