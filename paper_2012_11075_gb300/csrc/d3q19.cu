@@ -183,6 +183,7 @@ template <typename T>
 __global__ void __launch_bounds__(kBlock3) d3_chem_pot(const T* __restrict__ rho,
                                                        T* __restrict__ mu, const P3 p) {
   const int x = blockIdx.x * kBlock3 + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
+  chain_wait();
   if (x >= p.nx) return;
   const Nbr3 nb(p, x, y, z);
   // sums of the axis and edge neighbours, then the centre's share taken off
@@ -195,6 +196,7 @@ __global__ void __launch_bounds__(kBlock3) d3_chem_pot(const T* __restrict__ rho
     if (i < 7) ax += nbr(i); else ed += nbr(i);
   }
   mu[nb.at(0, 0, 0)] = mu3(ax, ed, rho[nb.at(0, 0, 0)], consts3(p, T(0)));
+  chain_signal();
 }
 
 // 12 grad(phi) from v(dx, dy, dz) = phi(x + (dx, dy, dz)); see grad3x12.
@@ -480,6 +482,7 @@ __global__ void __launch_bounds__(kBlock3) d3_collide(const double* __restrict__
                                                       const double* __restrict__ rho,
                                                       const double* __restrict__ mu, const P3 p) {
   const int x = blockIdx.x * kBlock3 + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
+  chain_wait();
   if (x >= p.nx) return;
   const Nbr3 nb(p, x, y, z);
   Node3<double, WB> n(src, rho, mu, p, nb);
@@ -487,6 +490,7 @@ __global__ void __launch_bounds__(kBlock3) d3_collide(const double* __restrict__
   const unsigned k = nb.at(0, 0, 0);
 #pragma unroll
   for (int i = 0; i < kQ3; ++i) (dst + i * p.plane)[k] = n.g[i];
+  chain_signal();
 }
 
 // Fields and statistics of kMomPlanes3 planes per CTA: one record for all of
@@ -501,6 +505,7 @@ __global__ void __launch_bounds__(kBlock3) d3_moments(const T* __restrict__ src,
   const int x = blockIdx.x * kBlock3 + threadIdx.x, y = blockIdx.y;
   const int z0 = blockIdx.z * kMomPlanes3, z1 = min(z0 + kMomPlanes3, p.nz);
   StatsAcc<T> acc;
+  chain_wait();
   for (int z = z0; z < z1 && x < p.nx; ++z) {
     const Nbr3 nb(p, x, y, z);
     const Node3<T, WB> n(src, rho, mu, p, nb);
@@ -844,22 +849,31 @@ double shift3(const wblbe3_params& p, int i) {
   return i == 0 ? rr - (1.0 - w3(0)) * p.rho0 : w3(i) * p.rho0;
 }
 
+// A kernel chained to the stream's previous one (see ChainedLaunch).
+template <typename... K, typename... A>
+cudaError_t launch3(void (*kernel)(K...), dim3 grid, int block, cudaStream_t s, A... args) {
+  ChainedLaunch l(grid, block, 0, s, true);
+  return cudaLaunchKernelEx(&l.cfg, kernel, static_cast<K>(args)...);
+}
+
 // Density and chemical potential of the current state, then the moments
 // (fields and statistics), or in FP64 the collision into the other buffer.
 template <typename T, bool WB>
-void pass3_typed(wblbe3_ctx* h, bool moments, const Out3& out, const P3& q, dim3 g) {
+cudaError_t pass3_typed(wblbe3_ctx* h, bool moments, const Out3& out, const P3& q, dim3 g) {
   const T* src = static_cast<const T*>(h->buf[h->cur]);
   T* rho = static_cast<T*>(h->rho);
   T* mu = static_cast<T*>(h->mu);
-  d3_density<T><<<g, kBlock3, 0, h->stream>>>(src, rho, q);
-  d3_chem_pot<T><<<g, kBlock3, 0, h->stream>>>(rho, mu, q);
+  cudaError_t e = launch3(d3_density<T>, g, kBlock3, h->stream, src, rho, q);
+  if (e == cudaSuccess) e = launch3(d3_chem_pot<T>, g, kBlock3, h->stream, rho, mu, q);
+  if (e != cudaSuccess) return e;
   if (moments) {
     const dim3 gm(g.x, g.y, (h->p.nz + kMomPlanes3 - 1) / kMomPlanes3);
-    d3_moments<T, WB><<<gm, kBlock3, 0, h->stream>>>(src, rho, mu, q, out);
-  } else if constexpr (sizeof(T) == 8) {
-    d3_collide<WB><<<g, kBlock3, 0, h->stream>>>(src, static_cast<T*>(h->buf[1 - h->cur]), rho, mu,
-                                                 q);
+    return launch3(d3_moments<T, WB>, gm, kBlock3, h->stream, src, rho, mu, q, out);
   }
+  if constexpr (sizeof(T) == 8)
+    return launch3(d3_collide<WB>, g, kBlock3, h->stream, src,
+                   static_cast<T*>(h->buf[1 - h->cur]), rho, mu, q);
+  return cudaErrorInvalidValue;              // FP32 steps: fp32_step
 }
 
 // Planes per CTA of the FP32 step kernel: the run whose waves of resident CTAs
@@ -884,18 +898,16 @@ int step_run(const wblbe3_ctx* h) {
 
 cudaError_t fp32_step(wblbe3_ctx* h, const P3& q) {
   const int run = step_run(h);
-  ChainedLaunch l(dim3((h->p.nx + kTX3 - 1) / kTX3, (h->p.ny + kTY3 - 1) / kTY3,
-                       (h->p.nz + run - 1) / run),
-                  kNT3, 0, h->stream, true);
+  const dim3 grid((h->p.nx + kTX3 - 1) / kTX3, (h->p.ny + kTY3 - 1) / kTY3,
+                  (h->p.nz + run - 1) / run);
   const float* src = static_cast<const float*>(h->buf[h->cur]);
   float* dst = static_cast<float*>(h->buf[1 - h->cur]);
   float* rho = static_cast<float*>(h->rho);
-  ChainedLaunch d(grid3(h), kBlock3, 0, h->stream, true);
-  const cudaError_t e = cudaLaunchKernelEx(&d.cfg, d3_density<float>, src, rho, q);
+  const cudaError_t e = launch3(d3_density<float>, grid3(h), kBlock3, h->stream, src, rho, q);
   if (e != cudaSuccess) return e;
   return h->p.scheme == WBLBE_WELL_BALANCED
-             ? cudaLaunchKernelEx(&l.cfg, d3_step_f32<true>, src, dst, (const float*)rho, q, run)
-             : cudaLaunchKernelEx(&l.cfg, d3_step_f32<false>, src, dst, (const float*)rho, q, run);
+             ? launch3(d3_step_f32<true>, grid, kNT3, h->stream, src, dst, rho, q, run)
+             : launch3(d3_step_f32<false>, grid, kNT3, h->stream, src, dst, rho, q, run);
 }
 
 wblbe_status pass3(wblbe3_ctx* h, bool moments, const Out3& out) {
@@ -907,13 +919,11 @@ wblbe_status pass3(wblbe3_ctx* h, bool moments, const Out3& out) {
   }
   const dim3 g = grid3(h);
   const bool wb = h->p.scheme == WBLBE_WELL_BALANCED;
-  if (h->p.precision == WBLBE_FP64)
-    wb ? pass3_typed<double, true>(h, moments, out, q, g)
-       : pass3_typed<double, false>(h, moments, out, q, g);
-  else
-    wb ? pass3_typed<float, true>(h, moments, out, q, g)
-       : pass3_typed<float, false>(h, moments, out, q, g);
-  CU3(h, cudaGetLastError());
+  CU3(h, h->p.precision == WBLBE_FP64
+             ? (wb ? pass3_typed<double, true>(h, moments, out, q, g)
+                   : pass3_typed<double, false>(h, moments, out, q, g))
+             : (wb ? pass3_typed<float, true>(h, moments, out, q, g)
+                   : pass3_typed<float, false>(h, moments, out, q, g)));
   h->launches += 3;
   return WBLBE_OK;
 }
