@@ -45,12 +45,12 @@ BYTES_PER_LU = {"f32": 72, "f64": 144}          # 9 reads + 9 writes per node up
 SUBSTEPS = {"f32": 200, "f64": 40}              # lattice steps per benchmark step
 # FP64 flops per lattice update of the FP64 step kernel, from the ncu
 # instruction mix (2 x DFMA + DADD + DMUL per node, halo work included;
-# 2048^2 well-balanced case: DADD 41.5, DMUL 21.2, DFMA 48.75)
-FP64_FLOPS_PER_LU = 160.3
+# 2048^2 well-balanced case: DADD 41.5, DMUL 16.2, DFMA 40.2)
+FP64_FLOPS_PER_LU = 138.1
 # FP64 flops per lattice update of the three D3Q19 kernels (density 18 DADD;
-# chemical potential 19 DADD + 4 DMUL + 4 DFMA; collide 78 DADD + 32 DMUL +
-# 81 DFMA; ncu op mix on a 128^3 droplet, one thread per node, no halo work)
-D3_FLOPS_PER_LU = 321.0
+# chemical potential 19 DADD + 4 DMUL + 4 DFMA; collide 71 DADD + 18 DMUL +
+# 72 DFMA; ncu op mix on a 128^3 droplet, one thread per node, no halo work)
+D3_FLOPS_PER_LU = 282.0
 # oldest state (lattice steps since initialisation) a timed step may start
 # from; see time_device
 MAX_STATE_AGE = 1200
@@ -563,10 +563,10 @@ def run_d3q19(args, stream, torch, fp64_peak=None):
     lattice with one droplet of radius n/4 (rho_l = 1, rho_g = 0.1,
     kappa = 0.01, W = 4, tau = 1.0); K benchmark steps of S lattice steps,
     timed by CUDA events on the launching stream, in FP64 and in
-    FP32-shifted storage.  Three kernels per step (density, chemical
+    FP32-shifted storage.  FP64: three kernels per step (density, chemical
     potential, collide-stream); algorithmic bytes per update 19 populations
     read and written (304 in FP64, 152 in FP32); the kernels move about
-    496 / 248 (the density and chemical-potential fields, and the
+    496 / 236 (the density and chemical-potential fields, and the
     populations read twice)."""
     from paper_2012_11075_gb300 import wblbe
     from paper_2012_11075_gb300 import workloads as wl
@@ -622,7 +622,7 @@ def run_d3q19(args, stream, torch, fp64_peak=None):
                      "roofline": {"bound": "hbm", "achieved": 152 * l32 / 1e9, "peak": peak,
                                   "unit": "GB/s", "frac": 152 * l32 / 1e9 / peak,
                                   "peak_source": "of measured"},
-                     "hbm_frac_moved": 248 * l32 / 1e9 / peak,
+                     "hbm_frac_moved": 236 * l32 / 1e9 / peak,
                      "umax": st32["umax"], "mass_drift_rel": st32["mass_drift_rel"],
                      "nonfinite": bool(st32["nonfinite"])}}
 

@@ -449,7 +449,8 @@ wblbe_status wblbe3_create(const wblbe3_params* params, void* dev_workspace,
 /* u = 0, f = f^eq(rho, 0); rho [nz][ny][nx] on the host or device. */
 wblbe_status wblbe3_init_rho(wblbe3_handle h, const double* rho,
                              int32_t rho_on_device);
-/* Advance nsteps steps (three kernels per step; asynchronous). */
+/* Advance nsteps steps (FP64: three kernels per step, FP32: two;
+ * asynchronous). */
 wblbe_status wblbe3_step(wblbe3_handle h, int64_t nsteps);
 /* rho, u ([3][nz][ny][nx]), mu (each may be NULL) and the stats of the
  * current state.  Synchronises. */
