@@ -143,7 +143,7 @@ int e6_partials(int nx, int ny);
 // Tile kernel of small and medium lattices, schemes 0 and 1 (tile.cu): whether
 // a lattice takes it, the per-CTA records its statistics modes write (0: it
 // does not take it), and the launch.
-bool tile_path(int sch, bool fp64, int nx, int ny);
+bool tile_path(int sch, bool fp64, int mode, int nx, int ny);
 int tile_records(bool fp64, int nx, int ny);
 cudaError_t launch_tile(int sch, bool fp64, int mode, const void* src, void* dst,
                         const KParams& kp, const MomentsOut& mo, cudaStream_t s, bool chained);

@@ -14,7 +14,7 @@
 // again in every tile (0.56 to 1.5 times the tile's densities).  The chain of
 // phases, not the traffic, bounds it up to about 256^2.  us per step with the
 // strip kernel and here: FP64 4 x 256 48.9 and 5.1, 100^2 49.2 and 5.7, 256^2
-// 51.2 and 18.2; FP32 100^2 8.1 and 2.0, 256^2 7.5 and 2.8, 512^2 8.7 and 5.4,
+// 51.2 and 17.4; FP32 100^2 8.1 and 2.0, 256^2 7.5 and 2.8, 512^2 8.7 and 5.4,
 // 1023 x 771 19.9 and 12.0, 1024^2 18.3 and 14.3.  Each node goes through the same device functions in
 // the same order as in the strip kernel, so the result is the same bit for
 // bit.
@@ -27,11 +27,24 @@ namespace wblbe {
 
 namespace {
 
+// Resident CTAs the register budget must allow (0: left to the compiler).  Left
+// alone the FP64 pair of rows gets 80 registers; asked for four CTAs it gets 98
+// to 102, and the fewer resident warps wait less for the FP64 pipe than the
+// shorter live ranges cost; us per step before and after: well-balanced 256^2
+// 18.2 and 17.4, 512^2 59.2 and 56.9, 1023 x 771 173.8 and 166.9, standard
+// 18.9 and 17.5, 61.7 and 57.3, 181.5 and 168.0.  (1 gives the same code; 6, 80
+// registers again, 17.8.)  The FP32 shapes are faster as they are: 1024^2 15.2,
+// with 1 15.9.
+template <typename T, int PR>
+constexpr int min_ctas() {
+  return sizeof(T) == 8 && PR == 2 ? 4 : 0;
+}
+
 // A thread owns PR nodes of one column (rows ty * PR ..); the TW * TH / PR
 // owners come first, and the other threads of the CTA (if any) start on the
 // frame, whose work would otherwise follow the owners' own.
 template <typename T, int SCH, int MODE, int TW, int TH, int PR, int NT>
-__global__ void __launch_bounds__(NT)
+__global__ void __launch_bounds__(NT, min_ctas<T, PR>())
     lbm_tile_kernel(const T* __restrict__ src, T* __restrict__ dst, const KParams p,
                     const MomentsOut mo) {
   static_assert(SCH == kSchStandard || SCH == kSchWB, "potential-form schemes");
@@ -370,8 +383,8 @@ cudaError_t launch_shape(const void* src, void* dst, const KParams& kp, const Mo
 //                         other warps (4 x 256: 5.1, 16 x 8 5.9; 100^2: 5.7
 //                         and 6.0; 128^2, 512 tiles: 6.5 and 6.0)
 //         16 x 8, 1, 256  up to one tile per SM (128^2: 6.0, 16 x 16 10.7)
-//         16 x 16, 2, 128 the rest: row sums shared by two rows (256^2: 18.2,
-//                         16 x 8 18.6; 512^2: 59.2 and 60.8, 32 x 16 66.9)
+//         16 x 16, 2, 128 the rest: row sums shared by two rows (256^2: 17.4,
+//                         16 x 8 18.6; 512^2: 56.9 and 60.8, 32 x 16 66.9)
 //   FP32  16 x 8, 2, 192  up to three tiles per SM (128^2: 2.2, 32 x 16 2.7;
 //                         256^2, 512 tiles: both 2.8)
 //         32 x 16, 2, 256 the rest (512^2: 5.4, 16 x 8 6.3; 1024^2 14.3 and
@@ -381,9 +394,11 @@ constexpr long long kSMs = 152, kAny = 1LL << 40;
 constexpr Shape kShapes64[] = {{8, 4, 380}, {16, 8, kSMs}, {16, 16, kAny}};
 constexpr Shape kShapes32[] = {{16, 8, 3 * kSMs}, {32, 16, kAny}};
 // Above these many nodes the strip kernel reads less and is faster: FP64
-// 1500^2 490 us per step here and 492 there, 2048^2 894 and 865; FP32 1500^2
-// 35.8 and 38.3, 2048^2 62.6 and 58.4.
-constexpr long long kMaxNodes64 = 2250000, kMaxNodes32 = 3000000;
+// 1600 x 1500 486 us per step here and 531 there, 1900^2 734 and 743, 2048^2
+// 844 and 833; FP32 1500^2 35.8 and 38.3, 2048^2 62.6 and 58.4.  The FP64 passes
+// that reduce statistics change over earlier (kMaxStats64; steps of 1900^2 with
+// them 983 here and 846 there).
+constexpr long long kMaxNodes64 = 3610000, kMaxStats64 = 2250000, kMaxNodes32 = 3000000;
 
 long long tiles_of(const Shape& s, int nx, int ny) {
   return (long long)((nx + s.tw - 1) / s.tw) * ((ny + s.th - 1) / s.th);
@@ -429,13 +444,14 @@ cudaError_t launch_scheme_tile(bool fp64, int mode, const void* src, void* dst, 
 
 }  // namespace
 
-bool tile_path(int sch, bool fp64, int nx, int ny) {
-  return (sch == kSchStandard || sch == kSchWB) &&
-         (long long)nx * ny <= (fp64 ? kMaxNodes64 : kMaxNodes32) && (ny + 3) / 4 <= 65535;
+bool tile_path(int sch, bool fp64, int mode, int nx, int ny) {
+  const long long most = !fp64 ? kMaxNodes32 : mode == kModeStep ? kMaxNodes64 : kMaxStats64;
+  return (sch == kSchStandard || sch == kSchWB) && (long long)nx * ny <= most &&
+         (ny + 3) / 4 <= 65535;
 }
 
 int tile_records(bool fp64, int nx, int ny) {
-  if (!tile_path(kSchWB, fp64, nx, ny)) return 0;
+  if (!tile_path(kSchWB, fp64, kModeStepStats, nx, ny)) return 0;
   return (int)tiles_of((fp64 ? kShapes64 : kShapes32)[shape_of(fp64, nx, ny)], nx, ny);
 }
 

@@ -252,7 +252,7 @@ wblbe_launch default_launch(const wblbe_params& p) {
 // strip kernel.
 bool takes_tiles(const wblbe_ctx* h, int mode) {
   return (mode == kModeMoments || !h->launch_set) &&
-         tile_path(h->p.scheme, h->p.precision == WBLBE_FP64, h->p.nx, h->p.ny);
+         tile_path(h->p.scheme, h->p.precision == WBLBE_FP64, mode, h->p.nx, h->p.ny);
 }
 
 // mode: kModeStep, kModeMoments or kModeStepStats (see StripMode); chained:
