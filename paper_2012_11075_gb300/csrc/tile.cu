@@ -395,10 +395,14 @@ constexpr Shape kShapes64[] = {{8, 4, 380}, {16, 8, kSMs}, {16, 16, kAny}};
 constexpr Shape kShapes32[] = {{16, 8, 3 * kSMs}, {32, 16, kAny}};
 // Above these many nodes the strip kernel reads less and is faster: FP64
 // 1600 x 1500 486 us per step here and 531 there, 1900^2 734 and 743, 2048^2
-// 844 and 833; FP32 1500^2 35.8 and 38.3, 2048^2 62.6 and 58.4.  The FP64 passes
-// that reduce statistics change over earlier (kMaxStats64; steps of 1900^2 with
-// them 983 here and 846 there).
-constexpr long long kMaxNodes64 = 3610000, kMaxStats64 = 2250000, kMaxNodes32 = 3000000;
+// 844 and 833; FP32 1500^2 35.8 and 38.3, 2048^2 62.6 and 58.4.
+constexpr long long kMaxNodes64 = 3610000, kMaxNodes32 = 3000000;
+// The passes that reduce statistics change over earlier: one CTA sums the
+// records, one per tile here and one per run of rows there.  us here and there,
+// read back: FP64 step with statistics 1023 x 771 241 and 250, 1100^2 353 and
+// 352, 1500^2 628 and 551; moments 1100^2 258 and 237, 1500^2 446 and 359; FP32
+// moments 1000 x 900 60 and 54, step 53 and 52, 1500^2 100 and 74, 98 and 77.
+constexpr long long kMaxStats64 = 1200000, kMaxStats32 = 800000;
 
 long long tiles_of(const Shape& s, int nx, int ny) {
   return (long long)((nx + s.tw - 1) / s.tw) * ((ny + s.th - 1) / s.th);
@@ -445,7 +449,9 @@ cudaError_t launch_scheme_tile(bool fp64, int mode, const void* src, void* dst, 
 }  // namespace
 
 bool tile_path(int sch, bool fp64, int mode, int nx, int ny) {
-  const long long most = !fp64 ? kMaxNodes32 : mode == kModeStep ? kMaxNodes64 : kMaxStats64;
+  const bool step = mode == kModeStep;
+  const long long most = fp64 ? (step ? kMaxNodes64 : kMaxStats64)
+                              : (step ? kMaxNodes32 : kMaxStats32);
   return (sch == kSchStandard || sch == kSchWB) && (long long)nx * ny <= most &&
          (ny + 3) / 4 <= 65535;
 }

@@ -58,3 +58,23 @@ def test_tile_kernel_equals_strip_kernel_bitwise(scheme, precision):
         tol = nx * ny * 2.0 ** -52
         assert sa["mass"] == pytest.approx(sb["mass"], rel=tol)
         assert sa["kinetic"] == pytest.approx(sb["kinetic"], rel=tol, abs=1e-300)
+
+
+@pytest.mark.parametrize("scheme", [wblbe.STANDARD, wblbe.WELL_BALANCED])
+@pytest.mark.parametrize("precision,nx,ny", [(wblbe.FP64, 1201, 1001),
+                                             (wblbe.FP32_SHIFTED, 901, 889)])
+def test_steps_on_tiles_with_statistics_on_strips(scheme, precision, nx, ny):
+    # just above the node count at which passes with statistics leave the tiles
+    rng = np.random.default_rng(nx)
+    rho = 0.6 + 0.3 * rng.uniform(-1, 1, (ny, nx))
+    runs = []
+    for strip in (False, True):
+        s = _solver(nx, ny, scheme, precision, strip)
+        s.init_rho(rho)
+        code, done, st = s.run_until_equilibrium(0.0, 7, 3)
+        runs.append((s.get_populations(), s.moments()[0], code, done, st))
+        s.close()
+    (fa, ma, ca, da, sa), (fb, mb, cb, db, sb) = runs
+    assert np.array_equal(fa, fb) and (ca, da, sa) == (cb, db, sb)
+    for k in ("rho", "ux", "uy", "mu"):
+        assert np.array_equal(ma[k], mb[k]), k
