@@ -433,7 +433,9 @@ const char* wblbe_slabs_last_error(wblbe_slabs_handle h);
 typedef struct wblbe3_ctx* wblbe3_handle;
 
 typedef struct {
-  int32_t nx, ny, nz;              /* ny, nz <= 65535                      */
+  int32_t nx, ny, nz;              /* ny, nz <= 65535; a plane (nx rounded
+                                    * up to 16, times ny nz) has fewer than
+                                    * 2^32 - 127 elements                  */
   double tau, kappa, beta, rho_l, rho_g;
   double rho0;                     /* Eq. mFeq; well-balanced scheme only  */
   int32_t scheme;                  /* WBLBE_STANDARD | WBLBE_WELL_BALANCED */

@@ -29,6 +29,7 @@
 
 #include <cmath>
 #include <cstdarg>
+#include <cstdint>
 #include <cstdio>
 #include <new>
 
@@ -43,6 +44,7 @@ namespace {
 constexpr int kQ3 = 19;
 constexpr int kBlock3 = 128;
 constexpr size_t kAlign3 = 256;
+constexpr long long kMaxPlane3 = (1LL << 32) - kBlock3;   // elements of a population plane
 
 // D3Q19 in the order rest, 6 axis (+x, -x, +y, -y, +z, -z), 12 edges in
 // opposite pairs ((1,1,0), (-1,-1,0)), ((1,-1,0), (-1,1,0)), ((1,0,1),
@@ -111,7 +113,7 @@ __device__ __forceinline__ long long at3(const P3& p, int x, int y, int z) {
 }
 
 // Element offsets of a node's wrapped neighbour columns, rows and planes
-// (below, own, above): 32 bits, a plane has fewer than 2^32 elements.
+// (below, own, above): 32 bits, a plane has at most kMaxPlane3 elements.
 struct Nbr3 {
   unsigned x[3], y[3], z[3];
   __device__ __forceinline__ Nbr3(const P3& p, int xx, int yy, int zz) {
@@ -802,9 +804,12 @@ bool params3_valid(const wblbe3_params* p, char* why, size_t n) {
   if (p->precision != WBLBE_FP64 && p->precision != WBLBE_FP32_SHIFTED) {
     snprintf(why, n, "unknown precision %d", p->precision); return false;
   }
-  if ((long long)((p->nx + 15) / 16 * 16) * p->ny * p->nz >= (1LL << 40) ||
-      p->ny > 65535 || p->nz > 65535) {
-    snprintf(why, n, "lattice too large (ny, nz <= 65535)"); return false;
+  // the kernels' element offsets within a plane, and the node numbers of the
+  // last block, are 32 bits (Nbr3, node_of)
+  if (p->ny > 65535 || p->nz > 65535 || p->nx > INT32_MAX - 15 ||
+      (long long)((p->nx + 15) / 16 * 16) * p->ny > kMaxPlane3 / p->nz) {
+    snprintf(why, n, "lattice too large (ny, nz <= 65535, fewer than 2^32 elements in a plane)");
+    return false;
   }
   return true;
 }
