@@ -160,8 +160,7 @@ __device__ __forceinline__ bool node_of(const P3& p, int& x, int& y, int& z) {
 // mirror-symmetric moving sum (the collision repeats that sum for the exact
 // mass balance).
 template <typename T, bool FLAT>
-__global__ void __launch_bounds__(kBlock3) d3_density(const T* __restrict__ src,
-                                                      T* __restrict__ rho, const P3 p) {
+__global__ void __launch_bounds__(kBlock3) d3_density(const T* src, T* rho, const P3 p) {
   int x, y, z;
   const bool on = node_of<FLAT>(p, x, y, z);
   chain_wait();
@@ -206,8 +205,7 @@ __device__ __forceinline__ float mu3(float ax, float ed, float c, const NodeCons
 // The field holds rho - rho_ref (rho_ref = 0 in FP64), which the Laplacian
 // does not see and a, b take up through dl = rho_ref - rho_l, dg.
 template <typename T, bool FLAT>
-__global__ void __launch_bounds__(kBlock3) d3_chem_pot(const T* __restrict__ rho,
-                                                       T* __restrict__ mu, const P3 p) {
+__global__ void __launch_bounds__(kBlock3) d3_chem_pot(const T* rho, T* mu, const P3 p) {
   int x, y, z;
   const bool on = node_of<FLAT>(p, x, y, z);
   chain_wait();
@@ -215,7 +213,7 @@ __global__ void __launch_bounds__(kBlock3) d3_chem_pot(const T* __restrict__ rho
   const Nbr3 nb(p, x, y, z);
   // sums of the axis and edge neighbours, then the centre's share taken off
   // once per sum (rather than from every neighbour): 6 (ax/18 + ed/36)
-  auto nbr = [&](int i) { return __ldg(rho + nb.at(cx3(i), cy3(i), cz3(i))); };
+  auto nbr = [&](int i) { return rho[nb.at(cx3(i), cy3(i), cz3(i))]; };
   T ax = nbr(1), ed = nbr(7);
 #pragma unroll
   for (int i = 2; i < kQ3; ++i) {
@@ -242,9 +240,8 @@ __device__ __forceinline__ void grad3_sums(const V& v, T& gx, T& gy, T& gz) {
 // (edge differences); the factor 1/12 is folded into the constants that
 // use the gradients.
 template <typename T>
-__device__ __forceinline__ void grad3x12(const T* __restrict__ phi, const Nbr3& nb, T& gx, T& gy,
-                                         T& gz) {
-  grad3_sums<T>([&](int dx, int dy, int dz) { return __ldg(phi + nb.at(dx, dy, dz)); }, gx, gy, gz);
+__device__ __forceinline__ void grad3x12(const T* phi, const Nbr3& nb, T& gx, T& gy, T& gz) {
+  grad3_sums<T>([&](int dx, int dy, int dz) { return phi[nb.at(dx, dy, dz)]; }, gx, gy, gz);
 }
 
 // One component of u = (j + F/2) / rho (Eq. rhoU) from 12 grad mu and 12 grad
@@ -485,8 +482,8 @@ __device__ __forceinline__ void update3_f64(double (&g)[19], double r, double gm
 template <typename T, bool WB>
 struct Node3 {
   T g[kQ3], rs, r, gmx, gmy, gmz, grx, gry, grz, ux, uy, uz;
-  __device__ __forceinline__ Node3(const T* __restrict__ src, const T* __restrict__ rho,
-                                   const T* __restrict__ mu, const P3& p, const Nbr3& nb) {
+  __device__ __forceinline__ Node3(const T* src, const T* rho, const T* mu, const P3& p,
+                                   const Nbr3& nb) {
 #pragma unroll
     for (int i = 0; i < kQ3; ++i) g[i] = (src + i * p.plane)[nb.at(-cx3(i), -cy3(i), -cz3(i))];
     rs = rho[nb.at(0, 0, 0)];                  // rho - rho_ref (rho in FP64)
@@ -504,10 +501,9 @@ struct Node3 {
 
 // FP64 step: the collision of one node, and its stores.
 template <bool WB, bool FLAT>
-__global__ void __launch_bounds__(kBlock3) d3_collide(const double* __restrict__ src,
-                                                      double* __restrict__ dst,
-                                                      const double* __restrict__ rho,
-                                                      const double* __restrict__ mu, const P3 p) {
+__global__ void __launch_bounds__(kBlock3) d3_collide(const double* src, double* dst,
+                                                      const double* rho, const double* mu,
+                                                      const P3 p) {
   int x, y, z;
   const bool on = node_of<FLAT>(p, x, y, z);
   chain_wait();
@@ -526,10 +522,8 @@ __global__ void __launch_bounds__(kBlock3) d3_collide(const double* __restrict__
 // (one CTA) are shared by several nodes of each thread.
 constexpr int kMomPlanes3 = 8;
 template <typename T, bool WB>
-__global__ void __launch_bounds__(kBlock3) d3_moments(const T* __restrict__ src,
-                                                      const T* __restrict__ rho,
-                                                      const T* __restrict__ mu, const P3 p,
-                                                      const Out3 out) {
+__global__ void __launch_bounds__(kBlock3) d3_moments(const T* src, const T* rho, const T* mu,
+                                                      const P3 p, const Out3 out) {
   const int x = blockIdx.x * kBlock3 + threadIdx.x, y = blockIdx.y;
   const int z0 = blockIdx.z * kMomPlanes3, z1 = min(z0 + kMomPlanes3, p.nz);
   StatsAcc<T> acc;
@@ -577,8 +571,7 @@ constexpr int kMinB3 = 4;          // resident CTAs (128 registers)
 
 template <bool WB>
 __global__ void __launch_bounds__(kNT3, kMinB3)
-    d3_step_f32(const float* __restrict__ src, float* __restrict__ dst,
-                const float* __restrict__ rho, const P3 p, int run) {
+    d3_step_f32(const float* src, float* dst, const float* rho, const P3 p, int run) {
   constexpr int TX = kTX3, TY = kTY3;
   constexpr int FW = TX + 4, FH = TY + 4, MW = TX + 2, MH = TY + 2;
   __shared__ float rho_s[4][FH][FW];           // [f & 3][2 + y][2 + x]

@@ -1056,6 +1056,10 @@ __device__ __forceinline__ void emit_node(const KParams& p, const MomentsOut& mo
 // and the step after runs unbalanced (256^2 FP64, 128 CTAs: 18.0 us per step
 // signalled at the end, 46 us from the start, 19.0 us without).  Kernels
 // launched without the attribute pass through both.
+// A waiting kernel is resident while the grid before it writes what it will
+// read, so its pointers are plain ones (no __restrict__, no __ldg): those would
+// let the compiler take the non-coherent load path, which is for data that
+// nothing writes while the kernel lives.
 __device__ __forceinline__ void chain_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -1075,10 +1079,9 @@ __device__ __forceinline__ void chain_signal() {
 // pitch >= nx + ghost_off + 8.
 // Offsets within a plane are 32-bit: pitch * ny < 2^31 (checked by the host).
 template <typename T, int SCH, int MODE, int TX, bool GHOST = false>
-__device__ __forceinline__ void strip_pass(const T* __restrict__ src, T* __restrict__ dst,
-                                           const KParams& p, const MomentsOut& mo, int x0,
-                                           int y0, int y1, double* stats_rec,
-                                           unsigned char* smem_raw) {
+__device__ __forceinline__ void strip_pass(const T* src, T* dst, const KParams& p,
+                                           const MomentsOut& mo, int x0, int y0, int y1,
+                                           double* stats_rec, unsigned char* smem_raw) {
   constexpr bool STATS = MODE != kModeStep;
   constexpr int R = Staging<T>::kRows;     // rows per iteration
   constexpr int PDG = Staging<T>::kAhead;  // row groups requested ahead of use
@@ -1519,8 +1522,7 @@ __device__ __forceinline__ void strip_pass(const T* __restrict__ src, T* __restr
 // from), write the per-CTA stats record.
 template <typename T, int SCH, int MODE, int TX>
 __global__ void __launch_bounds__(TX, Staging<T>::min_blocks(TX, SCH == kSchWB && MODE == kModeStep))
-    lbm_strip_kernel(const T* __restrict__ src, T* __restrict__ dst,
-                     const KParams p, const MomentsOut mo) {
+    lbm_strip_kernel(const T* src, T* dst, const KParams p, const MomentsOut mo) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   chain_wait();
   const int x0 = blockIdx.x * TX;

@@ -45,8 +45,7 @@ constexpr int min_ctas() {
 // frame, whose work would otherwise follow the owners' own.
 template <typename T, int SCH, int MODE, int TW, int TH, int PR, int NT>
 __global__ void __launch_bounds__(NT, min_ctas<T, PR>())
-    lbm_tile_kernel(const T* __restrict__ src, T* __restrict__ dst, const KParams p,
-                    const MomentsOut mo) {
+    lbm_tile_kernel(const T* src, T* dst, const KParams p, const MomentsOut mo) {
   static_assert(SCH == kSchStandard || SCH == kSchWB, "potential-form schemes");
   static_assert(sizeof(T) == 8 || PR == 2, "FP32 threads own a pair of rows");
   constexpr bool STATS = MODE != kModeStep;
@@ -267,8 +266,7 @@ __global__ void __launch_bounds__(NT, min_ctas<T, PR>())
 // every SM) 5.3 and 4.9, 100^2 (3 on some) 5.6 and 6.2.
 template <int SCH>
 __global__ void __launch_bounds__(128)
-    lbm_tile_split_kernel(const double* __restrict__ src, double* __restrict__ dst,
-                          const KParams p) {
+    lbm_tile_split_kernel(const double* src, double* dst, const KParams p) {
   constexpr int TW = 8, TH = 4, FW = TW + 4, FH = TH + 4;
   static_assert(TW * TH == 32 && FW * FH - 32 == 64 && (TW + 2) * (TH + 2) - 32 <= 32,
                 "a warp's nodes, two warps' frame and one warp's ring");
