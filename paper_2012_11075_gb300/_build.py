@@ -20,7 +20,7 @@ DEBUG_LIB_PATH = LIB_DIR / f"libwblbe_bounds_{platform.machine()}.so"
 SOURCES = [CSRC / "batch.cu", CSRC / "wblbe.cu", CSRC / "strip_variants.cu",
            CSRC / "wblbe_noalloc.cu", CSRC / "probe.cu", CSRC / "slabs.cu", CSRC / "d3q19.cu",
            CSRC / "tile.cu"]
-DEPENDS = SOURCES + [CSRC / "lbm_kernels.cuh", CSRC / "strip_launch.cuh",
+DEPENDS = SOURCES + [CSRC / "lbm_kernels.cuh", CSRC / "strip_launch.cuh", CSRC / "batch_cut.h",
                      ROOT / "include" / "wblbe.h"]
 
 NVCC_FLAGS = [

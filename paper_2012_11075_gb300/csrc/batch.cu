@@ -38,6 +38,7 @@
 #include <vector>
 
 #include "../../include/wblbe.h"
+#include "batch_cut.h"
 #include "lbm_kernels.cuh"
 
 using namespace wblbe;
@@ -510,26 +511,14 @@ wblbe_status ensure_case_tiles(wblbe_batch* b, wblbe_batch::Case& c, int rows) {
   return WBLBE_OK;
 }
 
-// Rows per tile for the running cases: the configured ones, halved (down to
-// 8) while that leaves fewer than two tiles per resident CTA and the tile
-// table holds the finer cut.  With less than that, CTAs idle while the
-// longest tile of each step marches its rows: a tile's row takes about 0.7 us
-// whatever runs beside it.  us per step of 64-step launches, 128-column
-// tiles, rows 128 / 64 / 32 / 16 / 8: 32 cases of 64-300 columns (50 to 979
-// tiles) 141 / 73 / 37 / 23 / 18; 128 cases of 64-512 (432 to 7480) 188 / 121
-// / 107 / 118 / 139; 400 (1292 to 22771) 303 / 297 / 316 / 352 / 417.
-// Results do not depend on the cut.
+// The cut of the running cases (see cut_rows).
 int effective_rows(const wblbe_batch* b) {
-  auto total = [&](int rows) {
+  return cut_rows(b->cfg.rows_per_tile, resident_ctas(b), b->max_tiles, [&](int rows) {
     long long n = 0;
     for (const auto& c : b->cases)
       if (c.used && c.running) n += tile_count(c, b->cfg.tile_x, rows);
     return n;
-  };
-  const long long want = 2LL * resident_ctas(b);
-  int rows = b->cfg.rows_per_tile;
-  while (rows >= 16 && total(rows) < want && total(rows / 2) <= b->max_tiles) rows /= 2;
-  return rows;
+  });
 }
 
 wblbe_status upload_case_entry(wblbe_batch* b, int ci) {
