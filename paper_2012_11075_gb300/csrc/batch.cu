@@ -513,12 +513,14 @@ wblbe_status ensure_case_tiles(wblbe_batch* b, wblbe_batch::Case& c, int rows) {
 
 // The cut of the running cases (see cut_rows).
 int effective_rows(const wblbe_batch* b) {
-  return cut_rows(b->cfg.rows_per_tile, resident_ctas(b), b->max_tiles, [&](int rows) {
+  auto total = [&](int rows) {
     long long n = 0;
     for (const auto& c : b->cases)
       if (c.used && c.running) n += tile_count(c, b->cfg.tile_x, rows);
     return n;
-  });
+  };
+  return cut_rows(b->cfg.rows_per_tile, resident_ctas(b), b->max_tiles, b->cfg.steps_per_launch,
+                  total);
 }
 
 wblbe_status upload_case_entry(wblbe_batch* b, int ci) {
@@ -890,7 +892,9 @@ wblbe_status wblbe_batch_set_config(wblbe_batch_handle b, const wblbe_batch_conf
                   config->tile_x != 256) ||
       config->rows_per_tile < 4 || config->steps_per_launch < 1)
     return bfail(b, WBLBE_EINVAL, "config: tile_x 32/64/128/256, rows_per_tile >= 4, steps >= 1");
-  const bool retile = config->tile_x != b->cfg.tile_x || config->rows_per_tile != b->cfg.rows_per_tile;
+  const bool retile = config->tile_x != b->cfg.tile_x ||
+                      config->rows_per_tile != b->cfg.rows_per_tile ||
+                      config->steps_per_launch != b->cfg.steps_per_launch;   // see cut_rows
   if (config->tile_x != b->cfg.tile_x) drop_batch_graph(b);
   b->cfg = *config;
   if (retile) b->tiles_dirty = true;

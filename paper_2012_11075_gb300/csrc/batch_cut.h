@@ -1,6 +1,8 @@
 // The rule that chooses a batch's cut (host arithmetic only).
 #pragma once
 
+#include <limits>
+
 namespace wblbe {
 
 // Rows per tile for the running cases: the configured ones, halved (down to
@@ -16,10 +18,15 @@ namespace wblbe {
 //   FP64 0.76 453 and 420, 0.99 2615 and 1837, 1.40 341 and 353, 1.50 1475 and
 //        1456, 1.55 420 and 445, 1.70 1845 and 1856.
 // Results do not depend on the cut.  total(rows): tiles of the running cases
-// when cut at `rows`.
+// when cut at `rows`.  A launch of `steps` steps numbers its work items, and
+// each resident CTA's last claim past them, in an int: a finer cut has to keep
+// to that as well.
 template <typename Total>
-int cut_rows(int rows, long long resident, long long max_tiles, Total total) {
-  while (rows >= 16 && 10 * total(rows) < 13 * resident && total(rows / 2) <= max_tiles) rows /= 2;
+int cut_rows(int rows, long long resident, long long max_tiles, long long steps, Total total) {
+  const long long most = std::numeric_limits<int>::max() - resident;
+  while (rows >= 16 && 10 * total(rows) < 13 * resident && total(rows / 2) <= max_tiles &&
+         total(rows / 2) <= most / steps)
+    rows /= 2;
   return rows;
 }
 
