@@ -20,6 +20,8 @@
 // bit.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "lbm_kernels.cuh"
 #include "strip_launch.cuh"
 
@@ -463,6 +465,42 @@ cudaError_t launch_tile(int sch, bool fp64, int mode, const void* src, void* dst
                         const KParams& kp, const MomentsOut& mo, cudaStream_t s, bool chained) {
   return sch == kSchWB ? launch_scheme_tile<kSchWB>(fp64, mode, src, dst, kp, mo, s, chained)
                        : launch_scheme_tile<kSchStandard>(fp64, mode, src, dst, kp, mo, s, chained);
+}
+
+// Lattices of few rows and many columns: their last row of tiles is mostly
+// padding, which the strip kernel does not have.  us per step there and here:
+// FP64 200000 x 2 348 and 121, 40000 x 4 75 and 58, 10000 x 2 25.3 and 17.2,
+// 10000 x 4 25.5 and 26.7, 40000 x 8 95 and 102; FP32 200000 x 2 25 and 12.6,
+// 40000 x 2 6.5 and 4.7, 25000 x 4 5.1 and 5.4, 80000 x 18 31.3 and 24.9, 80000 x
+// 12 15.0 and 17.9.  Neither the row count nor the padding alone draws that
+// line, so the two times are estimated (us; over 189 FP64 and 192 FP32 sizes of
+// 1 to 49 rows and 1500 to 500000 columns the choice is never more than 3 %
+// slower than the tiles, nor more than 17 % slower than the better kernel).
+// rows_per_cta: of the strip kernel's launch, 128 columns wide.
+bool flat_takes_strips(bool fp64, int nx, int ny, int rows_per_cta) {
+  const int last = fp64 ? 2 : 1;
+  if (ny >= 64 || shape_of(fp64, nx, ny) != last) return false;
+  const Shape& t = (fp64 ? kShapes64 : kShapes32)[last];
+  const int cols = (nx + t.tw - 1) / t.tw, whole = ny / t.th, rest = ny % t.th;
+  const int strips = (nx + 127) / 128, runs = (ny + rows_per_cta - 1) / rows_per_cta;
+  const int ctas = strips * runs;
+  auto waves = [](int n) { return (n + (int)kSMs - 1) / (int)kSMs; };
+  if (fp64) {
+    // bound by the FP64 pipes: a tile's time is its four-row groups', a strip
+    // CTA's its rows', shared evenly by the SMs; a lone CTA waits for its chain
+    const double tiles = 3.0 + cols / (double)kSMs * (whole * 7.8 + (rest ? 3.0 + 1.2 * ((rest + 3) / 4) : 0.0));
+    const int full = strips * (ny / rows_per_cta);          // CTAs with all their rows
+    const double strip = std::max({5.0 + waves(ctas) * (3.0 + 4.0 * ny / runs),
+                                   5.0 + waves(full) * (3.0 + 4.0 * rows_per_cta),
+                                   7.6 + 4.8 * rows_per_cta});
+    return strip < 0.98 * tiles;
+  }
+  // bound by the requests in flight: a base per tile and a share per row; a base
+  // per strip CTA and a share per pair of rows, after one CTA's own chain
+  const double tiles = 1.5 + cols * (whole * 0.0066 + (rest ? 0.0036 + 0.00019 * rest : 0.0));
+  const double strip = 2.0 + 0.7 * ((rows_per_cta + 1) / 2) +
+                       ctas * (0.0028 + 0.00135 * (runs == 1 ? ny + (ny & 1) : ny / (double)runs));
+  return strip < 0.98 * tiles;
 }
 
 unsigned int tile_bounds_errors(bool reset) { return read_bounds_errors(reset); }

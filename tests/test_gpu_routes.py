@@ -55,3 +55,34 @@ def test_batch_is_not_cut_finer_than_it_needs():
         t[rows] = _us(lambda: b.advance(3), 3 * 32)
         b.close()
     assert t[16] < 1.12 * t[15], t
+
+
+# few rows, many columns: the tile kernel's padding made the default step 1.3
+# to 3.6 times slower than the strip kernel's (which set_launch selects)
+@pytest.mark.parametrize("scheme", [wblbe.STANDARD, wblbe.WELL_BALANCED])
+@pytest.mark.parametrize("precision,nx,ny", [
+    (wblbe.FP64, 200000, 1), (wblbe.FP64, 200000, 4), (wblbe.FP64, 40000, 2),
+    (wblbe.FP64, 200000, 17), (wblbe.FP64, 10000, 1), (wblbe.FP32_SHIFTED, 200000, 2),
+    (wblbe.FP32_SHIFTED, 40000, 1), (wblbe.FP32_SHIFTED, 500000, 5),
+    # and a few that stay on the tiles
+    (wblbe.FP64, 10000, 5), (wblbe.FP64, 40000, 12), (wblbe.FP32_SHIFTED, 25000, 6)])
+def test_flat_lattices_take_the_faster_kernel(scheme, precision, nx, ny):
+    rng = np.random.default_rng(nx + ny)
+    rho = 0.6 + 0.3 * rng.uniform(-1, 1, (ny, nx))
+    out = []
+    for strip in (False, True):
+        s = wblbe.Solver(wblbe.Params(nx, ny, 0.9, 0.0128, 0.01, 1.0, 0.2, scheme=scheme,
+                                      precision=precision))
+        if strip:
+            s.set_launch(*s.get_launch())
+        s.init_rho(rho)
+        s.step(6)
+        code, done, st = s.run_until_equilibrium(0.0, 5, 3)
+        out.append((s.get_populations(), s.moments()[0], st["mu_min"], st["mu_max"], st["umax"],
+                    _us(lambda: s.step(32), 32)))
+        s.close()
+    (fa, ma, *sa, ta), (fb, mb, *sb, tb) = out
+    assert np.array_equal(fa, fb) and sa == sb
+    for k in ("rho", "ux", "uy", "mu"):
+        assert np.array_equal(ma[k], mb[k]), k
+    assert ta < 1.2 * tb, (ta, tb)
