@@ -146,8 +146,9 @@ int e6_partials(int nx, int ny);
 bool tile_path(int sch, bool fp64, int mode, int nx, int ny);
 int tile_records(bool fp64, int nx, int ny);
 // Whether a lattice that the tile kernel could take has so few rows that the
-// strip kernel, with this many rows per CTA, is faster.
-bool flat_takes_strips(bool fp64, int nx, int ny, int rows_per_cta);
+// strip kernel, with this many rows per CTA, is faster (stats: in the modes
+// that reduce statistics).
+bool flat_takes_strips(bool fp64, bool stats, int nx, int ny, int rows_per_cta);
 cudaError_t launch_tile(int sch, bool fp64, int mode, const void* src, void* dst,
                         const KParams& kp, const MomentsOut& mo, cudaStream_t s, bool chained);
 // Strip-kernel launches for scheme codes 0-3 without instantiating the

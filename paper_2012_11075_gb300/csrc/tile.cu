@@ -476,31 +476,37 @@ cudaError_t launch_tile(int sch, bool fp64, int mode, const void* src, void* dst
 // line, so the two times are estimated (us; over 189 FP64 and 192 FP32 sizes of
 // 1 to 49 rows and 1500 to 500000 columns the choice is never more than 3 %
 // slower than the tiles, nor more than 17 % slower than the better kernel).
+// stats: for the passes with statistics, which the strips do in a smaller part
+// of their step's time, and whose final pass reads one record per CTA (moments
+// FP64 20000 x 4 84 us on tiles, 72 on strips, FP32 40000 x 20 63 and 50).
 // rows_per_cta: of the strip kernel's launch, 128 columns wide.
-bool flat_takes_strips(bool fp64, int nx, int ny, int rows_per_cta) {
+bool flat_takes_strips(bool fp64, bool stats, int nx, int ny, int rows_per_cta) {
   const int last = fp64 ? 2 : 1;
   if (ny >= 64 || shape_of(fp64, nx, ny) != last) return false;
   const Shape& t = (fp64 ? kShapes64 : kShapes32)[last];
   const int cols = (nx + t.tw - 1) / t.tw, whole = ny / t.th, rest = ny % t.th;
   const int strips = (nx + 127) / 128, runs = (ny + rows_per_cta - 1) / rows_per_cta;
-  const int ctas = strips * runs;
+  const int ctas = strips * runs, records = cols * (whole + (rest ? 1 : 0));
   auto waves = [](int n) { return (n + (int)kSMs - 1) / (int)kSMs; };
   if (fp64) {
     // bound by the FP64 pipes: a tile's time is its four-row groups', a strip
     // CTA's its rows', shared evenly by the SMs; a lone CTA waits for its chain
-    const double tiles = 3.0 + cols / (double)kSMs * (whole * 7.8 + (rest ? 3.0 + 1.2 * ((rest + 3) / 4) : 0.0));
+    const double tiles =
+        3.0 + cols / (double)kSMs * (whole * 7.8 + (rest ? 3.0 + 1.2 * ((rest + 3) / 4) : 0.0));
     const int full = strips * (ny / rows_per_cta);          // CTAs with all their rows
     const double strip = std::max({5.0 + waves(ctas) * (3.0 + 4.0 * ny / runs),
                                    5.0 + waves(full) * (3.0 + 4.0 * rows_per_cta),
                                    7.6 + 4.8 * rows_per_cta});
-    return strip < 0.98 * tiles;
+    return stats ? 4.0 + 0.8 * strip < 0.97 * (tiles + 0.01 * (records - ctas))
+                 : strip < 0.98 * tiles;
   }
   // bound by the requests in flight: a base per tile and a share per row; a base
   // per strip CTA and a share per pair of rows, after one CTA's own chain
   const double tiles = 1.5 + cols * (whole * 0.0066 + (rest ? 0.0036 + 0.00019 * rest : 0.0));
   const double strip = 2.0 + 0.7 * ((rows_per_cta + 1) / 2) +
                        ctas * (0.0028 + 0.00135 * (runs == 1 ? ny + (ny & 1) : ny / (double)runs));
-  return strip < 0.98 * tiles;
+  return stats ? 2.0 + 0.5 * strip < 0.97 * (tiles + 0.004 * (records - ctas))
+               : strip < 0.98 * tiles;
 }
 
 unsigned int tile_bounds_errors(bool reset) { return read_bounds_errors(reset); }

@@ -109,7 +109,7 @@ struct wblbe_ctx {
   wblbe_launch launch;
   bool launch_set;               // the caller chose the strip kernel's shape
   wblbe_launch moments;          // the default shape, of the moments pass
-  bool flat;                     // few rows: strips rather than tiles
+  bool flat[2];                  // few rows: strips rather than tiles (steps, statistics)
   int64_t steps;
   int64_t launches;
   double mass0;
@@ -252,7 +252,7 @@ wblbe_launch default_launch(const wblbe_params& p) {
 // alone (its default launch shape included); steps unless the caller chose a launch shape, which is one of the
 // strip kernel.
 bool takes_tiles(const wblbe_ctx* h, int mode) {
-  return (mode == kModeMoments || !h->launch_set) && !h->flat &&
+  return (mode == kModeMoments || !h->launch_set) && !h->flat[mode != kModeStep] &&
          tile_path(h->p.scheme, h->p.precision == WBLBE_FP64, mode, h->p.nx, h->p.ny);
 }
 
@@ -488,8 +488,9 @@ wblbe_status wblbe_create(const wblbe_params* params, void* dev_workspace,
   h->cur = 0;
   h->launch = default_launch(*params);
   h->moments = h->launch;
-  h->flat = flat_takes_strips(params->precision == WBLBE_FP64, params->nx, params->ny,
-                              h->launch.rows_per_cta);
+  for (int stats = 0; stats < 2; ++stats)
+    h->flat[stats] = flat_takes_strips(params->precision == WBLBE_FP64, stats, params->nx,
+                                       params->ny, h->launch.rows_per_cta);
   *out = h;
   return WBLBE_OK;
 }
