@@ -517,15 +517,14 @@ __global__ void __launch_bounds__(kBlock3) d3_collide(const double* src, double*
   chain_signal();
 }
 
-// Fields and statistics of kMomPlanes3 planes per CTA: one record for all of
-// them, so that the reduction's shuffles and the final pass over the records
-// (one CTA) are shared by several nodes of each thread.
-constexpr int kMomPlanes3 = 8;
+// Fields and statistics of `planes` planes per CTA: one record for all of them,
+// so that the reduction's shuffles and the final pass over the records (one
+// CTA) are shared by several nodes of each thread.
 template <typename T, bool WB>
 __global__ void __launch_bounds__(kBlock3) d3_moments(const T* src, const T* rho, const T* mu,
-                                                      const P3 p, const Out3 out) {
+                                                      const P3 p, const Out3 out, int planes) {
   const int x = blockIdx.x * kBlock3 + threadIdx.x, y = blockIdx.y;
-  const int z0 = blockIdx.z * kMomPlanes3, z1 = min(z0 + kMomPlanes3, p.nz);
+  const int z0 = blockIdx.z * planes, z1 = min(z0 + planes, p.nz);
   StatsAcc<T> acc;
   chain_wait();
   for (int z = z0; z < z1 && x < p.nx; ++z) {
@@ -759,7 +758,8 @@ struct Layout3 {
   int pitch;
   long long plane;
   size_t off_a, off_b, off_rho, off_mu, off_stage, off_partials, off_stats, total;
-  long long records;
+  int planes;                     // planes per CTA of the moments pass
+  long long records;              // its CTAs
 };
 
 size_t elem3(const wblbe3_params* p) { return p->precision == WBLBE_FP64 ? 8 : 4; }
@@ -770,8 +770,14 @@ Layout3 layout3(const wblbe3_params* p) {
   L.plane = (long long)L.pitch * p->ny * p->nz;
   const size_t pops = align3((size_t)kQ3 * L.plane * elem3(p));
   const size_t field = align3((size_t)L.plane * elem3(p));
-  L.records = (long long)((p->nx + kBlock3 - 1) / kBlock3) * p->ny *
-              ((p->nz + kMomPlanes3 - 1) / kMomPlanes3);
+  // up to 8, while that leaves 400 CTAs (2.6 per SM): with fewer, a CTA's planes
+  // one after another are the pass.  us of the whole call with 1, 2, 4 and 8
+  // planes: FP64 8^3 42, 42, 50, 58; 32^3 55, 53, 53, 58; 40^3 78, 68, 59, 65; 64^3
+  // 131, 109, 105, 101; FP32 24^3 41, 40, 43, 53; 48^3 54, 45, 44, 54; 96^3 123, 97,
+  // 82, 79
+  const long long rows = (long long)((p->nx + kBlock3 - 1) / kBlock3) * p->ny;
+  for (L.planes = 8; L.planes > 1 && rows * ((p->nz + L.planes - 1) / L.planes) < 400;) L.planes /= 2;
+  L.records = rows * ((p->nz + L.planes - 1) / L.planes);
   size_t off = 0;
   L.off_a = off; off += pops;
   L.off_b = off; off += pops;
@@ -906,8 +912,8 @@ cudaError_t pass3_typed(wblbe3_ctx* h, bool moments, const Out3& out, const P3& 
              : launch3(d3_chem_pot<T, false>, gn, kBlock3, h->stream, rho, mu, q);
   if (e != cudaSuccess) return e;
   if (moments) {
-    const dim3 gm(g.x, g.y, (h->p.nz + kMomPlanes3 - 1) / kMomPlanes3);
-    return launch3(d3_moments<T, WB>, gm, kBlock3, h->stream, src, rho, mu, q, out);
+    const dim3 gm(g.x, g.y, (h->p.nz + h->L.planes - 1) / h->L.planes);
+    return launch3(d3_moments<T, WB>, gm, kBlock3, h->stream, src, rho, mu, q, out, h->L.planes);
   }
   if constexpr (sizeof(T) == 8)
     return flat ? launch3(d3_collide<WB, true>, gn, kBlock3, h->stream, src,
