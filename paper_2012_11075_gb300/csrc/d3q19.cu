@@ -813,11 +813,32 @@ bool params3_valid(const wblbe3_params* p, char* why, size_t n) {
   return true;
 }
 
+// Planes per CTA of the FP32 step kernel: the run whose waves of resident CTAs
+// (on nsm SMs) take the fewest plane iterations in all (a run of n planes takes
+// n + 4, of which the first four store nothing).
+int step_run(const wblbe3_params* p, int nsm) {
+  const long long tiles = (long long)((p->nx + kTX3 - 1) / kTX3) * ((p->ny + kTY3 - 1) / kTY3);
+  const long long resident = (long long)nsm * kMinB3;
+  int best = p->nz;
+  long long cost = -1;
+  for (int segs = 1; segs <= p->nz && segs <= 65535; ++segs) {
+    const int run = (p->nz + segs - 1) / segs;
+    const long long n = tiles * ((p->nz + run - 1) / run);
+    const long long c = (n + resident - 1) / resident * (run + 4);
+    if (cost < 0 || c < cost) {
+      cost = c;
+      best = run;
+    }
+  }
+  return best;
+}
+
 }  // namespace
 
 struct wblbe3_ctx {
   wblbe3_params p;
   Layout3 L;
+  int run;                        // planes per CTA of the FP32 step (step_run)
   int device;
   cudaStream_t stream;
   void* buf[2];                   // population buffers (float64 or float32)
@@ -923,28 +944,8 @@ cudaError_t pass3_typed(wblbe3_ctx* h, bool moments, const Out3& out, const P3& 
   return cudaErrorInvalidValue;              // FP32 steps: fp32_step
 }
 
-// Planes per CTA of the FP32 step kernel: the run whose waves of resident CTAs
-// take the fewest plane iterations in all (a run of n planes takes n + 4, of
-// which the first four store nothing).
-int step_run(const wblbe3_ctx* h) {
-  const long long tiles = (long long)((h->p.nx + kTX3 - 1) / kTX3) * ((h->p.ny + kTY3 - 1) / kTY3);
-  const long long resident = 152LL * kMinB3;
-  int best = h->p.nz;
-  long long cost = -1;
-  for (int segs = 1; segs <= h->p.nz && segs <= 65535; ++segs) {
-    const int run = (h->p.nz + segs - 1) / segs;
-    const long long n = tiles * ((h->p.nz + run - 1) / run);
-    const long long c = (n + resident - 1) / resident * (run + 4);
-    if (cost < 0 || c < cost) {
-      cost = c;
-      best = run;
-    }
-  }
-  return best;
-}
-
 cudaError_t fp32_step(wblbe3_ctx* h, const P3& q) {
-  const int run = step_run(h);
+  const int run = h->run;
   const dim3 grid((h->p.nx + kTX3 - 1) / kTX3, (h->p.ny + kTY3 - 1) / kTY3,
                   (h->p.nz + run - 1) / run);
   const float* src = static_cast<const float*>(h->buf[h->cur]);
@@ -1027,9 +1028,16 @@ wblbe_status wblbe3_create(const wblbe3_params* params, void* dev_workspace,
     delete h;
     return f3(nullptr, WBLBE_ECUDA, "no CUDA device");
   }
+  int nsm = 0;
+  if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess ||
+      nsm < 1) {
+    delete h;
+    return f3(nullptr, WBLBE_ECUDA, "cudaDeviceGetAttribute failed");
+  }
   unsigned char* ws = static_cast<unsigned char*>(dev_workspace);
   h->p = *params;
   h->L = L;
+  h->run = step_run(params, nsm);
   h->stream = static_cast<cudaStream_t>(cuda_stream);
   h->buf[0] = ws + L.off_a;
   h->buf[1] = ws + L.off_b;

@@ -130,3 +130,28 @@ def test_d3q19_moments_whatever_the_planes_per_cta(shape, precision):
     assert st["kinetic"] == pytest.approx(0.5 * (m["rho"] * u2).sum(), rel=tol)
     assert st["umax"] == pytest.approx(np.sqrt(u2.max()), rel=1e-15)
     assert st["mu_min"] == m["mu"].min() and st["mu_max"] == m["mu"].max()
+
+
+def _d3_issue_us(nz):
+    """Host time of issuing one FP32 step of a 1 x 1 x nz lattice."""
+    import time
+
+    import torch
+    s = wblbe.Solver3(wblbe.Params3(1, 1, nz, 0.95, 0.01, 0.01, 1.0, 0.2,
+                                    precision=wblbe.FP32_SHIFTED))
+    s.init_rho(np.full((nz, 1, 1), 0.6))
+    best = float("inf")
+    for _ in range(7):
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        s.step(20)                       # 40 launches: well within the launch queue
+        best = min(best, (time.perf_counter() - t) / 20 * 1e6)
+    torch.cuda.synchronize()
+    s.close()
+    return best
+
+
+def test_host_work_of_a_d3q19_step_does_not_grow_with_the_lattice():
+    """Choosing the run of planes again in every step cost some hundred us of
+    host time for 65535 planes; two launches take about ten."""
+    assert _d3_issue_us(65535) < _d3_issue_us(64) + 30.0
