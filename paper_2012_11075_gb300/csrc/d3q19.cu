@@ -133,6 +133,13 @@ struct Nbr3 {
   }
 };
 
+// Element `off` of a population plane or a field (checked in the bounds-checked
+// build, as are the stores below).
+template <typename T>
+__device__ __forceinline__ T elem3_at(const T* plane, unsigned off, const P3& p) {
+  return WB_IN(off, p.plane) ? plane[off] : T(0);
+}
+
 // The node of a thread of the density, chemical-potential and FP64 collision
 // kernels.  Rows that are not whole blocks are numbered along x, then y, then z
 // without a break at their ends: an FP64 warp instruction costs the same with
@@ -168,7 +175,8 @@ __global__ void __launch_bounds__(kBlock3) d3_density(const T* src, T* rho, cons
   const Nbr3 nb(p, x, y, z);
   T g[kQ3];
 #pragma unroll
-  for (int i = 0; i < kQ3; ++i) g[i] = (src + i * p.plane)[nb.at(-cx3(i), -cy3(i), -cz3(i))];
+  for (int i = 0; i < kQ3; ++i)
+    g[i] = elem3_at(src + i * p.plane, nb.at(-cx3(i), -cy3(i), -cz3(i)), p);
   T s;
   if (sizeof(T) == 8) {
     s = g[0];                                     // f_0 (c_0 = 0)
@@ -177,7 +185,8 @@ __global__ void __launch_bounds__(kBlock3) d3_density(const T* src, T* rho, cons
   } else {
     s = g[0] + moving_sum3(g);
   }
-  rho[nb.at(0, 0, 0)] = s;
+  const unsigned k = nb.at(0, 0, 0);
+  if (WB_IN(k, p.plane)) rho[k] = s;
   chain_signal();
 }
 
@@ -213,14 +222,15 @@ __global__ void __launch_bounds__(kBlock3) d3_chem_pot(const T* rho, T* mu, cons
   const Nbr3 nb(p, x, y, z);
   // sums of the axis and edge neighbours, then the centre's share taken off
   // once per sum (rather than from every neighbour): 6 (ax/18 + ed/36)
-  auto nbr = [&](int i) { return rho[nb.at(cx3(i), cy3(i), cz3(i))]; };
+  auto nbr = [&](int i) { return elem3_at(rho, nb.at(cx3(i), cy3(i), cz3(i)), p); };
   T ax = nbr(1), ed = nbr(7);
 #pragma unroll
   for (int i = 2; i < kQ3; ++i) {
     if (i == 7) continue;
     if (i < 7) ax += nbr(i); else ed += nbr(i);
   }
-  mu[nb.at(0, 0, 0)] = mu3(ax, ed, rho[nb.at(0, 0, 0)], consts3(p, T(0)));
+  const unsigned k = nb.at(0, 0, 0);
+  if (WB_IN(k, p.plane)) mu[k] = mu3(ax, ed, rho[k], consts3(p, T(0)));
   chain_signal();
 }
 
@@ -240,8 +250,10 @@ __device__ __forceinline__ void grad3_sums(const V& v, T& gx, T& gy, T& gz) {
 // (edge differences); the factor 1/12 is folded into the constants that
 // use the gradients.
 template <typename T>
-__device__ __forceinline__ void grad3x12(const T* phi, const Nbr3& nb, T& gx, T& gy, T& gz) {
-  grad3_sums<T>([&](int dx, int dy, int dz) { return phi[nb.at(dx, dy, dz)]; }, gx, gy, gz);
+__device__ __forceinline__ void grad3x12(const T* phi, const Nbr3& nb, const P3& p, T& gx, T& gy,
+                                         T& gz) {
+  grad3_sums<T>([&](int dx, int dy, int dz) { return elem3_at(phi, nb.at(dx, dy, dz), p); }, gx, gy,
+                gz);
 }
 
 // One component of u = (j + F/2) / rho (Eq. rhoU) from 12 grad mu and 12 grad
@@ -485,11 +497,12 @@ struct Node3 {
   __device__ __forceinline__ Node3(const T* src, const T* rho, const T* mu, const P3& p,
                                    const Nbr3& nb) {
 #pragma unroll
-    for (int i = 0; i < kQ3; ++i) g[i] = (src + i * p.plane)[nb.at(-cx3(i), -cy3(i), -cz3(i))];
-    rs = rho[nb.at(0, 0, 0)];                  // rho - rho_ref (rho in FP64)
+    for (int i = 0; i < kQ3; ++i)
+      g[i] = elem3_at(src + i * p.plane, nb.at(-cx3(i), -cy3(i), -cz3(i)), p);
+    rs = elem3_at(rho, nb.at(0, 0, 0), p);     // rho - rho_ref (rho in FP64)
     r = sizeof(T) == 4 ? rs + consts3(p, T(0)).rho_ref : rs;
-    grad3x12<T>(mu, nb, gmx, gmy, gmz);
-    grad3x12<T>(rho, nb, grx, gry, grz);
+    grad3x12<T>(mu, nb, p, gmx, gmy, gmz);
+    grad3x12<T>(rho, nb, p, grx, gry, grz);
     T jx, jy, jz;
     momentum3(g, jx, jy, jz);
     const T inv = recip(r);
@@ -513,7 +526,8 @@ __global__ void __launch_bounds__(kBlock3) d3_collide(const double* src, double*
   update3_f64<WB>(n.g, n.r, n.gmx, n.gmy, n.gmz, n.grx, n.gry, n.grz, n.ux, n.uy, n.uz, p);
   const unsigned k = nb.at(0, 0, 0);
 #pragma unroll
-  for (int i = 0; i < kQ3; ++i) (dst + i * p.plane)[k] = n.g[i];
+  for (int i = 0; i < kQ3; ++i)
+    if (WB_IN(k, p.plane)) (dst + i * p.plane)[k] = n.g[i];
   chain_signal();
 }
 
@@ -532,13 +546,15 @@ __global__ void __launch_bounds__(kBlock3) d3_moments(const T* src, const T* rho
     const Node3<T, WB> n(src, rho, mu, p, nb);
     const double rd = sizeof(T) == 4 ? widen(n.rs) + p.rho_ref : (double)n.r;
     const double ux = widen(n.ux), uy = widen(n.uy), uz = widen(n.uz);
-    const T muc = mu[nb.at(0, 0, 0)];
+    const T muc = elem3_at(mu, nb.at(0, 0, 0), p);
     const size_t k = ((size_t)z * p.ny + y) * p.nx + x;
-    if (out.rho) out.rho[k] = rd;
-    if (out.ux) out.ux[k] = ux;
-    if (out.uy) out.uy[k] = uy;
-    if (out.uz) out.uz[k] = uz;
-    if (out.mu) out.mu[k] = widen(muc);
+    if (WB_IN(k, p.nodes)) {
+      if (out.rho) out.rho[k] = rd;
+      if (out.ux) out.ux[k] = ux;
+      if (out.uy) out.uy[k] = uy;
+      if (out.uz) out.uz[k] = uz;
+      if (out.mu) out.mu[k] = widen(muc);
+    }
     acc.add(rd, muc, __fma_rn(uz, uz, __fma_rn(ux, ux, __dmul_rn(uy, uy))));
   }
   write_stats_record<kBlock3>(
@@ -628,7 +644,7 @@ __global__ void __launch_bounds__(kNT3, kMinB3)
     for (int i = 0; i < kQ3; ++i) {
       const unsigned xz = (cz3(i) == 1 ? zb : (cz3(i) == 0 ? zc : za)) + c.x[1 - cx3(i)];
       const float* pl = src + i * p.plane;
-      g[i] = make_float2(pl[xz + c.y[1 - cy3(i)]], pl[xz + c.y[2 - cy3(i)]]);
+      g[i] = make_float2(elem3_at(pl, xz + c.y[1 - cy3(i)], p), elem3_at(pl, xz + c.y[2 - cy3(i)], p));
     }
   };
   const unsigned layer = (unsigned)p.pitch * (unsigned)p.ny;
@@ -644,7 +660,7 @@ __global__ void __launch_bounds__(kNT3, kMinB3)
   const float2 zero = make_float2(0.f, 0.f);
   float2 prs = zero, pgx = zero, pgy = zero, pgz = zero;   // rho - rho_ref, 12 grad rho of f - 2
   auto ld2 = [&](const Col& c, unsigned z) {
-    return make_float2(rho[z + c.y[1] + c.x[1]], rho[z + c.y[2] + c.x[1]]);
+    return make_float2(elem3_at(rho, z + c.y[1] + c.x[1], p), elem3_at(rho, z + c.y[2] + c.x[1], p));
   };
   float2 nr = ld2(own, zc), nh = has_frame ? ld2(frame, zc) : zero;
   for (; f < z1 + 2; ++f) {
@@ -652,7 +668,7 @@ __global__ void __launch_bounds__(kNT3, kMinB3)
     const bool upd = mine_a && c >= z0;
     rho_s[f & 3][2 + ty][2 + tx] = nr.x;
     rho_s[f & 3][3 + ty][2 + tx] = nr.y;
-    if (has_frame) {
+    if (has_frame && WB_IN(hy, FH - 1) && WB_IN(hx, FW)) {
       rho_s[f & 3][hy][hx] = nh.x;
       rho_s[f & 3][hy + 1][hx] = nh.y;
     }
@@ -689,8 +705,8 @@ __global__ void __launch_bounds__(kNT3, kMinB3)
       grad3_planes(rb, rc, ra, x, y, gx, gy, gz);
       if (has_ring) {
         const float2 h = mu_at(rax + 1, ray + 1, rbx + 1, rby + 1);
-        mu_s[(f + 3) & 3][ray][rax] = h.x;
-        mu_s[(f + 3) & 3][rby][rbx] = h.y;
+        if (WB_IN(ray, MH) && WB_IN(rax, MW)) mu_s[(f + 3) & 3][ray][rax] = h.x;
+        if (WB_IN(rby, MH) && WB_IN(rbx, MW)) mu_s[(f + 3) & 3][rby][rbx] = h.y;
       }
     }
     __syncthreads();
@@ -700,12 +716,13 @@ __global__ void __launch_bounds__(kNT3, kMinB3)
                    mz);
       const uint32_t key = (uint32_t)(((long long)c * p.ny + y0 + ty) * p.nx + x0 + tx);
       update3_x2<WB>(g, prs, mx, my, mz, pgx, pgy, pgz, q, key, key + (uint32_t)p.nx, ht);
-      float* da = dst + (zm2 + own.x[1] + own.y[1]);
-      float* db = dst + (zm2 + own.x[1] + own.y[2]);
+      const unsigned ka = zm2 + own.x[1] + own.y[1], kb = zm2 + own.x[1] + own.y[2];
+      float *da = dst + ka, *db = dst + kb;
+      const bool in_a = WB_IN(ka, p.plane), in_b = mine_b && WB_IN(kb, p.plane);
 #pragma unroll
       for (int i = 0; i < kQ3; ++i) {
-        da[i * p.plane] = g[i].x;
-        if (mine_b) db[i * p.plane] = g[i].y;
+        if (in_a) da[i * p.plane] = g[i].x;
+        if (in_b) db[i * p.plane] = g[i].y;
       }
     }
     prs = rs;
@@ -732,9 +749,11 @@ __global__ void d3_init(const double* __restrict__ rho_in, T* __restrict__ dst, 
   for (int i = 0; i < kQ3; ++i) {
     const int xx = wrap3(x + cx3(i), p.nx), yy = wrap3(y + cy3(i), p.ny),
               zz = wrap3(z + cz3(i), p.nz);
-    const double r = rho_in[(size_t)(zz * p.ny + yy) * p.nx + xx] - p.rho_ref;
+    const size_t from = (size_t)(zz * p.ny + yy) * p.nx + xx;
+    const double r = (WB_IN(from, p.nodes) ? rho_in[from] : 0.0) - p.rho_ref;
     // WB: f_0^eq - s_0 = rho - rho_ref, f_i^eq - s_i = 0; standard: w_i (rho - rho_ref)
-    dst[i * p.plane + at3(p, x, y, z)] = (T)(wb ? (i == 0 ? r : 0.0) : w3(i) * r);
+    const long long k = at3(p, x, y, z);
+    if (WB_IN(k, p.plane)) dst[i * p.plane + k] = (T)(wb ? (i == 0 ? r : 0.0) : w3(i) * r);
   }
 }
 
@@ -744,10 +763,11 @@ __global__ void d3_get(const T* __restrict__ src, double* __restrict__ f, const 
                        double shift) {
   const int x = blockIdx.x * kBlock3 + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
   if (x >= p.nx) return;
-  const double v = (double)src[dir * p.plane + at3(p, wrap3(x - cx3(dir), p.nx),
-                                                   wrap3(y - cy3(dir), p.ny),
-                                                   wrap3(z - cz3(dir), p.nz))];
-  f[(size_t)(z * p.ny + y) * p.nx + x] = v + shift;
+  const long long k = at3(p, wrap3(x - cx3(dir), p.nx), wrap3(y - cy3(dir), p.ny),
+                          wrap3(z - cz3(dir), p.nz));
+  const double v = WB_IN(k, p.plane) ? (double)src[dir * p.plane + k] : 0.0;
+  const size_t to = (size_t)(z * p.ny + y) * p.nx + x;
+  if (WB_IN(to, p.nodes)) f[to] = v + shift;
 }
 
 thread_local char g_d3_error[256] = "";
@@ -1152,3 +1172,8 @@ wblbe_status wblbe3_destroy(wblbe3_handle h) {
 const char* wblbe3_last_error(wblbe3_handle h) { return h ? h->err : g_d3_error; }
 
 }  // extern "C"
+
+namespace wblbe {
+// bounds-check count of this translation unit's kernels (see lbm_kernels.cuh)
+unsigned int d3_bounds_errors(bool reset) { return read_bounds_errors(reset); }
+}  // namespace wblbe

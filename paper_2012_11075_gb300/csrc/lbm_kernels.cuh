@@ -128,8 +128,8 @@ constexpr int kStatRec = 6;       // mass, kinetic, umax^2, mu_min, mu_max, nonf
 enum SchemeId : int { kSchStandard = 0, kSchWB = 1, kSchPressure = 2, kSchTextbook = 3 };
 
 // Bounds-checked build (-DWBLBE_DEBUG_BOUNDS): every global access of the
-// strip kernels and the shared-memory slots computed at run time are checked
-// before use; a bad access is skipped and counted in g_bounds_errors (no
+// strip, tile and D3Q19 kernels and the shared-memory slots computed at run
+// time are checked before use; a bad access is skipped and counted in g_bounds_errors (no
 // trap), which the host reads with wblbe_debug_bounds_errors.  Without the
 // flag the checks compile to nothing.
 #ifdef WBLBE_DEBUG_BOUNDS

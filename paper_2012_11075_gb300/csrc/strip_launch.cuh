@@ -161,5 +161,6 @@ cudaError_t allow_smem_strip_all();
 unsigned int variants_bounds_errors(bool reset);
 unsigned int batch_bounds_errors(bool reset);
 unsigned int tile_bounds_errors(bool reset);
+unsigned int d3_bounds_errors(bool reset);
 
 }  // namespace wblbe

@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(NT, min_ctas<T, PR>())
     pull(f, xc == 0 ? nx - 1 : xc - 1, xc, xc == nx - 1 ? 0 : xc + 1,
          (unsigned)((yc == 0 ? ny - 1 : yc - 1) * p.pitch), (unsigned)(yc * p.pitch),
          (unsigned)((yc == ny - 1 ? 0 : yc + 1) * p.pitch));
-    rho_s[fy][fx] = rho_of(f);
+    if (WB_IN(fy, FH) && WB_IN(fx, FW)) rho_s[fy][fx] = rho_of(f);
   }
   T rs[PR];
   const int fx = 2 + tx, fy = 2 + r0;
@@ -168,8 +168,8 @@ __global__ void __launch_bounds__(NT, min_ctas<T, PR>())
       const int ax = h < TW + 2 ? 1 + h : 1, ay = h < TW + 2 ? 1 : h - TW;
       const int bx = h < TW + 2 ? 1 + h : TW + 2, by = h < TW + 2 ? TH + 2 : h - TW;
       const float2 m = mu2(ax, ay, bx, by);
-      mu_s[ay][ax] = m.x;
-      mu_s[by][bx] = m.y;
+      if (WB_IN(ay, FH) && WB_IN(ax, FW)) mu_s[ay][ax] = m.x;
+      if (WB_IN(by, FH) && WB_IN(bx, FW)) mu_s[by][bx] = m.y;
     }
   } else {
     if (owner) {
@@ -201,7 +201,8 @@ __global__ void __launch_bounds__(NT, min_ctas<T, PR>())
         hy = 2 + (q >> 1);
       }
       const T *rn = rho_s[hy + 1], *rc = rho_s[hy], *rb = rho_s[hy - 1];
-      mu_s[hy][hx] = chem_pot(rc[hx], rc[hx + 1], rc[hx - 1], rn[hx], rb[hx], rn[hx + 1],
+      if (WB_IN(hy, FH) && WB_IN(hx, FW))
+        mu_s[hy][hx] = chem_pot(rc[hx], rc[hx + 1], rc[hx - 1], rn[hx], rb[hx], rn[hx + 1],
                                  rn[hx - 1], rb[hx + 1], rb[hx - 1], two_beta, dl, dg, kappa6);
     }
   }

@@ -896,8 +896,9 @@ extern "C" unsigned int wblbe_debug_bounds_errors(int32_t reset) {
   const unsigned int b = batch_bounds_errors(reset != 0);
   const unsigned int c = variants_bounds_errors(reset != 0);
   const unsigned int d = tile_bounds_errors(reset != 0);
+  const unsigned int e = d3_bounds_errors(reset != 0);
   unsigned int sum = 0;
-  for (unsigned int v : {a, b, c, d}) {
+  for (unsigned int v : {a, b, c, d, e}) {
     if (v == 0xFFFFFFFFu || v == 0xFFFFFFFEu) return v;
     sum += v;
   }
