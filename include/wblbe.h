@@ -125,11 +125,15 @@ typedef struct {
   int32_t nonfinite;
 } wblbe_stats;
 
-/* Launch shape of the fused step kernel: tile_x lattice columns per CTA
+/* Launch shape of the fused strip kernel: tile_x lattice columns per CTA
  * (32, 64, 128 or 256) and rows_per_cta rows marched by each CTA (>= 1).
- * Results do not depend on it.  Lattices of up to about two million nodes
- * (standard and well-balanced schemes) run in a two-dimensional tile kernel
- * of their own until wblbe_set_launch asks for a shape. */
+ * Results do not depend on it.  Smaller lattices of the standard and
+ * well-balanced schemes do not run the strip kernel but one with
+ * two-dimensional tiles, whose shapes are its own: steps up to 3.61 (FP64)
+ * and 3.0 (FP32) million nodes until wblbe_set_launch asks for a shape,
+ * passes that reduce statistics up to 1.2 and 0.8 million (steps of
+ * wblbe_run_until_equilibrium likewise until then, moments always).  Lattices
+ * of fewer than 64 rows and very many columns stay on the strips. */
 typedef struct {
   int32_t tile_x;
   int32_t rows_per_cta;
@@ -155,8 +159,12 @@ wblbe_status wblbe_create(const wblbe_params* params, void* dev_workspace,
  * precisions), returns EINVAL: the stored state depends on them. */
 wblbe_status wblbe_set_params(wblbe_handle h, const wblbe_params* params);
 
-/* Choose the launch shape (see wblbe_launch).  EINVAL on unsupported
- * values.  The default is picked from the lattice size at creation. */
+/* Choose the strip kernel and its launch shape (see wblbe_launch); it stays
+ * chosen for the handle's life.  EINVAL on unsupported values.
+ * wblbe_get_launch gives the shape that the strip kernel has or would have
+ * (the default, picked from the lattice size at creation, before any
+ * wblbe_set_launch): handing that back selects the strip kernel, so a lattice
+ * that runs in the tile kernel should be left alone to keep it. */
 wblbe_status wblbe_set_launch(wblbe_handle h, const wblbe_launch* launch);
 wblbe_status wblbe_get_launch(wblbe_handle h, wblbe_launch* launch);
 

@@ -11,7 +11,8 @@
 //      rho and grad rho of the own nodes              (registers)
 //   3. grad mu, the collision and the stores,
 // at the price of evaluating the frame's densities and chemical potentials
-// again in every tile (0.56 to 1.5 times the tile's densities).  The chain of
+// again in every tile (0.41 times the tile's densities at 32 x 16, 0.56 at 16 x
+// 16, 0.88 at 16 x 8, 2.0 at 8 x 4).  The chain of
 // phases, not the traffic, bounds it up to about 256^2.  us per step with the
 // strip kernel and here: FP64 4 x 256 48.9 and 5.1, 100^2 49.2 and 5.7, 256^2
 // 51.2 and 17.4; FP32 100^2 8.1 and 2.0, 256^2 7.5 and 2.8, 512^2 8.7 and 5.4,
@@ -390,6 +391,8 @@ cudaError_t launch_shape(const void* src, void* dst, const KParams& kp, const Mo
 //                         256^2, 512 tiles: both 2.8)
 //         32 x 16, 2, 256 the rest (512^2: 5.4, 16 x 8 6.3; 1024^2 14.3 and
 //                         20.7, 64 x 16 15.7, 32 x 32 15.8)
+// (The SM count is a constant here because it decides the number of records, and
+// with it the workspace size that a caller asks for without a device.)
 struct Shape { int tw, th; long long max_tiles; };
 constexpr long long kSMs = 152, kAny = 1LL << 40;
 constexpr Shape kShapes64[] = {{8, 4, 380}, {16, 8, kSMs}, {16, 16, kAny}};
