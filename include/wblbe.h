@@ -128,12 +128,12 @@ typedef struct {
 /* Launch shape of the fused strip kernel: tile_x lattice columns per CTA
  * (32, 64, 128 or 256) and rows_per_cta rows marched by each CTA (>= 1).
  * Results do not depend on it.  Smaller lattices of the standard and
- * well-balanced schemes do not run the strip kernel but one with
- * two-dimensional tiles, whose shapes are its own: steps up to 3.61 (FP64)
- * and 3.0 (FP32) million nodes until wblbe_set_launch asks for a shape,
- * passes that reduce statistics up to 1.2 and 0.8 million (steps of
- * wblbe_run_until_equilibrium likewise until then, moments always).  Lattices
- * of fewer than 64 rows and very many columns stay on the strips. */
+ * well-balanced schemes run a kernel with two-dimensional tiles of its own
+ * shapes instead: steps up to 3.61 (FP64) and 3.0 (FP32) million nodes, steps
+ * that reduce statistics (wblbe_run_until_equilibrium) up to 1.2 and 0.8
+ * million, both until wblbe_set_launch asks for a shape, and moments up to 1.2
+ * and 0.8 million always.  Lattices of fewer than 64 rows and very many
+ * columns stay on the strips. */
 typedef struct {
   int32_t tile_x;
   int32_t rows_per_cta;
@@ -159,12 +159,12 @@ wblbe_status wblbe_create(const wblbe_params* params, void* dev_workspace,
  * precisions), returns EINVAL: the stored state depends on them. */
 wblbe_status wblbe_set_params(wblbe_handle h, const wblbe_params* params);
 
-/* Choose the strip kernel and its launch shape (see wblbe_launch); it stays
- * chosen for the handle's life.  EINVAL on unsupported values.
- * wblbe_get_launch gives the shape that the strip kernel has or would have
- * (the default, picked from the lattice size at creation, before any
- * wblbe_set_launch): handing that back selects the strip kernel, so a lattice
- * that runs in the tile kernel should be left alone to keep it. */
+/* Choose the strip kernel and its launch shape (see wblbe_launch) for the rest
+ * of the handle's life.  EINVAL on unsupported values.  wblbe_get_launch gives
+ * the shape that the strip kernel has or would have (before any
+ * wblbe_set_launch the default, picked from the lattice size at creation).
+ * Handing that to wblbe_set_launch selects the strip kernel: a lattice that
+ * runs in the tile kernel is best left alone. */
 wblbe_status wblbe_set_launch(wblbe_handle h, const wblbe_launch* launch);
 wblbe_status wblbe_get_launch(wblbe_handle h, wblbe_launch* launch);
 
@@ -354,8 +354,9 @@ wblbe_status wblbe_batch_get_populations(wblbe_batch_handle b, int64_t case_id,
 /* Free a case's slot, arena range and tiles. */
 wblbe_status wblbe_batch_retire(wblbe_batch_handle b, int64_t case_id);
 
-/* Cases resident and running, tiles of the running cases, free arena bytes
- * (any pointer may be NULL). */
+/* Cases resident and running, tiles of the running cases at the configured
+ * rows_per_tile (what admission holds against max_tiles; a launch may cut them
+ * finer, see wblbe_batch_config), free arena bytes (any pointer may be NULL). */
 wblbe_status wblbe_batch_counts(wblbe_batch_handle b, int32_t* resident,
                                 int32_t* running, int32_t* tiles,
                                 size_t* arena_free);
